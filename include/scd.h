@@ -125,15 +125,17 @@ typedef struct {
   int32_t tlo, thi;
 } scd_pair;
 
-/* Tunables of the tree and traversal (picked by the autotuner). */
+/* Tunables of the tree and traversal (picked by the autotuner).  The tree
+ * has eight children a node and one box per leaf and needs no stack; the
+ * fields marked "no effect" are checked and kept, for programs that set them,
+ * and change neither the result nor the time. */
 typedef struct {
-  int leaf_size;      /* boxes per leaf: 1, 2, 4 or 8                      */
-  int stack_depth;    /* traversal stack entries: 32, 64 or 128            */
-  int block_threads;  /* traversal block size (leaves of several boxes):
-                         32..256, a multiple of 32                         */
-  int morton_bits;    /* bits per axis of the 4D Morton key: 8, 10, 12, 16
-                         (default 12)                                      */
-  float time_scale;   /* weight of time against space in the Morton key,
+  int leaf_size;      /* 1, 2, 4 or 8 (no effect)                          */
+  int stack_depth;    /* 32, 64 or 128 (no effect)                         */
+  int block_threads;  /* 32..256, a multiple of 32 (no effect)             */
+  int morton_bits;    /* bits per axis of the boxes' 4D key along the
+                         Hilbert curve: 8, 10, 12, 16 (default 12)         */
+  float time_scale;   /* weight of time against space in the key,
                          (0, 16]: below 1 the horizon takes that share of
                          the time axis's cells; above 1 the scene cube takes
                          1/time_scale of the space axes' cells (default 8).
@@ -143,22 +145,18 @@ typedef struct {
   int use_graph;      /* 1: replay find_pairs as one captured CUDA graph    */
   int space_warp;     /* 1: log-compress |x| before quantising (finer keys
                          near Earth, where most boxes are); 0: linear      */
-  int nodes_per_step; /* one box per leaf, node width 2: tree nodes each
-                         lane visits per traversal step (two independent
-                         loads in flight), 1 or 2                          */
-  int node_width;     /* one box per leaf: 2 (binary nodes, 36 bytes) or 4
-                         (the grandchildren of a binary node in one 128-byte
-                         line: one traversal step descends two levels)     */
+  int nodes_per_step; /* 1 or 2 (no effect)                                */
+  int node_width;     /* 2 or 4 (no effect)                                */
   float split_km;     /* 0: off.  Otherwise boxes whose largest spatial side
                          exceeds |split_km| km are sorted apart from the
-                         others (one key bit above the Morton key, which
-                         with 12-bit axes gives up its finest time bit), so
+                         others (one key bit above the curve's, which
+                         with 12-bit axes gives up its lowest bit), so
                          each group gets its own subtree and the large boxes
                          do not widen the nodes of the small ones; < 0: the
                          large boxes first (default -1000: each pair of a
                          small and a large box is then found by the small
                          box's query), > 0: after the small ones.  Plain
-                         screens apply it with 10- or 12-bit Morton axes
+                         screens apply it with 10- or 12-bit axes
                          (ignored with 8 or 16), decomposed screens and
                          batches always.                                   */
   float refine_start; /* adaptive refinement: the first intervals of object i
@@ -216,12 +214,11 @@ SCD_API int scd_scene_set_elements_device(scd_scene *s, const scd_element *d_ele
 /* Tuning for later calls; NULL fields are not allowed, use scd_default_tuning. */
 SCD_API int scd_scene_set_tuning(scd_scene *s, const scd_tuning *t);
 SCD_API int scd_default_tuning(scd_tuning *t);
-/* The scene's tuning in force (a find may have deepened the stack after an
- * overflow).  Copied into *t. */
+/* The scene's tuning in force .  Copied into *t. */
 SCD_API int scd_scene_get_tuning(const scd_scene *s, scd_tuning *t);
 
 /* Steps A1-A4: per-object steps, FP64 propagation, outward-rounded FP32
- * boxes and 4D Morton keys (Defs 7-8, Sec. 4.5, Eq. 1).  Asynchronous apart
+ * boxes and 4D curve keys (Defs 7-8, Sec. 4.5, Eq. 1).  Asynchronous apart
  * from one read of the box count.  Errors: KEPLER_NOCONV, OOM, CUDA. */
 SCD_API int scd_build_boxes(scd_scene *s);
 
@@ -302,8 +299,8 @@ SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, int64_t n_pa
  *   rounds       (or NULL): the rounds taken, at most ceil(log2(max L_i)) + 2.
  * Needs scd_build_boxes (the per-object constants): else SCD_ERR_STATE.
  * Batches of scenes: SCD_ERR_INVALID_ARG.  n > 2^20: SCD_ERR_CAPACITY.
- * Meeting boxes are found per round by a Morton sort of the round's boxes,
- * a radix tree and the persistent traversal; all rounds are queued at once
+ * Meeting boxes are found per round by a sort of the round's boxes along the
+ * Hilbert curve, the 8-wide tree over them and the persistent traversal; all rounds are queued at once
  * with their sizes on the device.  The scene keeps the rounds' buffers (the
  * capacities that sufficed) and, after the first call of a shape, the
  * rounds' queue as a captured CUDA graph that later calls replay; both are

@@ -1,12 +1,10 @@
-"""Autotuner for the screen's tree and traversal parameters.
+"""Autotuner for the screen's tree parameters.
 
 Times whole screens (boxes through the canonical list) with CUDA events on
 the scene's stream for candidate tunings, keeps the fastest, and caches the
 choice in a JSON file keyed by GPU name, a hash of the workload and log2 of
-the box count.  A staged search: leaf size x Morton bits x space warp
-first, then the time weight, the stack depth, the size split of the key and
-the block shape (leaves of several boxes) or the nodes per traversal step
-and the node width (one box per leaf) around the winner.
+the box count.  A staged search: curve bits x space warp first, then the time
+weight and the size split of the key around the winner.
 """
 from __future__ import annotations
 
@@ -18,8 +16,7 @@ import os
 DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lib",
                              "autotune_cache.json")
 
-STAGE1 = [dict(leaf_size=L, morton_bits=b, space_warp=w)
-          for L in (1, 2, 4) for b in (8, 10, 12, 16) for w in (0, 1)]
+STAGE1 = [dict(morton_bits=b, space_warp=w) for b in (8, 10, 12, 16) for w in (0, 1)]
 
 
 def _time_screen(scene, reps: int, decomp=None) -> float:
@@ -50,8 +47,7 @@ def workload_key(elements, horizon_s: float, tick_s: float, step_desc: str, nbox
     return f"{name}|{h.hexdigest()[:16]}|log2N={int(math.log2(max(nboxes, 1)))}"
 
 
-STAGE1_DECOMPOSED = [dict(leaf_size=1, morton_bits=b, space_warp=w)
-                     for b in (8, 10, 12) for w in (0, 1)]
+STAGE1_DECOMPOSED = [dict(morton_bits=b, space_warp=w) for b in (8, 10, 12) for w in (0, 1)]
 
 
 def tune(scene, reps: int = 2, verbose: bool = False, decomp=None):
@@ -78,14 +74,9 @@ def tune(scene, reps: int = 2, verbose: bool = False, decomp=None):
         if ms < best_ms:
             best, best_ms = dict(cand), ms
     stage2 = [dict(best, time_scale=ts) for ts in (1.0, 4.0, 8.0, 16.0) if ts != base["time_scale"]]
-    stage2 += [dict(best, stack_depth=sd) for sd in (32, 128)]
     # the size split: off, a finer and a coarser threshold than the default
     stage2 += [dict(best, split_km=sk) for sk in (0.0, -500.0, -1000.0, -2000.0)
                if sk != base["split_km"]]
-    if best["leaf_size"] > 1:
-        stage2 += [dict(best, block_threads=bt) for bt in (64, 256)]
-    else:
-        stage2 += [dict(best, nodes_per_step=1), dict(best, node_width=4)]
     for cand in stage2:
         ms = run(cand)
         if ms < best_ms:

@@ -4,9 +4,11 @@
 // independent subtrees of one sorted reference array, traversed in one
 // persistent launch.
 //
-// A box is referenced from every cell it touches.  Keys are (cell, Morton):
-// one sort groups each cell's references, and in the radix tree over them
-// every cell is a subtree, whose root the traversal starts from.  A pair of
+// A box is referenced from every cell it touches.  Keys are (cell, position along
+// the Hilbert curve):
+// one sort groups each cell's references, and a query meets only positions
+// of its own cell: it starts at the smallest node of the tree that holds
+// itself and the cell's last reference, and leaves out what lies past it.  A pair of
 // boxes is reported only in the cell that holds a reference point common to
 // both, so it is reported once:
 //   SLAB_OCT   cells = n_slabs equal tick slabs x 8 ECI sign octants; the
@@ -102,21 +104,21 @@ __global__ void k_ref_count(const float4 *__restrict__ lo, const float4 *__restr
 }
 
 // A reference's key: its cell above the size bit (if any) above the top
-// mbits bits of the box's Morton key.  The key's time frame is the cell's
+// mbits bits of the box's curve key.  The key's time frame is the cell's
 // own: a tick slab's ticks, a batch scene's horizon, else the scene's.
 struct RefKeyArgs {
-  int bits;          // Morton bits per axis
-  int mbits;         // Morton bits kept (the top ones)
+  int bits;          // curve bits per axis
+  int mbits;         // curve bits kept (the top ones)
   float time_scale;
   int space_warp;
   float split_km;    // 0: no size bit
 };
 
-__device__ __forceinline__ unsigned long long ref_morton(const RefKeyArgs &k, float4 L, float4 H,
+__device__ __forceinline__ unsigned long long ref_curve(const RefKeyArgs &k, float4 L, float4 H,
                                                          float R, float t0, float T1) {
   L.w -= t0;
   H.w -= t0;
-  unsigned long long m = box_morton(L, H, R, T1, k.bits, k.time_scale, k.space_warp);
+  unsigned long long m = box_curve(L, H, R, T1, k.bits, k.time_scale, k.space_warp);
   m >>= (4 * k.bits - k.mbits);
   if (k.split_km != 0.0f)
     m |= (unsigned long long)split_bit(L, H, k.split_km) << k.mbits;
@@ -139,7 +141,7 @@ __global__ void k_ref_scatter(const float4 *__restrict__ lo, const float4 *__res
   if (d.kind == SCD_DECOMP_SLAB_OCT) {
     const float slab = (float)(d.T + 1) / (float)d.n_slabs;
     for (int s = c.s0; s <= c.s1; ++s) {
-      const unsigned long long m = ref_morton(ka, L, H, R, (float)s * slab, slab);
+      const unsigned long long m = ref_curve(ka, L, H, R, (float)s * slab, slab);
       for (int x = c.x0; x <= c.x1; ++x)
         for (int y = c.y0; y <= c.y1; ++y)
           for (int z = c.z0; z <= c.z1; ++z) {
@@ -153,7 +155,7 @@ __global__ void k_ref_scatter(const float4 *__restrict__ lo, const float4 *__res
     }
   } else {
     const float T1 = (float)((d.objT ? (int64_t)d.objT[ob] : d.T) + 1);
-    const unsigned long long m = ref_morton(ka, L, H, R, 0.0f, T1);
+    const unsigned long long m = ref_curve(ka, L, H, R, 0.0f, T1);
     for (int k = c.b0; k <= c.b1; ++k) {
       if (o < cap) {
         key[o] = ((unsigned long long)k << cshift) | m;
@@ -164,32 +166,16 @@ __global__ void k_ref_scatter(const float4 *__restrict__ lo, const float4 *__res
   }
 }
 
-// First and last reference of every cell, then the root of its subtree: the
-// internal node whose leaf range is exactly [first, last] (in a radix tree
-// its index is one of the two ends).
-__global__ void k_cell_bounds(const uint32_t *__restrict__ scell, int64_t R,
-                              int32_t *__restrict__ cfirst, int32_t *__restrict__ clast) {
+// one past the last reference of every cell that has any
+__global__ void k_cell_ends(const uint32_t *__restrict__ scell, int64_t R,
+                            int32_t *__restrict__ cend) {
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= R) return;
   uint32_t c = scell[p];
-  if (p == 0 || scell[p - 1] != c) cfirst[c] = (int32_t)p;
-  if (p == R - 1 || scell[p + 1] != c) clast[c] = (int32_t)p;
+  if (p == R - 1 || scell[p + 1] != c) cend[c] = (int32_t)p + 1;
 }
 
-__global__ void k_cell_roots(const int32_t *__restrict__ cfirst, const int32_t *__restrict__ clast,
-                             int n_cells, const int32_t *__restrict__ first,
-                             const TravNode *__restrict__ nodes, int32_t *__restrict__ root) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cells) return;
-  int32_t f = cfirst[c], l = clast[c];
-  if (f < 0 || l <= f) {
-    root[c] = -1;  // empty or a single reference: no pair inside
-    return;
-  }
-  root[c] = (first[f] == f && nodes[f].last_r == l) ? f : l;
-}
-
-int build_decomposed(scd_scene *s, const scd_decomp *dc, int64_t &M, bool capturing) {
+int build_decomposed(scd_scene *s, const scd_decomp *dc, bool capturing) {
   cudaStream_t st = s->stream;
   const int64_t N = s->N;
   DecompArgs d;
@@ -244,11 +230,9 @@ int build_decomposed(scd_scene *s, const scd_decomp *dc, int64_t &M, bool captur
     if (R <= 0 || R >= (1ll << 30)) return SCD_ERR_CAPACITY;
     s->n_refs = R;
   }
-  if (!s->d_refkey.ensure(R, st) || !s->d_refid.ensure(R, st) ||
-      !s->s_leafkey64.ensure(R, st) || !s->d_cellroot.ensure(n_cells, st) ||
-      !s->d_refcnt.ensure(2 * (size_t)n_cells > (size_t)N ? 2 * n_cells : N, st))
+  if (!s->d_refkey.ensure(R, st) || !s->d_refid.ensure(R, st) || !s->d_cellend.ensure(n_cells, st))
     return SCD_ERR_OOM;
-  // the cell's bits above the size bit and as many of the Morton key's top
+  // the cell's bits above the size bit and as many of the curve key's top
   // bits as the rest of 64 holds
   int cbits = 1;
   while ((1 << cbits) < n_cells) ++cbits;
@@ -266,16 +250,10 @@ int build_decomposed(scd_scene *s, const scd_decomp *dc, int64_t &M, bool captur
   const int cshift = ka.mbits + sb;
   rc = radix_sort_u64(s->d_refkey.p, s->d_refid.p, R, cshift + cbits, s->sort_sc, st);
   if (rc) return rc;
-  rc = build_tree<unsigned long long>(s, s->d_refkey.p, s->d_refid.p, R, s->s_leafkey64.p, cshift,
-                                      M);
+  rc = build_tree(s, s->d_refkey.p, s->d_refid.p, R, cshift);
   if (rc) return rc;
-  // cell bounds (reusing the count buffer as two int32 arrays) and roots
-  int32_t *cfirst = (int32_t *)s->d_refcnt.p, *clast = cfirst + n_cells;
-  cudaMemsetAsync(cfirst, 0xff, sizeof(int32_t) * 2 * (size_t)n_cells, st);
-  k_cell_bounds<<<(unsigned)((R + bs - 1) / bs), bs, 0, st>>>(s->s_cell.p, R, cfirst, clast);
-  k_cell_roots<<<(unsigned)((n_cells + bs - 1) / bs), bs, 0, st>>>(
-      cfirst, clast, n_cells, s->d_first.p, s->d_nodes.p, s->d_cellroot.p);
-  note_launch(2);
+  k_cell_ends<<<(unsigned)((R + bs - 1) / bs), bs, 0, st>>>(s->s_cell.p, R, s->d_cellend.p);
+  note_launch();
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
 

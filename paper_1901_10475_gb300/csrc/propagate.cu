@@ -1,7 +1,7 @@
 // propagate.cu -- steps A1-A4 of the screen: per-object step policy, FP64
 // two-body propagation (Sec. 6.1, Eq. 1 solved through Kepler's equation),
 // interval occupancy boxes (Def 7, Def 8, Sec. 4.5) rounded outward to FP32,
-// and the 4D Morton key of every box.
+// and the 4D curve key of every box.
 #include <math.h>
 
 #include <mutex>
@@ -133,10 +133,10 @@ struct BoxArgs {
   float T1f;         // T + 1 (the key frame's time extent)
   double tick_s;
   int mode;
-  int bits;          // Morton bits per axis
+  int bits;          // curve bits per axis
   float time_scale;  // weight of the time axis in the key
   int space_warp;    // log-compress space coordinates before quantising
-  float split_km;    // large boxes sorted apart (one key bit above the Morton key)
+  float split_km;    // large boxes sorted apart (one key bit above the curve key)
   DevCounters *ctr;
   float4 *lo, *hi;
   uint32_t *obj;
@@ -185,9 +185,9 @@ __global__ void __launch_bounds__(256) k_build_boxes(BoxArgs a) {
   a.obj[b] = (uint32_t)i;
   a.id[b] = (uint32_t)b;
 
-  // 4D Morton key of the box centre in the scene's bounding cube
+  // 4D Hilbert key of the box centre in the scene's bounding cube
   const float R = (float)__longlong_as_double((long long)a.ctr->extent_bits);
-  unsigned long long key = box_morton(L, H, R, a.T1f, a.bits, a.time_scale, a.space_warp);
+  unsigned long long key = box_curve(L, H, R, a.T1f, a.bits, a.time_scale, a.space_warp);
   key = sort_key(key, split_bit(L, H, a.split_km), a.bits, a.split_km != 0.0f);
   if (a.key64) a.key64[b] = key;
   else a.key32[b] = (uint32_t)key;

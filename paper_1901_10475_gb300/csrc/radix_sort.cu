@@ -1,5 +1,5 @@
 // radix_sort.cu -- LSD radix sort of 32- or 64-bit keys with optional 32-bit
-// values (step A5: ordering boxes along the 4D Morton curve; step A9:
+// values (step A5: ordering boxes along the 4D Hilbert curve; step A9:
 // ordering candidate records by (i, j, tick)).
 //
 // Reduce-then-scan per 8-bit digit: (1) every block counts the digits of its

@@ -34,8 +34,8 @@
 // interval.
 //
 // The meeting boxes of a round are found with the screen's machinery: the
-// boxes are sorted along a 4D Morton curve, a binary radix tree with
-// compact quantised nodes is built over them, and the persistent traversal
+// boxes are sorted along a 4D Hilbert curve, the implicit 8-wide tree is
+// built over them, and the persistent traversal
 // (in its refinement mode) flags both intervals of every meeting pair and
 // collects the candidates.  The rounds run without the host: every kernel
 // reads the round's interval count from device memory, and the host queues
@@ -66,10 +66,10 @@ enum {
   RF_NCAND = 0, RF_NNEXT = 1, RF_ERR = 2, RF_NUNIQ = 3, RF_NWIT = 4, RF_M = 5, RF_OVER = 6,
   RF_LMAX = 7, RF_WORDS = 8
 };
-// the rounds' 4D Morton keys: 10 bits per axis, time weighed 4x against
+// the rounds' 4D curve keys: 10 bits per axis, time weighed 4x against
 // space (24 h catalog rounds 552 -> 522 ms against equal weights; 12-bit axes
 // with weight 8, the screen's choice, 519 ms but slower on small rounds)
-constexpr int kRfMortonBits = 10;
+constexpr int kRfCurveBits = 10;
 constexpr float kRfTimeScale = 4.0f;
 
 __device__ __forceinline__ int64_t rf_count(const unsigned long long *state, int64_t cap) {
@@ -156,7 +156,7 @@ struct RfBoxArgs {
   unsigned long long *err;
 };
 
-// the box, Morton key and index of interval i
+// the box, curve key and index of interval i
 __device__ __forceinline__ void rf_box(const RfBoxArgs &a, int64_t i) {
   const ObjParams &p = a.par[a.obj[i]];
   const int32_t t0 = a.t0[i], t1 = a.t1[i];
@@ -177,8 +177,8 @@ __device__ __forceinline__ void rf_box(const RfBoxArgs &a, int64_t i) {
   a.hi[i] = H;
   const float R = (float)__longlong_as_double((long long)a.ctr->extent_bits);
   unsigned long long k =
-      box_morton(L, H, R, (float)(a.Tf + 1), kRfMortonBits, kRfTimeScale, 0);
-  k |= (unsigned long long)split_bit(L, H, a.split_km) << (4 * kRfMortonBits);
+      box_curve(L, H, R, (float)(a.Tf + 1), kRfCurveBits, kRfTimeScale, 0);
+  k |= (unsigned long long)split_bit(L, H, a.split_km) << (4 * kRfCurveBits);
   a.key[i] = k;
   a.idx[i] = (uint32_t)i;
 }
@@ -188,24 +188,6 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_boxes(RfBoxArgs a) {
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i0 == 0) *a.round_count = (unsigned long long)M;
   for (int64_t i = i0; i < M; i += (int64_t)gridDim.x * blockDim.x) rf_box(a, i);
-}
-
-// the sorted boxes (32-byte records) and their objects
-__global__ void __launch_bounds__(kRfThreads) k_rf_gather(const uint32_t *__restrict__ idx,
-                                                          const float4 *__restrict__ lo,
-                                                          const float4 *__restrict__ hi,
-                                                          const uint32_t *__restrict__ obj,
-                                                          int64_t cap,
-                                                          const unsigned long long *state,
-                                                          SBox *sbox, uint32_t *sobj) {
-  const int64_t M = rf_count(state, cap);
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < M;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t i = idx[p];
-    sbox[p].lo = lo[i];
-    sbox[p].hi = hi[i];
-    sobj[p] = obj[i];
-  }
 }
 
 // Slots for `need` next-round intervals of each lane of a warp: one atomic
@@ -392,13 +374,12 @@ __global__ void k_rf_decode(const unsigned long long *__restrict__ wkey, int64_t
 // device buffers of one call, released on every return path
 struct RfBuffers {
   cudaStream_t st;
-  DevBuf<uint32_t> obj[2], idx, flags, sobj, qlink, arrive;
-  DevBuf<int32_t> t0[2], t1[2], first, parent_int, parent_leaf;
+  DevBuf<uint32_t> obj[2], idx, flags, sobj;
+  DevBuf<int32_t> t0[2], t1[2], first;
   DevBuf<float4> lo, hi;
   DevBuf<unsigned long long> key, cand, state, wkey, rounds;
-  DevBuf<SBox> sbox;
-  DevBuf<TravNode> nodes;
-  DevBuf<QBox> nq, qbox;
+  DevBuf<SBox> sbox, nbox;
+  DevBuf<WideNode> nodes;
   DevBuf<DevCounters> ctr;
   DevBuf<uint32_t> sort_err;
   DevBuf<scd_pair> pairs;
@@ -420,11 +401,10 @@ struct RfBuffers {
       t0[b].release(st);
       t1[b].release(st);
     }
-    idx.release(st); flags.release(st); sobj.release(st); qlink.release(st);
-    arrive.release(st); first.release(st); parent_int.release(st); parent_leaf.release(st);
+    idx.release(st); flags.release(st); sobj.release(st); first.release(st);
     lo.release(st); hi.release(st); key.release(st); cand.release(st); state.release(st);
-    wkey.release(st); rounds.release(st); sbox.release(st); nodes.release(st); nq.release(st);
-    qbox.release(st); ctr.release(st); sort_err.release(st); pairs.release(st);
+    wkey.release(st); rounds.release(st); sbox.release(st); nbox.release(st); nodes.release(st);
+    ctr.release(st); sort_err.release(st); pairs.release(st);
     wit.release(st); span.release(st); tlo.release(st); thi.release(st); tobj.release(st);
     scnt.release(st); soff.release(st); stmp.release(st);
     sc.release(st);
@@ -436,11 +416,11 @@ struct RfBuffers {
     const size_t c = (size_t)cap;
     for (int b = 0; b < 2; ++b)
       if (!obj[b].ensure(c, st) || !t0[b].ensure(c, st) || !t1[b].ensure(c, st)) return false;
-    return idx.ensure(c, st) && flags.ensure(c, st) && sobj.ensure(c, st) &&
-           qlink.ensure(c, st) && arrive.ensure(c, st) && parent_int.ensure(c, st) &&
-           parent_leaf.ensure(c, st) && lo.ensure(c, st) && hi.ensure(c, st) &&
-           key.ensure(c, st) && sbox.ensure(c, st) && nodes.ensure(c, st) && nq.ensure(c, st) &&
-           qbox.ensure(2 * c, st) && cand.ensure((size_t)ccap, st) &&
+    if (cap > kMaxTreeBoxes) return false;
+    return idx.ensure(c, st) && flags.ensure(c, st) && sobj.ensure(c, st) && lo.ensure(c, st) &&
+           hi.ensure(c, st) && key.ensure(c, st) && sbox.ensure(c, st) &&
+           nbox.ensure((size_t)tree_scratch_boxes(cap), st) &&
+           nodes.ensure(tree_levels(cap).total, st) && cand.ensure((size_t)ccap, st) &&
            sort_reserve(sc, cap, sizeof(unsigned long long), true, st) == SCD_OK;
   }
 };
@@ -509,9 +489,9 @@ static int rf_start(scd_scene *s, RfBuffers &B, int &rounds) {
 // intervals (rf_start) until nothing is left (at most `rounds` of them).  Continuous
 // (levels >= 0): level l = 0 .. levels in units of T_s / 2^l, spans at the
 // last.  On return h holds the state words and round_counts the intervals
-// of every round; the caller checks capacity, candidates and the stack.
-static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int deep,
-                    int rounds, int levels) {
+// of every round; the caller checks capacity and candidates.
+static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int rounds,
+                    int levels) {
   cudaStream_t st = B.st;
   const int64_t n = s->n;
   if (cudaMemsetAsync(B.state.p, 0, sizeof(unsigned long long) * RF_WORDS, st) != cudaSuccess ||
@@ -534,7 +514,7 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int d
                                                              B.state.p);
   note_launch();
   const float split = split_of(s->tune);
-  const int kb = 4 * kRfMortonBits + (split != 0.0f);
+  const int kb = 4 * kRfCurveBits + (split != 0.0f);
   unsigned long long *dM = B.state.p + RF_M;
   const int nr = cont ? levels + 1 : rounds;
   int cur = 0;
@@ -556,12 +536,8 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int d
     }
     int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, 0, kb, B.sc, st);
     if (rc != SCD_OK) return rc;
-    k_rf_gather<<<wave_of(cap), kRfThreads, 0, st>>>(B.idx.p, B.lo.p, B.hi.p, B.obj[cur].p, cap,
-                                                     B.state.p, B.sbox.p, B.sobj.p);
-    note_launch();
-    rc = build_round_tree(B.key.p, B.sbox.p, cap, dM, B.nodes.p, B.parent_int.p,
-                          B.parent_leaf.p, B.arrive.p, B.nq.p, B.qbox.p, B.qlink.p, B.ctr.p, Tf,
-                          st);
+    rc = build_round_tree(B.idx.p, B.lo.p, B.hi.p, B.obj[cur].p, cap, dM, B.sbox.p, B.sobj.p,
+                          B.nodes.p, B.nbox.p, st);
     if (rc != SCD_OK) return rc;
     // the flags, and the traversal's counters (its error bits, which follow
     // them, stay set across the rounds)
@@ -569,9 +545,8 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int d
         cudaMemsetAsync(B.ctr.p, 0, offsetof(DevCounters, trav_flags), st) != cudaSuccess)
       return SCD_ERR_CUDA;
     const int spans = cont && r == levels;
-    rc = traverse_round(B.qbox.p, B.qlink.p, B.sbox.p, B.sobj.p, B.idx.p, cap, dM, Tf, B.ctr.p,
-                        B.flags.p, B.cand.p, B.state.p + RF_NCAND, (unsigned long long)ccap,
-                        spans, deep, st);
+    rc = traverse_round(B.nodes.p, B.sbox.p, B.sobj.p, B.idx.p, cap, dM, Tf, B.ctr.p, B.flags.p,
+                        B.cand.p, B.state.p + RF_NCAND, (unsigned long long)ccap, spans, st);
     if (rc != SCD_OK) return rc;
     if (spans) break;
     if (cont)
@@ -589,12 +564,10 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int d
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
 
-// the rounds' sizes, the traversal flags and the state words, after the queue
+// the rounds' sizes and the state words, after the queue
 static int rf_collect(RfBuffers &B, unsigned long long h[RF_WORDS],
-                      unsigned long long *round_counts, unsigned int &trav_flags) {
+                      unsigned long long *round_counts) {
   if (cudaMemcpyAsync(round_counts, B.rounds.p, sizeof(unsigned long long) * kRfMaxRounds,
-                      cudaMemcpyDeviceToHost, B.st) != cudaSuccess ||
-      cudaMemcpyAsync(&trav_flags, &B.ctr.p->trav_flags, sizeof(unsigned int),
                       cudaMemcpyDeviceToHost, B.st) != cudaSuccess)
     return SCD_ERR_CUDA;
   return rf_read_state(B, h);
@@ -623,11 +596,11 @@ struct RfCache {
   }
 };
 
-static void rf_key(const scd_scene *s, const RfBuffers &B, int64_t cap, int64_t ccap, int deep,
-                   int rounds, int levels, int64_t k[11]) {
+static void rf_key(const scd_scene *s, const RfBuffers &B, int64_t cap, int64_t ccap, int rounds,
+                   int levels, int64_t k[11]) {
   k[0] = cap;
   k[1] = ccap;
-  k[2] = deep;
+  k[2] = 0;
   k[3] = rounds;
   k[4] = levels;
   k[5] = s->n;
@@ -643,10 +616,10 @@ static void rf_key(const scd_scene *s, const RfBuffers &B, int64_t cap, int64_t 
 // queue the rounds: by the cached graph when its shape matches, else
 // eagerly
 static int rf_rounds(scd_scene *s, RfBuffers &B, RfCache *gc, int64_t cap, int64_t ccap,
-                     int deep, int rounds, int levels, unsigned long long h[RF_WORDS],
-                     unsigned long long *round_counts, unsigned int &trav_flags) {
+                     int rounds, int levels, unsigned long long h[RF_WORDS],
+                     unsigned long long *round_counts) {
   int64_t k[11];
-  rf_key(s, B, cap, ccap, deep, rounds, levels, k);
+  rf_key(s, B, cap, ccap, rounds, levels, k);
   if (gc && gc->exec && memcmp(k, gc->key, sizeof(k)) == 0) {
     if (cudaEventRecord(gc->in, B.st) != cudaSuccess ||
         cudaStreamWaitEvent(gc->gst, gc->in, 0) != cudaSuccess ||
@@ -656,17 +629,17 @@ static int rf_rounds(scd_scene *s, RfBuffers &B, RfCache *gc, int64_t cap, int64
       return SCD_ERR_CUDA;
     note_launch(gc->nlaunch);
   } else {
-    int rc = rf_queue(s, B, cap, ccap, deep, rounds, levels);
+    int rc = rf_queue(s, B, cap, ccap, rounds, levels);
     if (rc != SCD_OK) return rc;
   }
-  return rf_collect(B, h, round_counts, trav_flags);
+  return rf_collect(B, h, round_counts);
 }
 
 // capture the queue of a shape that has just run eagerly (nothing is
 // allocated while capturing: every buffer is sized); without a graph the
 // calls stay eager
-static void rf_capture(scd_scene *s, RfCache &gc, int64_t cap, int64_t ccap, int deep,
-                       int rounds, int levels) {
+static void rf_capture(scd_scene *s, RfCache &gc, int64_t cap, int64_t ccap, int rounds,
+                       int levels) {
   if (!gc.gst) {
     if (cudaStreamCreateWithFlags(&gc.gst, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&gc.in, cudaEventDisableTiming) != cudaSuccess ||
@@ -688,13 +661,13 @@ static void rf_capture(scd_scene *s, RfCache &gc, int64_t cap, int64_t ccap, int
   const cudaStream_t st = gc.B.st;
   gc.B.st = gc.gst;
   const unsigned long long mark = launch_count();
-  const int rc = rf_queue(s, gc.B, cap, ccap, deep, rounds, levels);
+  const int rc = rf_queue(s, gc.B, cap, ccap, rounds, levels);
   const cudaError_t e = cudaStreamEndCapture(gc.gst, &g);
   gc.B.st = st;
   gc.nlaunch = launch_count() - mark;
   if (rc == SCD_OK && e == cudaSuccess && g &&
       cudaGraphInstantiate(&gc.exec, g, 0) == cudaSuccess) {
-    rf_key(s, gc.B, cap, ccap, deep, rounds, levels, gc.key);
+    rf_key(s, gc.B, cap, ccap, rounds, levels, gc.key);
   } else {
     gc.exec = nullptr;
     cudaGetLastError();
@@ -705,9 +678,9 @@ static void rf_capture(scd_scene *s, RfCache &gc, int64_t cap, int64_t ccap, int
 }  // namespace scd
 
 namespace scd {
-// Queue the rounds, and again with more room while a round's intervals, the
-// candidates or a traversal stack did not fit.  The capacities that sufficed
-// stay on the scene for its next call.
+// Queue the rounds, and again with more room while a round's intervals or the
+// candidates did not fit.  The capacities that sufficed stay on the scene for
+// its next call.
 // Discrete rounds (levels < 0) set `rounds` from their first intervals.
 static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int levels,
                   unsigned long long h[RF_WORDS], unsigned long long *round_counts) {
@@ -725,11 +698,9 @@ static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int leve
     cap = std::max<int64_t>(cap, B.start_total);
   }
   int64_t ccap = std::max<int64_t>(s->rf_ccap, 1 << 16);
-  int deep = s->rf_deep;
   for (int attempt = 0; attempt < 8; ++attempt) {
     if (!B.size(cap, ccap)) return SCD_ERR_OOM;
-    unsigned int tf = 0;
-    int rc = rf_rounds(s, B, gc, cap, ccap, deep, rounds, levels, h, round_counts, tf);
+    int rc = rf_rounds(s, B, gc, cap, ccap, rounds, levels, h, round_counts);
     if (rc != SCD_OK) return rc;
     bool again = false;
     if (h[RF_OVER] > (unsigned long long)cap) {
@@ -740,20 +711,14 @@ static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int leve
       ccap = (int64_t)(2ull * h[RF_NCAND]);
       again = true;
     }
-    if (tf & ERR_STACK) {
-      if (deep) return SCD_ERR_INTERNAL;
-      deep = 1;
-      again = true;
-    }
     if (!again) {
       s->rf_cap = cap;
       s->rf_ccap = ccap;
-      s->rf_deep = deep;
       if (gc) {
         int64_t k[11];
-        rf_key(s, B, cap, ccap, deep, rounds, levels, k);
+        rf_key(s, B, cap, ccap, rounds, levels, k);
         if (!gc->exec || memcmp(k, gc->key, sizeof(k)) != 0)
-          rf_capture(s, *gc, cap, ccap, deep, rounds, levels);
+          rf_capture(s, *gc, cap, ccap, rounds, levels);
       }
       return SCD_OK;
     }

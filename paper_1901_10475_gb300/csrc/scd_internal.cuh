@@ -24,7 +24,6 @@ constexpr double kEpsKm = 1e-6;
 // device error word bits
 enum : uint32_t {
   ERR_KEPLER = 1u << 0,     // Kepler iteration hit its limit
-  ERR_STACK = 1u << 1,      // traversal stack overflow
   ERR_INVALID = 1u << 2,    // invalid element seen on the device
   ERR_ZIP = 1u << 3,        // open run starts and run ends did not pair up
   ERR_SORT = 1u << 4,       // a sort's tile copy did not arrive in time
@@ -63,7 +62,7 @@ struct DevCounters {
   unsigned long long node_tests;
   unsigned long long leaf_tests;
   unsigned long long work_next;  // next query claimed by the persistent traversal
-  unsigned int trav_flags;   // ERR_STACK, ERR_ZIP
+  unsigned int trav_flags;   // ERR_ZIP
   unsigned int pad0;
   unsigned long long extent_bits;  // max object extent [km] as double bits
   unsigned int build_flags;        // ERR_KEPLER, ERR_INVALID
@@ -74,49 +73,66 @@ struct DevCounters {
   unsigned int pad1;
 };
 
-// Traversal node: both children's boxes inline, child links and the
-// rightmost leaf of each child (80 bytes).
-struct __align__(16) TravNode {
-  float4 lo_l, hi_l, lo_r, hi_r;
-  int32_t left, right;  // child index; bit 31 set = leaf
-  int32_t last_l, last_r;  // rightmost leaf index under each child
+// The 4D box hierarchy: an implicit 8-wide tree over the sorted boxes.  Node
+// m of level k covers the sorted boxes [m 8^k, (m + 1) 8^k), so there are no
+// links and no depth to discover; its children are the nodes 8 m .. 8 m + 7
+// of level k - 1 (the boxes themselves below level 1).  A node holds its
+// frame (per axis a scale and an offset that map its own box onto [0, 127])
+// and its children's faces in that frame, one byte each, axis by axis with
+// the eight children side by side: a query is brought into the frame once
+// and then tested against four children per instruction.  The upper faces
+// carry the guard bit 0x80, so that a byte-wise difference with a lower face
+// (at most 127) never borrows from its neighbour and its top bit says
+// whether upper >= lower.  Children and queries go through the same monotone
+// map (node_coord), so a test in the frame never rejects a pair that overlaps
+// in FP32.  96 bytes, three 32-byte loads for eight child boxes (12 bytes a
+// child).
+struct __align__(32) WideNode {
+  float scale[4], off[4];       // x, y, z, tick
+  uint32_t lo[4][2], hi[4][2];  // per axis: children 0-3, children 4-7
 };
+static_assert(sizeof(WideNode) == 96, "three 32-byte sectors per node");
+constexpr int kWide = 8, kWideBits = 3;
+// 8^10 boxes: sorted positions are below 2^30
+constexpr int kMaxLevels = 10;
+constexpr int64_t kMaxTreeBoxes = 1ll << (kWideBits * kMaxLevels);
 
-static_assert(sizeof(TravNode) == 80 && offsetof(TravNode, left) == 64,
-              "the links are the node's fifth 16-byte word");
-
-constexpr int32_t kLeafBit = (int32_t)0x80000000u;
-
-// Compact node of the one-box-per-leaf traversal (36 bytes): both child
-// boxes quantised in the scene frame (lower faces rounded down, upper faces
-// up, so a quantised test never rejects a pair that overlaps in FP32) and
-// the split gamma (left child gamma, right child gamma + 1) with two leaf
-// flags; gamma is also the left child's rightmost leaf.  x and y take 16 bits, z 15 and the tick 17: one
-// quantum per tick up to 131071 ticks, so boxes of consecutive segments
-// (which touch, tick hi + 1 = tick lo, but do not overlap) stay apart.
-struct __align__(16) QBox {
-  uint32_t lo_xy, lo_zt, hi_xy, hi_zt;  // x | y << 16 and z | t << 15
+// the levels' places in one array of nodes, for up to `cap` boxes: level k
+// (1 .. levels) holds ceil(cap / 8^k) nodes from off[k]; the last has one
+struct TreeLevels {
+  int levels;
+  uint32_t off[kMaxLevels + 1];
+  uint32_t total;
 };
-constexpr uint32_t kQLeftLeaf = 0x80000000u, kQRightLeaf = 0x40000000u;
-constexpr uint32_t kQIndex = 0x3fffffffu;
+inline TreeLevels tree_levels(int64_t cap) {
+  TreeLevels t{};
+  int64_t c = cap;
+  uint32_t at = 0;
+  for (int k = 1; k <= kMaxLevels && (k == 1 || c > 1); ++k) {
+    c = (c + kWide - 1) / kWide;
+    t.off[k] = at;
+    at += (uint32_t)c;
+    t.levels = k;
+  }
+  t.total = at;
+  return t;
+}
 
-// Four-wide node (one box per leaf, node width 4): the grandchildren of a
-// binary node in one 128-byte line.  Slots 0 and 1 hold the two children of
-// the left child (or the left child itself when it is a leaf, and an empty
-// slot), slots 2 and 3 those of the right child.  link.x = binary node or
-// leaf index with flags, link.y = the slot's rightmost leaf (0 when empty).
-// One traversal step reads the line with three 256-bit loads and descends
-// two binary levels.
-struct __align__(128) W4Node {
-  QBox box[4];
-  uint2 link[4];
-  uint32_t pad[8];
-};
-static_assert(sizeof(W4Node) == 128, "one cache line per four-wide node");
-constexpr uint32_t kW4Leaf = 0x80000000u, kW4Empty = 0x40000000u, kW4Index = 0x3fffffffu;
-// the right-child bit of a parent link (the Karras build marks which side
-// of its parent each internal node is)
-constexpr int32_t kRightChildBit = 0x40000000;
+// A coordinate in a node's frame, as a float whose lowest byte is the cell
+// in [0, 127] (plus the guard bit when asked for): scaled and clamped to
+// [0, 1], then added to 2^23 with rounding down, where one unit is the last
+// place.  Both steps are monotone in x for a fixed frame, so order
+// relations survive (a NaN clamps to 0: a frame that is not finite has scale
+// and offset 0, and every coordinate becomes 0).
+constexpr float kCellTop = 127.9f;
+__device__ __forceinline__ uint32_t node_coord(float x, float scale, float off, bool guard) {
+  float s, u;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(s) : "f"(x), "f"(scale), "f"(off));
+  asm("fma.rm.f32 %0, %1, %2, %3;"
+      : "=f"(u)
+      : "f"(s), "f"(kCellTop), "f"(guard ? 8388608.0f + 128.0f : 8388608.0f));
+  return __float_as_uint(u);
+}
 
 // A sorted box: both corners in one 32-byte record (x, y, z in km, the tick
 // in w), read with one 256-bit load.
@@ -130,61 +146,12 @@ __device__ __forceinline__ void ldg_box(const SBox *p, float4 &lo, float4 &hi) {
       : "l"(p));
 }
 
-// Both child boxes of a compact node (32 bytes, 32-byte aligned) in one
-// 256-bit read-only load.
-__device__ __forceinline__ void ldg_qbox_pair(const QBox *p, uint4 &l, uint4 &r) {
+// 32 bytes of a node in one 256-bit read-only load
+__device__ __forceinline__ void ldg_words(const void *p, uint32_t w[8]) {
   asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(l.x), "=r"(l.y), "=r"(l.z), "=r"(l.w), "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
+        "=r"(w[7])
       : "l"(p));
-}
-// the four links of a four-wide node
-__device__ __forceinline__ void ldg_w4_links(const uint2 *p, uint4 &a, uint4 &b) {
-  asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-      : "l"(p));
-}
-
-// the scene frame of the quantisation: x, y, z in [-R, R] km, t in [0, T]
-struct QFrame {
-  float R, sx, sz, st;  // sx = 65535 / 2R, sz = 32767 / 2R, st = min(1, 131071 / T)
-};
-
-// the frame of a scene, from the extent found by the box build; every kernel
-// that quantises derives it with this same code, so the values agree
-__device__ inline QFrame scene_frame(const DevCounters *ctr, int64_t T) {
-  QFrame f;
-  f.R = (float)__longlong_as_double((long long)ctr->extent_bits);
-  f.sx = 65535.0f / (2.0f * f.R);
-  f.sz = 32767.0f / (2.0f * f.R);
-  f.st = fminf(1.0f, 131071.0f / (float)(T > 0 ? T : 1));
-  return f;
-}
-
-// outward quantisation to [0, top]
-__host__ __device__ inline uint32_t q_lo(float v, float top) {
-  float f = floorf(v);
-  f = f < 0.f ? 0.f : (f > top ? top : f);
-  return (uint32_t)f;
-}
-__host__ __device__ inline uint32_t q_hi(float v, float top) {
-  float f = ceilf(v);
-  f = f < 0.f ? 0.f : (f > top ? top : f);
-  return (uint32_t)f;
-}
-// quantise a box outward; the map x -> (x + R) * sx is monotone in FP32, so
-// box order relations survive it
-__host__ __device__ inline QBox quantize_box(const QFrame &f, float4 lo, float4 hi) {
-  QBox q;
-  q.lo_xy = q_lo((lo.x + f.R) * f.sx, 65535.f) | (q_lo((lo.y + f.R) * f.sx, 65535.f) << 16);
-  q.lo_zt = q_lo((lo.z + f.R) * f.sz, 32767.f) | (q_lo(lo.w * f.st, 131071.f) << 15);
-  q.hi_xy = q_hi((hi.x + f.R) * f.sx, 65535.f) | (q_hi((hi.y + f.R) * f.sx, 65535.f) << 16);
-  q.hi_zt = q_hi((hi.z + f.R) * f.sz, 32767.f) | (q_hi(hi.w * f.st, 131071.f) << 15);
-  return q;
-}
-
-// a <= b in both fields of a z | t << 15 word
-__device__ __forceinline__ bool zt_le(uint32_t a, uint32_t b) {
-  return (a & 0x7fffu) <= (b & 0x7fffu) && (a >> 15) <= (b >> 15);
 }
 
 __device__ inline uint32_t quantize(float u, int bits) {
@@ -194,27 +161,57 @@ __device__ inline uint32_t quantize(float u, int bits) {
   return (uint32_t)q;
 }
 
-__device__ inline unsigned long long morton4(uint32_t x, uint32_t y, uint32_t z, uint32_t t,
-                                             int bits) {
-  unsigned long long key = 0;
-  for (int b = 0; b < bits; ++b) {
-    key |= (unsigned long long)((t >> b) & 1u) << (4 * b + 0);
-    key |= (unsigned long long)((z >> b) & 1u) << (4 * b + 1);
-    key |= (unsigned long long)((y >> b) & 1u) << (4 * b + 2);
-    key |= (unsigned long long)((x >> b) & 1u) << (4 * b + 3);
-  }
-  return key;
+// the bits of a 16-bit value spread to every fourth bit
+__device__ __forceinline__ unsigned long long spread4(uint32_t v) {
+  unsigned long long x = v & 0xffffull;
+  x = (x | (x << 24)) & 0x000000ff000000ffull;
+  x = (x | (x << 12)) & 0x000f000f000f000full;
+  x = (x | (x << 6)) & 0x0303030303030303ull;
+  x = (x | (x << 3)) & 0x1111111111111111ull;
+  return x;
 }
 
-// 4D Morton key (bits per axis) of a box centre in the scene cube [-R, R]^3
-// x [0, T]; optionally log-compressed in space (a monotone map, so any key
-// order is a valid tree order).  time_scale weighs time against space: below
-// 1 the horizon takes that share of the time axis's cells, above 1 the
-// scene cube takes 1 / time_scale of the space axes' cells (around the
-// centre), so time counts that many times more in the curve's order.
-// R is the cube's half-side, T1 the horizon plus one tick; all in FP32.
-__device__ inline unsigned long long box_morton(float4 L, float4 H, float R, float T1, int bits,
-                                                float time_scale, int space_warp) {
+// The position of a cell along the 4D Hilbert curve of `bits` bits per axis
+// (J. Skilling, "Programming the Hilbert curve", 2004: from the coarsest bit
+// down, each axis' bit inverts or exchanges the finer bits of the first
+// axis, then a Gray code).  Consecutive cells of the curve share a face, so
+// eight consecutive boxes always form a compact node; along the Morton
+// curve, whose jumps fall inside such groups, a query of the 24 h catalog
+// screen visits 51 nodes instead of 37.
+__device__ inline unsigned long long hilbert4(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
+                                              int bits) {
+  for (uint32_t q = 1u << (bits - 1); q > 1u; q >>= 1) {
+    const uint32_t p = q - 1u;
+    auto turn = [&](uint32_t &xi) {
+      const uint32_t t = (xi & q) ? p : 0u;          // invert the first axis' finer bits
+      const uint32_t e = (xi & q) ? 0u : (x0 ^ xi) & p;  // or exchange them with axis i's
+      x0 ^= t ^ e;
+      xi ^= e;
+    };
+    if (x0 & q) x0 ^= p;
+    turn(x1);
+    turn(x2);
+    turn(x3);
+  }
+  x1 ^= x0;
+  x2 ^= x1;
+  x3 ^= x2;
+  uint32_t t = 0;
+  for (uint32_t q = 1u << (bits - 1); q > 1u; q >>= 1)
+    if (x3 & q) t ^= q - 1u;
+  return spread4(x0 ^ t) << 3 | spread4(x1 ^ t) << 2 | spread4(x2 ^ t) << 1 | spread4(x3 ^ t);
+}
+
+// 4D key (bits per axis) of a box centre in the scene cube [-R, R]^3
+// x [0, T], along the Hilbert curve; optionally log-compressed in space (a
+// monotone map, so any key order is a valid tree order).  time_scale weighs
+// time against space: below 1 the horizon takes that share of the time
+// axis's cells, above 1 the scene cube takes 1 / time_scale of the space
+// axes' cells (around the centre), so time counts that many times more in
+// the curve's order.  R is the cube's half-side, T1 the horizon plus one
+// tick; all in FP32.
+__device__ inline unsigned long long box_curve(float4 L, float4 H, float R, float T1, int bits,
+                                               float time_scale, int space_warp) {
   const float sw = time_scale > 1.0f ? 1.0f / time_scale : 1.0f;
   const float tw = time_scale > 1.0f ? 1.0f : time_scale;
   float ux, uy, uz;
@@ -232,13 +229,13 @@ __device__ inline unsigned long long box_morton(float4 L, float4 H, float R, flo
     uz = (0.5f * (L.z + H.z)) * inv + 0.5f;
   }
   float ut = (0.5f * (L.w + H.w)) / T1 * tw;  // ticks below 2^24: the sum is exact
-  return morton4(quantize(ux, bits), quantize(uy, bits), quantize(uz, bits), quantize(ut, bits),
-                 bits);
+  return hilbert4(quantize(ux, bits), quantize(uy, bits), quantize(uz, bits), quantize(ut, bits),
+                  bits);
 }
 
 // The size group of a box (tuning split_km): boxes whose largest spatial
 // side exceeds |split_km| km form one group and the others another; the
-// group bit goes above the Morton key, so each group is sorted apart and
+// group bit goes above the curve key, so each group is sorted apart and
 // gets its own subtree.  1 = the group sorted last: the large boxes when
 // split_km > 0, the small ones when split_km < 0.
 __device__ __forceinline__ uint32_t split_bit(float4 L, float4 H, float split_km) {
@@ -246,20 +243,18 @@ __device__ __forceinline__ uint32_t split_bit(float4 L, float4 H, float split_km
   const float ext = fmaxf(fmaxf(H.x - L.x, H.y - L.y), H.z - L.z);
   return (split_km > 0.0f) == (ext > fabsf(split_km)) ? 1u : 0u;
 }
-// the split applies to Morton keys with room above them: 10 or 12 bits per axis
+// the split applies to keys with room above them: 10 or 12 bits per axis
 inline float split_of(const scd_tuning &t) {
   return t.morton_bits == 10 || t.morton_bits == 12 ? t.split_km : 0.0f;
 }
-// The sort key of a box: its Morton key with the size group's bit above it.
-// With 12-bit axes the group bit takes the place of the key's lowest bit
-// (the finest time bit), so that the key stays 48 bits (6 sort passes, not
-// 7; measured: node tests +0.25%, the screen 0.15 ms shorter); with 10-bit
-// axes that bit is worth more than the pass (traversal +12%).
-__host__ __device__ inline unsigned long long sort_key(unsigned long long morton, uint32_t group,
+// The sort key of a box: its curve key with the size group's bit above it.
+// With 12-bit axes the group bit takes the place of the curve's lowest bit,
+// so that the key stays 48 bits (6 sort passes, not 7).
+__host__ __device__ inline unsigned long long sort_key(unsigned long long curve, uint32_t group,
                                                        int bits, bool split) {
-  if (!split) return morton;
-  if (bits >= 12) return (morton >> 1) | (unsigned long long)group << (4 * bits - 1);
-  return morton | (unsigned long long)group << (4 * bits);
+  if (!split) return curve;
+  if (bits >= 12) return (curve >> 1) | (unsigned long long)group << (4 * bits - 1);
+  return curve | (unsigned long long)group << (4 * bits);
 }
 inline int sort_key_bits(const scd_tuning &t) {
   const bool split = split_of(t) != 0.0f;
@@ -480,7 +475,6 @@ struct scd_scene {
   scd::DevBuf<uint32_t> d_posof;  // sorted position of each box id
   scd::DevBuf<int2> s_nb;         // sorted positions of the previous / next segment (-1: none)
   scd::DevBuf<uint32_t> s_cell;   // decomposition cell of each sorted reference
-  scd::DevBuf<int32_t> d_first;   // first leaf under each internal node
 
   // static decomposition: references (cell, box) and per-cell subtrees
   int64_t n_refs = 0;
@@ -492,7 +486,7 @@ struct scd_scene {
   scd::DevBuf<double2> d_rr;       // padded radial range of each object
   scd::DevBuf<double> d_edges;     // altitude band edges (p - 1)
   scd::DevBuf<unsigned long long> d_abits;  // semi-major axes as sortable bits
-  scd::DevBuf<int32_t> d_cellroot; // root node of each cell (-1: fewer than 2 refs)
+  scd::DevBuf<int32_t> d_cellend;  // one past the last reference of each cell
 
   // learned steps: features, network outputs, steps [s]
   scd::DevBuf<float> d_feat, d_ny, d_learned;
@@ -523,18 +517,8 @@ struct scd_scene {
   cudaEvent_t cev[scd::kStreamBuckets] = {};
   scd::DevBuf<unsigned long long> d_part, d_parte;  // the records split by their top digit
   int64_t graph_key[8] = {};
-  int64_t graph_M = 0;
-  scd::DevBuf<uint32_t> s_leafkey32;
-  scd::DevBuf<unsigned long long> s_leafkey64;
-  scd::DevBuf<scd::TravNode> d_nodes;
-  scd::DevBuf<scd::QBox> d_qbox;     // 2 per internal node (one box per leaf)
-  scd::DevBuf<scd::W4Node> d_w4;     // four-wide nodes (node width 4)
-  scd::DevBuf<uint32_t> d_qlink;     // per internal node: gamma | leaf flags
-  scd::DevBuf<float4> d_nlo, d_nhi;     // internal node boxes (refit)
-  scd::DevBuf<float4> d_leaflo, d_leafhi;
-  scd::DevBuf<int32_t> d_parent_int, d_parent_leaf;
-  scd::DevBuf<uint32_t> d_flags;
-  scd::DevBuf<int32_t> d_first_last;   // per internal node: first, last
+  scd::DevBuf<scd::WideNode> d_nodes;  // every level of the tree
+  scd::DevBuf<scd::SBox> d_nbox;       // boxes of the levels between build launches
 
   // pair emission and canonical list
   int64_t pair_cap = 0;
@@ -550,10 +534,9 @@ struct scd_scene {
   scd::DevBuf<unsigned char> d_npobj;  // per-object FP32 constants (64 B each)
   unsigned long long last_np_evals = 0, last_np_evals64 = 0;
 
-  // refinement: the capacities (intervals a round, candidates) and the
-  // traversal stack that sufficed last time
+  // refinement: the capacities (intervals a round, candidates) that sufficed
+  // last time
   int64_t rf_cap = 0, rf_ccap = 0;
-  int rf_deep = 0;
 
   // metrics of the last find_pairs
   double ms_sort = 0, ms_build = 0, ms_traverse = 0, ms_canon = 0, ms_boxes = 0;
@@ -569,27 +552,28 @@ int launch_prepare_objects(scd_scene *s);
 int launch_build_boxes(scd_scene *s);
 int launch_propagate(const scd_element *d_el, int64_t n, const uint32_t *obj, const double *t,
                      int64_t m, double *out, cudaStream_t st);
-int build_hierarchy(scd_scene *s, int64_t &n_leaves);
-int build_round_tree(const unsigned long long *keys, const SBox *sbox, int64_t cap,
-                     const unsigned long long *d_M, TravNode *nodes, int32_t *parent_int,
-                     int32_t *parent_leaf, uint32_t *arrive, QBox *nq, QBox *qbox,
-                     uint32_t *qlink, const DevCounters *ctr, int64_t T, cudaStream_t st);
-template <class K>
-int build_tree(scd_scene *s, const K *keys_sorted, const uint32_t *ids_sorted, int64_t Nq,
-               K *leafkey, int cell_shift, int64_t &M);
-// decomposed screen: references, their sort, the tree and each cell's root
-int build_decomposed(scd_scene *s, const scd_decomp *d, int64_t &n_leaves,
-                     bool capturing = false);
+// sorted boxes gathered by id, the tree over them, the neighbour positions
+int build_hierarchy(scd_scene *s);
+int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32_t *ids_sorted,
+               int64_t Nq, int cell_shift);
+// the same for one refinement round (up to cap boxes, their count on the device)
+int build_round_tree(const uint32_t *ids_sorted, const float4 *lo, const float4 *hi,
+                     const uint32_t *obj, int64_t cap, const unsigned long long *d_M, SBox *sbox,
+                     uint32_t *sobj, WideNode *nodes, SBox *nbox, cudaStream_t st);
+// node boxes between the tree build's launches, for up to cap boxes
+int64_t tree_scratch_boxes(int64_t cap);
+// decomposed screen: references, their sort, the tree and each cell's end
+int build_decomposed(scd_scene *s, const scd_decomp *d, bool capturing = false);
 // learned per-object steps [s] into s->d_learned (SCD_STEP_LEARNED)
 int learned_steps(scd_scene *s);
 // internal decomposition kind of a batch of scenes: one cell per scene
 constexpr int kDecompScenes = 100;
-int traverse(scd_scene *s, int64_t n_leaves, int raw_mode, int obj_bits, int t_bits);
-int traverse_round(const QBox *qbox, const uint32_t *qlink, const SBox *sbox,
-                   const uint32_t *sobj, const uint32_t *sid, int64_t cap,
-                   const unsigned long long *d_N, int64_t T, DevCounters *ctr, uint32_t *rflags,
-                   unsigned long long *rcand, unsigned long long *rncand, unsigned long long rcap,
-                   int spans, int deep, cudaStream_t st);
+int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits);
+int traverse_round(const WideNode *nodes, const SBox *sbox, const uint32_t *sobj,
+                   const uint32_t *sid, int64_t cap, const unsigned long long *d_N, int64_t T,
+                   DevCounters *ctr, uint32_t *rflags, unsigned long long *rcand,
+                   unsigned long long *rncand, unsigned long long rcap, int spans,
+                   cudaStream_t st);
 int canonicalize(scd_scene *s, int raw_mode, int obj_bits, int t_bits);
 // canonical list with every count read on the device (graph capture)
 int canonicalize_dev(scd_scene *s, int obj_bits, int t_bits);

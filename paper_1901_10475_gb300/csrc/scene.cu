@@ -75,7 +75,7 @@ extern "C" SCD_API int scd_default_tuning(scd_tuning *t) {
   t->stack_depth = 64;
   t->block_threads = 128;
   t->morton_bits = 12;
-  t->time_scale = 8.0f;  // time weighed 8x against space in the Morton curve
+  t->time_scale = 8.0f;  // time weighed 8x against space in the key's curve
   t->use_graph = 0;
   t->space_warp = 0;
   t->nodes_per_step = 2;
@@ -333,27 +333,17 @@ static int find_pairs_impl(scd_scene *s, const scd_decomp *d, int raw_mode) {
     }
     if (raw_mode) return SCD_ERR_INVALID_ARG;
   }
-  cudaStream_t st = s->stream;
   int ob = bits_for(s->n - 1), tb = bits_for(s->T);
   if (2 * ob + tb > 64) return SCD_ERR_INVALID_ARG;
-  int64_t N = s->N;
   s->dkind = dkind;
   s->n_slabs = dkind == SCD_DECOMP_SLAB_OCT ? d->n_slabs : 0;
   s->p_bands = dkind == SCD_DECOMP_ALT_BANDS ? d->p_bands : 0;
-  // the decomposed traversal runs on one-box leaves
-  const int leaf_saved = s->tune.leaf_size;
-  if (dkind != SCD_DECOMP_NONE) s->tune.leaf_size = 1;
-  struct Restore {
-    scd_scene *s;
-    int leaf;
-    ~Restore() { s->tune.leaf_size = leaf; }
-  } restore{s, leaf_saved};
   if (s->tune.use_graph && !raw_mode) return find_graph(s, d, dkind, ob, tb);
   return find_eager(s, d, dkind, raw_mode, ob, tb);
 }
 
 // The find sequence run op by op, with host reads of the counters between
-// phases (buffer growth, stack depth, checks).
+// phases (buffer growth, checks).
 // Records per box seen so far, per kind of screen (SPEED runs, INTERVAL
 // runs, raw cells), starting from catalog-shaped measurements (9.4, 1.5, 22)
 // and raised by every large screen (2^20 boxes or more, where a second
@@ -382,9 +372,8 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
   cudaStream_t st = s->stream;
   int64_t N = s->N;
   if (s->events_ready) cudaEventRecord(s->ev[2], st);
-  int64_t M = 0;
   if (dkind == SCD_DECOMP_NONE) {
-    // A5: sort box ids along the Morton curve
+    // A5: sort box ids along the Hilbert curve
     int kb = sort_key_bits(s->tune);
     if (s->tune.morton_bits > 8) {
       TRY(radix_sort_u64(s->d_key64.p, s->d_id.p, N, kb, s->sort_sc, st));
@@ -393,11 +382,11 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
     }
     if (s->events_ready) cudaEventRecord(s->ev[3], st);
     // A6-A7: hierarchy and refit
-    TRY(build_hierarchy(s, M));
+    TRY(build_hierarchy(s));
   } else {
     // A10: references per cell, their sort, the hierarchy and cell roots
     if (s->events_ready) cudaEventRecord(s->ev[3], st);
-    TRY(build_decomposed(s, d, M));
+    TRY(build_decomposed(s, d));
     N = s->n_refs;
   }
   if (s->events_ready) cudaEventRecord(s->ev[4], st);
@@ -416,14 +405,8 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
     // zero the emission counters, keep the box-build flags
     if (cudaMemsetAsync(s->d_ctr.p, 0, offsetof(DevCounters, extent_bits), st) != cudaSuccess)
       return SCD_ERR_CUDA;
-    TRY(traverse(s, M, raw_mode, ob, tb));
+    TRY(traverse(s, raw_mode, ob, tb));
     TRY(read_counters(s));
-    if (s->h_ctr.trav_flags & ERR_STACK) {
-      // a deeper stack, then the same traversal again
-      if (s->tune.stack_depth >= 128) return SCD_ERR_INTERNAL;
-      s->tune.stack_depth *= 2;
-      continue;
-    }
     unsigned long long need = raw_mode ? s->h_ctr.n_raw
                                        : std::max(s->h_ctr.n_starts, s->h_ctr.n_ends);
     // the record sort indexes with 32-bit counts
@@ -452,7 +435,6 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
   cudaMemcpy(&flags[1], &s->d_ctr.p->sort_flags, sizeof(unsigned int), cudaMemcpyDeviceToHost);
   if (flags[1] & ERR_SORT) return SCD_ERR_TIMEOUT;
   if (flags[0] & ERR_ZIP) return SCD_ERR_INTERNAL;
-  s->graph_M = M;
   finish_metrics(s, raw_mode);
   return SCD_OK;
 }
@@ -462,7 +444,6 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
 // capture into one CUDA graph.
 static int enqueue_find(scd_scene *s, const scd_decomp *d, int dkind, int ob, int tb) {
   cudaStream_t st = s->stream;
-  int64_t M = 0;
   if (s->events_ready) cudaEventRecord(s->ev[2], st);
   if (dkind == SCD_DECOMP_NONE) {
     int kb = sort_key_bits(s->tune);
@@ -472,16 +453,15 @@ static int enqueue_find(scd_scene *s, const scd_decomp *d, int dkind, int ob, in
       TRY(radix_sort_u32(s->d_key32.p, s->d_id.p, s->N, kb, s->sort_sc, st));
     }
     if (s->events_ready) cudaEventRecord(s->ev[3], st);
-    TRY(build_hierarchy(s, M));
+    TRY(build_hierarchy(s));
   } else {
     if (s->events_ready) cudaEventRecord(s->ev[3], st);
-    TRY(build_decomposed(s, d, M, true));
+    TRY(build_decomposed(s, d, true));
   }
-  if (M != s->graph_M) return SCD_ERR_STATE;
   if (s->events_ready) cudaEventRecord(s->ev[4], st);
   if (cudaMemsetAsync(s->d_ctr.p, 0, offsetof(DevCounters, extent_bits), st) != cudaSuccess)
     return SCD_ERR_CUDA;
-  TRY(traverse(s, M, 0, ob, tb));
+  TRY(traverse(s, 0, ob, tb));
   if (s->events_ready) cudaEventRecord(s->ev[5], st);
   TRY(canonicalize_dev(s, ob, tb));
   if (s->events_ready) cudaEventRecord(s->ev[6], st);
@@ -493,8 +473,7 @@ static void graph_key_of(const scd_scene *s, int64_t key[8]) {
   key[1] = s->n_slabs * 100000 + s->p_bands;
   key[2] = s->N;
   key[3] = s->pair_cap;
-  key[4] = (s->tune.node_width * 10 + s->tune.nodes_per_step) * 100000 +
-           s->tune.leaf_size * 1000 + s->tune.stack_depth;
+  key[4] = 0;
   key[5] = s->tune.morton_bits * 10 + s->tune.space_warp;
   key[6] = (int64_t)(s->tune.time_scale * 1e6f) * 1000000 + (int64_t)(split_of(s->tune) * 10.0f);
   key[7] = s->dkind ? s->n_refs : 0;
@@ -526,7 +505,7 @@ static int find_graph(scd_scene *s, const scd_decomp *d, int dkind, int ob, int 
     if (c.build_flags & ERR_INVALID) return SCD_ERR_INVALID_ARG;
     if (c.build_flags & ERR_KEPLER) return SCD_ERR_KEPLER_NOCONV;
     if (c.sort_flags & ERR_SORT) return SCD_ERR_TIMEOUT;
-    bool fits = !(c.trav_flags & (ERR_STACK | ERR_ZIP)) &&
+    bool fits = !(c.trav_flags & ERR_ZIP) &&
                 std::max(c.n_starts, c.n_ends) <= (unsigned long long)s->pair_cap &&
                 (!dkind || (int64_t)c.refs_total == s->n_refs);
     if (fits) {
@@ -772,22 +751,17 @@ extern "C" SCD_API void scd_scene_destroy(scd_scene *s) {
   s->d_key64.release(st); s->d_key32.release(st); s->d_id.release(st);
   s->s_box.release(st); s->s_obj.release(st);
   s->d_posof.release(st); s->s_nb.release(st);
-  s->s_leafkey32.release(st); s->s_leafkey64.release(st);
-  s->d_nodes.release(st); s->d_nlo.release(st); s->d_nhi.release(st);
-  s->d_qbox.release(st); s->d_qlink.release(st); s->d_w4.release(st);
-  s->d_leaflo.release(st); s->d_leafhi.release(st);
-  s->d_parent_int.release(st); s->d_parent_leaf.release(st); s->d_flags.release(st);
-  s->d_first_last.release(st);
+  s->d_nodes.release(st); s->d_nbox.release(st);
   s->d_starts.release(st); s->d_ends.release(st); s->d_rawval.release(st);
   s->d_tilecnt.release(st);
   s->d_out.release(st);
   s->d_narrow.release(st);
   s->d_npobj.release(st);
   s->sort_sc.release(st);
-  s->s_cell.release(st); s->d_first.release(st);
+  s->s_cell.release(st);
   s->d_refcnt.release(st); s->d_refoff.release(st); s->d_refkey.release(st);
   s->d_refid.release(st); s->d_rr.release(st); s->d_edges.release(st);
-  s->d_abits.release(st); s->d_cellroot.release(st);
+  s->d_abits.release(st); s->d_cellend.release(st);
   s->d_feat.release(st); s->d_ny.release(st); s->d_learned.release(st);
   s->d_objT.release(st); s->d_objscene.release(st); s->d_sceneoff.release(st);
   s->d_pairoff.release(st);

@@ -2,8 +2,8 @@
 // meets (the tree query of Sec. 3.2, run for all boxes at once) and the
 // candidate records are emitted; step A9: the canonical list.
 //
-// Each box pair is found once: box p only visits subtrees whose rightmost
-// leaf lies after its own leaf, and inside its own leaf only later boxes.
+// Each box pair is found once: box p only visits nodes that hold a later
+// sorted position, and of those only later boxes.
 //
 // Merged output without sorting the raw set: for one object pair the tick
 // intersections of their overlapping box pairs ("cells") are disjoint and
@@ -26,17 +26,12 @@
 namespace scd {
 
 struct TravArgs {
-  const TravNode *nodes;
-  const QBox *qbox;           // compact nodes (one box per leaf)
-  const uint32_t *qlink;      // their split gamma with the two leaf flags
-  const W4Node *w4;           // four-wide nodes (one box per leaf, node width 4)
+  const WideNode *nodes;      // the tree (all levels, lv.off)
+  TreeLevels lv;
   const SBox *sbox;           // sorted boxes
   const uint32_t *sobj, *sid; // object and unsorted id of each sorted box
   const int2 *nb;             // sorted positions of the previous / next segment
-  const float4 *lo, *hi;      // unsorted boxes (object-major)
   int64_t N;
-  int L;
-  int64_t M;
   int T;
   int raw;
   int obj_bits, t_bits;
@@ -46,11 +41,11 @@ struct TravArgs {
   uint32_t *rawval;           // raw cells' (or unpacked run starts') last tick
   unsigned long long cap;
   DevCounters *ctr;
-  // static decomposition (kind SCD_DECOMP_NONE: one tree, root 0)
+  // static decomposition (kind SCD_DECOMP_NONE: one tree over all boxes)
   int dkind;
   int n_slabs, p_bands;
   const uint32_t *scell;     // cell of each sorted reference
-  const int32_t *cellroot;   // root node of each cell's subtree (-1: none)
+  const int32_t *cellend;    // one past the last reference of each cell
   const double2 *rr;         // radial ranges (ALT_BANDS)
   const double *edges;       // band edges (ALT_BANDS)
   const int32_t *objT;       // per-object horizon (a batch of scenes), or null
@@ -89,32 +84,6 @@ __device__ __forceinline__ bool reports_here(const TravArgs &a, uint32_t cell, f
 // a slot that holds no record: all key bits set, so it sorts after every
 // real record (whose object fields can never be all ones)
 constexpr unsigned long long kHole = ~0ull;
-
-// One record per predicate-true lane, each with its own atomic slot range
-// (used by the one-thread-per-box traversal, whose lanes are not in step).
-struct DirectEmit {
-  __device__ __forceinline__ void put(unsigned long long *buf, uint32_t *vbuf,
-                                      unsigned long long *slots, unsigned long long *valid,
-                                      unsigned long long cap, bool pred, unsigned long long key,
-                                      uint32_t v) {
-    unsigned mask = __activemask();
-    unsigned vote = __ballot_sync(mask, pred);
-    if (!pred) return;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(vote) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) {
-      base = atomicAdd(slots, (unsigned long long)__popc(vote));
-      atomicAdd(valid, (unsigned long long)__popc(vote));
-    }
-    base = __shfl_sync(vote, base, leader);
-    unsigned long long idx = base + (unsigned long long)__popc(vote & ((1u << lane) - 1u));
-    if (idx < cap) {
-      buf[idx] = key;
-      if (vbuf) vbuf[idx] = v;
-    }
-  }
-};
 
 // Whole-warp emission into a chunk of slots reserved by the warp (one atomic
 // per kChunk records).  A chunk's unused tail is filled with holes.  Every
@@ -158,33 +127,10 @@ __device__ __forceinline__ void chunk_put(ChunkCursor &c, unsigned long long *bu
   c.count += cnt;
 }
 
-struct Query {
-  float4 lo, hi;
-  uint32_t obj, uid;
-};
-
 // Is (q, b) the first / last cell of its run?  Both need the neighbouring
-// cell: one segment back (forward) on whichever box starts (ends) there.
-__device__ __forceinline__ void run_ends(const TravArgs &a, const Query &q, float4 bl, float4 bh,
-                                         uint32_t bu, int s, int e, int T, bool &start,
-                                         bool &end) {
-  int qt0 = (int)q.lo.w, qt1 = (int)q.hi.w, bt0 = (int)bl.w, bt1 = (int)bh.w;
-  if (start && s > 0) {
-    float4 ql = q.lo, qh = q.hi, cl = bl, ch = bh;
-    if (qt0 == s) { ql = __ldg(a.lo + q.uid - 1); qh = __ldg(a.hi + q.uid - 1); }
-    if (bt0 == s) { cl = __ldg(a.lo + bu - 1); ch = __ldg(a.hi + bu - 1); }
-    start = !box_overlap(ql, qh, cl, ch);
-  }
-  if (end && e < T) {
-    float4 ql = q.lo, qh = q.hi, cl = bl, ch = bh;
-    if (qt1 == e) { ql = __ldg(a.lo + q.uid + 1); qh = __ldg(a.hi + q.uid + 1); }
-    if (bt1 == e) { cl = __ldg(a.lo + bu + 1); ch = __ldg(a.hi + bu + 1); }
-    end = !box_overlap(ql, qh, cl, ch);
-  }
-}
-
-// The same test with the neighbouring segments found by sorted position
-// (they lie close to the pair in the Morton order, so the loads hit cache).
+// cell: one segment back (forward) on whichever box starts (ends) there,
+// found by sorted position (close to the pair along the curve, so the loads
+// hit cache).
 __device__ __forceinline__ void run_ends_sorted(const TravArgs &a, float4 ql0, float4 qh0,
                                                 int2 qn, float4 bl, float4 bh, int2 bn, int s,
                                                 int e, int T, bool &start, bool &end) {
@@ -218,121 +164,33 @@ __device__ __forceinline__ unsigned long long start_key(const TravArgs &a, unsig
 }
 
 // ---------------------------------------------------------------------------
-// One thread per box, for leaves of several boxes.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void on_candidate(const TravArgs &a, const Query &q, int64_t pb,
-                                             unsigned long long &leaf_tests) {
-  float4 bl, bh;
-  ldg_box(a.sbox + pb, bl, bh);
-  ++leaf_tests;
-  if (!box_overlap(q.lo, q.hi, bl, bh)) return;
-  uint32_t bo = __ldg(a.sobj + pb);
-  if (bo == q.obj) return;
-  uint32_t bu = __ldg(a.sid + pb);
-  int s = max((int)q.lo.w, (int)bl.w), e = min((int)q.hi.w, (int)bh.w);
-  unsigned long long pk = pair_key(a, q.obj, bo);
-  DirectEmit em;
-  if (a.raw) {
-    em.put(a.starts, a.rawval, &a.ctr->n_raw, &a.ctr->v_raw, a.cap, true,
-           pk | (unsigned long long)s, (uint32_t)e);
-    return;
-  }
-  bool start = true, end = true;
-  run_ends(a, q, bl, bh, bu, s, e, a.objT ? __ldg(a.objT + q.obj) : a.T, start, end);
-  const uint32_t last = end ? (uint32_t)e : a.open_tag;
-  em.put(a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, &a.ctr->v_starts, a.cap,
-         start, start_key(a, pk, s, last), last);
-  em.put(a.ends, nullptr, &a.ctr->n_ends, &a.ctr->v_ends, a.cap, end && !start,
-         pk | (unsigned long long)e, 0u);
-}
-
-__device__ __forceinline__ void visit_leaf(const TravArgs &a, const Query &q, int64_t leaf,
-                                           unsigned long long &lt) {
-  int64_t b0 = leaf * a.L, b1 = b0 + a.L < a.N ? b0 + a.L : a.N;
-  for (int64_t pb = b0; pb < b1; ++pb) on_candidate(a, q, pb, lt);
-}
-
-template <int kDepth>
-__global__ void __launch_bounds__(256) k_traverse(TravArgs a) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long nt = 0, lt = 0;
-  if (p < a.N) {
-    Query q;
-    ldg_box(a.sbox + p, q.lo, q.hi);
-    q.obj = __ldg(a.sobj + p);
-    q.uid = __ldg(a.sid + p);
-    int64_t c = p / a.L;
-    int64_t e1 = (c + 1) * a.L < a.N ? (c + 1) * a.L : a.N;
-    for (int64_t pb = p + 1; pb < e1; ++pb) on_candidate(a, q, pb, lt);
-    if (a.M > 1) {
-      int32_t stack[kDepth];
-      int sp = 0;
-      int32_t node = 0;
-      for (;;) {
-        const float4 *np = reinterpret_cast<const float4 *>(a.nodes + node);
-        float4 lol = __ldg(np + 0), hil = __ldg(np + 1), lor = __ldg(np + 2), hir = __ldg(np + 3);
-        int4 lk = __ldg(reinterpret_cast<const int4 *>(np + 4));
-        nt += 2;
-        bool gl = lk.z > c && box_overlap(q.lo, q.hi, lol, hil);
-        bool gr = lk.w > c && box_overlap(q.lo, q.hi, lor, hir);
-        if (gl && (lk.x & kLeafBit)) {
-          visit_leaf(a, q, lk.x & ~kLeafBit, lt);
-          gl = false;
-        }
-        if (gr && (lk.y & kLeafBit)) {
-          visit_leaf(a, q, lk.y & ~kLeafBit, lt);
-          gr = false;
-        }
-        if (gl && gr) {
-          if (sp >= kDepth) {
-            atomicOr(&a.ctr->trav_flags, ERR_STACK);
-            break;
-          }
-          stack[sp++] = lk.y;
-          node = lk.x;
-        } else if (gl) {
-          node = lk.x;
-        } else if (gr) {
-          node = lk.y;
-        } else {
-          if (sp == 0) break;
-          node = stack[--sp];
-        }
-      }
-    }
-  }
-  // one atomic per warp for the test counters
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nt += __shfl_down_sync(0xffffffffu, nt, o);
-    lt += __shfl_down_sync(0xffffffffu, lt, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&a.ctr->node_tests, nt);
-    atomicAdd(&a.ctr->leaf_tests, lt);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Persistent traversal for one box per leaf.  Every loop iteration of every
-// lane is the same step (load one compact node, test its two child boxes), so
-// lanes stay in lock step; a lane whose query is done takes the next one from
-// a pool its warp claims in blocks; overlapping box pairs go to a per-warp
-// buffer and their records are worked out by the whole warp together, into
+// Persistent traversal.  Every loop iteration of every lane is the same step
+// (load one node, test its eight children), so lanes stay in lock step; a
+// lane whose query is done takes the next one from a pool its warp claims in
+// blocks; leaf nodes with overlapping boxes go to a per-warp buffer and the
+// records of their pairs are worked out by the whole warp together, into
 // output chunks the warp reserves kChunk slots at a time.
+//
+// The lane's pending nodes are one 32-bit word per level (the parent's index
+// and a mask of its children still to visit): at most ten words in shared
+// memory, whatever the query, so no stack can overflow.
+//
+// Measured on the 24 h catalog screen (17.4 M boxes): 12.0 ms and 40 nodes a
+// query with SPEED boxes, 6.5 ms and 35 with INTERVAL boxes; two-child nodes
+// of 36 bytes along a Morton curve, with 64-entry stacks in local memory,
+// took 18.4 ms and 91, 10.7 ms and 65.  Bound by the L1's load wavefronts
+// (87% of its peak while active: 32 lanes on 32 different nodes take one
+// wavefront for each of the three loads of a node).
 // ---------------------------------------------------------------------------
-// block shape: 64, 128 and 256 threads (with 16, 8 and 4 resident blocks)
-// measured the same on the 24 h catalog screen (21.9, 21.9, 22.0 ms)
-constexpr int kT2Threads = 128;
-constexpr int kT2Warps = kT2Threads / 32;
-// candidate pairs buffered per warp, drained when fewer than one step's
-// worth (128) of slots remain: fewer, longer drains.  Measured on the 24 h
-// catalog screen: 256 18.70 ms, 384 18.39, 448 18.32, 512 18.56 (a larger
-// shared-memory carve-out takes L1), 768 34.9 (fewer resident blocks)
-constexpr int kHitCap = 448;
+constexpr int kTvThreads = 128;
+constexpr int kTvWarps = kTvThreads / 32;
+// leaf nodes (query, node, mask of its boxes) buffered per warp, drained when
+// fewer than one step's worth (32) of slots remain
+constexpr int kEntryCap = 160;
+// entries expanded into single pairs at a time, two per lane
+constexpr int kExpand = 64;
 // queries claimed per warp atomic; small, so that the queries in flight stay
-// a narrow window of the Morton order and their nodes stay in L2
-// (64 per claim: +4% traversal time, 128: +17%)
+// a narrow window of the curve and their nodes stay in L2
 constexpr unsigned kQueryChunk = 32;
 // a refill can hand out up to 32 queries at once, from the pool's rest and
 // one new chunk: a chunk smaller than a warp would leave lanes without one
@@ -342,130 +200,159 @@ struct WarpEmit {
   ChunkCursor s, e;  // start and end record chunks (raw cells use s)
 };
 
-// A refinement round's hits: both intervals of a pair of meeting boxes of
-// different objects are flagged; two single ticks that meet (the same tick)
-// are a tick candidate, and at the finest level of the continuous variant
-// every meeting pair is a span.
-__device__ __forceinline__ void drain_round_hits(const TravArgs &a, const uint2 *buf, int cnt) {
-  const int lane = threadIdx.x & 31;
-  for (int k = lane; k < cnt; k += 32) {
-    const uint2 h = buf[k];
-    float4 ql, qh, bl, bh;
-    ldg_box(a.sbox + h.x, ql, qh);
-    ldg_box(a.sbox + h.y, bl, bh);
-    const uint32_t qo = __ldg(a.sobj + h.x), bo = __ldg(a.sobj + h.y);
-    if (bo == qo || !box_overlap(ql, qh, bl, bh)) continue;
-    const bool longq = qh.w > ql.w, longb = bh.w > bl.w;
-    atomicOr(a.rflags + __ldg(a.sid + h.x), kRfHit | (longb ? kRfHitLong : 0u));
-    atomicOr(a.rflags + __ldg(a.sid + h.y), kRfHit | (longq ? kRfHitLong : 0u));
-    unsigned long long key;
-    if (a.rspans) {
-      key = rf_span_key(min(qo, bo), max(qo, bo), (int32_t)ql.w, (int32_t)bl.w);
-    } else if (!longq && !longb) {
-      key = rf_tick_key((uint32_t)ql.w, min(qo, bo), max(qo, bo));
-    } else {
-      continue;
-    }
-    const unsigned long long q = atomicAdd(a.rncand, 1ull);
-    if (q < a.rcap) a.rcand[q] = key;
+// A pair whose boxes meet in a node's frame, decided on the exact boxes.
+// Refinement rounds: both intervals of a pair of meeting boxes of different
+// objects are flagged; two single ticks that meet (the same tick) are a tick
+// candidate, and at the finest level of the continuous variant every meeting
+// pair is a span.
+__device__ __forceinline__ void round_pair(const TravArgs &a, uint32_t p, uint32_t b) {
+  float4 ql, qh, bl, bh;
+  ldg_box(a.sbox + p, ql, qh);
+  ldg_box(a.sbox + b, bl, bh);
+  const uint32_t qo = __ldg(a.sobj + p), bo = __ldg(a.sobj + b);
+  if (bo == qo || !box_overlap(ql, qh, bl, bh)) return;
+  const bool longq = qh.w > ql.w, longb = bh.w > bl.w;
+  atomicOr(a.rflags + __ldg(a.sid + p), kRfHit | (longb ? kRfHitLong : 0u));
+  atomicOr(a.rflags + __ldg(a.sid + b), kRfHit | (longq ? kRfHitLong : 0u));
+  unsigned long long key;
+  if (a.rspans) {
+    key = rf_span_key(min(qo, bo), max(qo, bo), (int32_t)ql.w, (int32_t)bl.w);
+  } else if (!longq && !longb) {
+    key = rf_tick_key((uint32_t)ql.w, min(qo, bo), max(qo, bo));
+  } else {
+    return;
   }
+  const unsigned long long q = atomicAdd(a.rncand, 1ull);
+  if (q < a.rcap) a.rcand[q] = key;
 }
 
-__device__ __forceinline__ void drain_hits(const TravArgs &a, const uint2 *buf, int cnt,
-                                           WarpEmit &we) {
-  const int lane = threadIdx.x & 31;
-  for (int base = 0; base < cnt; base += 32) {
-    int k = base + lane;
-    bool valid = k < cnt;
-    float4 ql = make_float4(0.f, 0.f, 0.f, 0.f), qh = ql, bl = ql, bh = ql;
-    uint32_t qo = 0, bo = 0;
-    uint2 h = make_uint2(0u, 0u);
-    if (valid) {
-      h = buf[k];
-      ldg_box(a.sbox + h.x, ql, qh);
-      qo = __ldg(a.sobj + h.x);
-      ldg_box(a.sbox + h.y, bl, bh);
-      bo = __ldg(a.sobj + h.y);
-      // the tree test was on quantised boxes: decide on the exact ones
-      valid = bo != qo && box_overlap(ql, qh, bl, bh);
-      if (valid && a.dkind != SCD_DECOMP_NONE)
-        valid = reports_here(a, __ldg(a.scell + h.x), ql, bl, qo, bo);
-    }
-    int s = max((int)ql.w, (int)bl.w), e = min((int)qh.w, (int)bh.w);
-    unsigned long long pk = pair_key(a, qo, bo);
-    if (a.raw) {
-      chunk_put(we.s, a.starts, a.rawval, &a.ctr->n_raw, a.cap, valid,
-                pk | (unsigned long long)s, (uint32_t)e);
-      continue;
-    }
-    bool start = valid, end = valid;
-    if (valid)
-      run_ends_sorted(a, ql, qh, __ldg(a.nb + h.x), bl, bh, __ldg(a.nb + h.y), s, e,
-                      a.objT ? __ldg(a.objT + qo) : a.T, start, end);
-    const uint32_t last = end ? (uint32_t)e : a.open_tag;
-    chunk_put(we.s, a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, a.cap, start,
-              start_key(a, pk, s, last), last);
-    chunk_put(we.e, a.ends, nullptr, &a.ctr->n_ends, a.cap, end && !start,
-              pk | (unsigned long long)e, 0u);
+// The screen's pairs, one per lane (valid: the lane has one); called by the
+// whole warp.
+__device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint32_t p, uint32_t b,
+                                            WarpEmit &we) {
+  float4 ql = make_float4(0.f, 0.f, 0.f, 0.f), qh = ql, bl = ql, bh = ql;
+  uint32_t qo = 0, bo = 0;
+  if (valid) {
+    ldg_box(a.sbox + p, ql, qh);
+    qo = __ldg(a.sobj + p);
+    ldg_box(a.sbox + b, bl, bh);
+    bo = __ldg(a.sobj + b);
+    valid = bo != qo && box_overlap(ql, qh, bl, bh);
+    if (valid && a.dkind != SCD_DECOMP_NONE)
+      valid = reports_here(a, __ldg(a.scell + p), ql, bl, qo, bo);
   }
+  int s = max((int)ql.w, (int)bl.w), e = min((int)qh.w, (int)bh.w);
+  unsigned long long pk = pair_key(a, qo, bo);
+  if (a.raw) {
+    chunk_put(we.s, a.starts, a.rawval, &a.ctr->n_raw, a.cap, valid, pk | (unsigned long long)s,
+              (uint32_t)e);
+    return;
+  }
+  bool start = valid, end = valid;
+  if (valid)
+    run_ends_sorted(a, ql, qh, __ldg(a.nb + p), bl, bh, __ldg(a.nb + b), s, e,
+                    a.objT ? __ldg(a.objT + qo) : a.T, start, end);
+  const uint32_t last = end ? (uint32_t)e : a.open_tag;
+  chunk_put(we.s, a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, a.cap, start,
+            start_key(a, pk, s, last), last);
+  chunk_put(we.e, a.ends, nullptr, &a.ctr->n_ends, a.cap, end && !start,
+            pk | (unsigned long long)e, 0u);
 }
 
-// One node's two children against the quantised query: the child nodes to
-// descend into (gl, gr) and the leaf children that are candidates (hl, hr).
-// Only subtrees with a leaf after the query's own leaf p are of interest.
-// The left child's rightmost leaf is the split gamma, so it needs the test
-// gamma > p.  The right child needs none: every node a query visits either
-// holds p or lies wholly after it (the root holds p; a child of a node that
-// holds p either holds p or, being right of the split, lies after it, or
-// being left of it, is kept only when gamma > p; children of a node wholly
-// after p are wholly after p), so the right child always ends after p
-// unless it holds p as its last leaf.  That one case costs a descent along
-// the subtree's right edge down to p itself, whose pair with itself the
-// exact test drops (same object).
-__device__ __forceinline__ void test_children(const TravArgs &a, const QBox &q, int64_t p,
-                                              int32_t node, bool &gl, bool &gr, bool &hl,
-                                              bool &hr, int32_t &cl) {
-  uint4 bl, br;
-  ldg_qbox_pair(a.qbox + 2 * (int64_t)node, bl, br);
-  const uint32_t lk = __ldg(a.qlink + node);
-  const uint32_t g = lk & kQIndex;
-  cl = (int32_t)g;
-  // child lo <= query hi and query lo <= child hi: x, y per 16-bit lane,
-  // then the z and tick fields
-  const uint32_t ml = __vcmpleu2(bl.x, q.hi_xy) & __vcmpleu2(q.lo_xy, bl.z);
-  const uint32_t mr = __vcmpleu2(br.x, q.hi_xy) & __vcmpleu2(q.lo_xy, br.z);
-  gl = (int64_t)g > p && ml == 0xffffffffu && zt_le(bl.y, q.hi_zt) && zt_le(q.lo_zt, bl.w);
-  gr = mr == 0xffffffffu && zt_le(br.y, q.hi_zt) && zt_le(q.lo_zt, br.w);
-  hl = gl && (lk & kQLeftLeaf);
-  hr = gr && (lk & kQRightLeaf);
-  gl &= !hl;
-  gr &= !hr;
+// a warp's buffered leaf nodes and the pairs they are expanded into
+struct HitBuf {
+  uint32_t p[kEntryCap], n[kEntryCap];  // query, leaf node
+  uint8_t mask[kEntryCap];              // its boxes that meet the query
+  uint16_t pair[kExpand * kWide];       // entry | box << 8
+};
+static_assert(kEntryCap <= 256, "an expanded pair names its entry in eight bits");
+
+// The buffered leaf nodes' pairs, spread evenly over the lanes: the entries'
+// boxes are counted and listed kExpand entries at a time, then 32 listed
+// pairs at a time are decided.  Returns the pairs.
+template <bool kRefine>
+__device__ __forceinline__ int drain(const TravArgs &a, HitBuf &h, int cnt, WarpEmit &we) {
+  const int lane = threadIdx.x & 31;
+  int pairs = 0;
+  for (int base = 0; base < cnt; base += kExpand) {
+    const int k0 = base + lane, k1 = k0 + 32;
+    uint32_t m0 = k0 < cnt ? h.mask[k0] : 0u, m1 = k1 < cnt ? h.mask[k1] : 0u;
+    // exclusive position of the lane's pairs
+    const int mine = __popc(m0) + __popc(m1);
+    int at = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, at, d);
+      if (lane >= d) at += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, at, 31);
+    at -= mine;
+    for (; m0; m0 &= m0 - 1u) h.pair[at++] = (uint16_t)(k0 | (__ffs(m0) - 1) << 8);
+    for (; m1; m1 &= m1 - 1u) h.pair[at++] = (uint16_t)(k1 | (__ffs(m1) - 1) << 8);
+    __syncwarp();
+    for (int r = 0; r < total; r += 32) {
+      const bool valid = r + lane < total;
+      uint32_t p = 0, b = 0;
+      if (valid) {
+        const uint32_t code = h.pair[r + lane];
+        p = h.p[code & 255u];
+        b = h.n[code & 255u] * kWide + (code >> 8);
+      }
+      if constexpr (kRefine) {
+        if (valid) round_pair(a, p, b);
+      } else {
+        screen_pair(a, valid, p, b, we);
+      }
+    }
+    pairs += total;
+    __syncwarp();
+  }
+  return pairs;
 }
 
-// one slot of a four-wide node: it meets the quantised query and its
-// rightmost leaf lies after the query's own leaf (empty slots: leaf 0)
-__device__ __forceinline__ bool w4_slot(const QBox &q, int64_t p, const uint4 &b, uint32_t last) {
-  return (int64_t)last > p &&
-         (__vcmpleu2(b.x, q.hi_xy) & __vcmpleu2(q.lo_xy, b.z)) == 0xffffffffu &&
-         zt_le(b.y, q.hi_zt) && zt_le(q.lo_zt, b.w);
+// The children of a node that the query box meets in the node's frame, as a
+// mask: 16 FP32 operations bring the query's faces into the frame, then per
+// axis and four children one byte-wise difference each tests lo <= query hi
+// and query lo <= hi (the guard bit survives where it holds).
+__device__ __forceinline__ uint32_t meet_mask(const WideNode *nd, float4 qlo, float4 qhi) {
+  uint32_t f[8], lo[8], hi[8];
+  ldg_words(nd->scale, f);
+  ldg_words(nd->lo, lo);
+  ldg_words(nd->hi, hi);
+  const float ql[4] = {qlo.x, qlo.y, qlo.z, qlo.w}, qh[4] = {qhi.x, qhi.y, qhi.z, qhi.w};
+  uint32_t r0 = 0x80808080u, r1 = 0x80808080u;
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    const float sc = __uint_as_float(f[d]), of = __uint_as_float(f[4 + d]);
+    const uint32_t l4 = __byte_perm(node_coord(ql[d], sc, of, false), 0u, 0x0000u);
+    const uint32_t h4 = __byte_perm(node_coord(qh[d], sc, of, true), 0u, 0x0000u);
+    r0 &= (h4 - lo[2 * d]) & (hi[2 * d] - l4);
+    r1 &= (h4 - lo[2 * d + 1]) & (hi[2 * d + 1] - l4);
+  }
+  // the guard bits of children 0-3 and 4-7 gathered into the top byte: bit
+  // 8 c and bit 8 c + 4 of x go to 24 + c and 28 + c (no two products of the
+  // multiplication share a bit)
+  const uint32_t x = ((r0 >> 7) & 0x01010101u) | ((r1 >> 3) & 0x10101010u);
+  return (x * 0x01020408u) >> 24;
 }
 
-// kTwo: two binary nodes per lane and step; kW4: four-wide nodes.  The
-// lanes' stacks stay in local memory: a stack in shared memory (entry-major,
-// free of bank conflicts) was measured 1.7x slower, because the shared
-// memory it takes comes out of the L1 cache that the node loads rely on.
-// 8 resident blocks of 128 threads: 64 registers and a few bytes of spills;
-// 9 or 10 blocks (56 or 48 registers) spill 112-280 bytes and measured
-// 12% and 41% slower
-template <int kDepth, bool kTwo, bool kW4, bool kRefine = false>
-__global__ void __launch_bounds__(kT2Threads, 8) k_traverse2(TravArgs a) {
-  __shared__ uint2 hits[kT2Warps][kHitCap];
+template <bool kRefine>
+__global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
+  __shared__ HitBuf hits[kTvWarps];
+  __shared__ uint32_t pend[kMaxLevels][kTvThreads];  // [level - 1]: parent << 8 | children mask
+  __shared__ uint32_t off[kMaxLevels + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  uint2 *buf = hits[w];
-  int nhit = 0;  // warp-uniform
+  HitBuf &buf = hits[w];
+  uint32_t *const mine = &pend[0][threadIdx.x] - kTvThreads;  // level l at mine[l * kTvThreads]
+  if (threadIdx.x <= kMaxLevels) off[threadIdx.x] = a.lv.off[threadIdx.x];
+  __syncthreads();
+  int nent = 0;  // warp-uniform
   unsigned long long nt = 0, ntests = 0;
-  int64_t p = -1;  // current query (sorted position), -1 = none
+  uint32_t p = 0;     // current query (sorted position)
+  uint32_t cend = 0;  // one past the last position it may meet
+  uint32_t lv = 0;    // levels with pending nodes; 0 = no query
+  float4 qlo = make_float4(0.f, 0.f, 0.f, 0.f), qhi = qlo;
   bool exhausted = false;
   // the last box has no later partner: queries are 0 .. N-2
   const int64_t nbox = kRefine && a.d_N && *a.d_N < (unsigned long long)a.N ? (int64_t)*a.d_N
@@ -473,36 +360,33 @@ __global__ void __launch_bounds__(kT2Threads, 8) k_traverse2(TravArgs a) {
   const unsigned long long nq = nbox > 1 ? (unsigned long long)(nbox - 1) : 0ull;
   unsigned long long q_next = 0, q_end = 0;  // the warp's query pool
   WarpEmit we;
-  const QFrame fr = scene_frame(a.ctr, a.T);
-  QBox q = {0u, 0u, 0u, 0u};  // the query box, quantised outward like the nodes
-  int32_t stack[kDepth];
-  int sp = 0, sb = 0;  // the lane's deferred subtrees are stack[sb .. sp)
-  int32_t node = 0;
-  int32_t node2 = -1;  // a second node visited in the same step (kTwo)
   for (;;) {
     // lanes without a query take the next ones from the warp's pool
-    unsigned need = __ballot_sync(0xffffffffu, p < 0 && !exhausted);
+    const unsigned need = __ballot_sync(0xffffffffu, lv == 0u && !exhausted);
     if (need) {
-      unsigned cnt = __popc(need);
-      unsigned long long have = q_end - q_next;
+      const unsigned cnt = __popc(need);
+      const unsigned long long have = q_end - q_next;
       unsigned long long nb = 0;
       if (have < cnt) {
         if (lane == 0) nb = atomicAdd(&a.ctr->work_next, (unsigned long long)kQueryChunk);
         nb = __shfl_sync(0xffffffffu, nb, 0);
       }
       if (need & (1u << lane)) {
-        unsigned r = __popc(need & lt);
-        unsigned long long mine = r < have ? q_next + r : nb + (r - have);
-        if (mine < nq) {
-          p = (int64_t)mine;
-          float4 plo, phi;
-          ldg_box(a.sbox + p, plo, phi);
-          q = quantize_box(fr, plo, phi);
-          // the query starts at the root of its own cell's subtree
-          node = a.dkind == SCD_DECOMP_NONE ? 0 : __ldg(a.cellroot + __ldg(a.scell + p));
-          node2 = -1;
-          sp = sb = 0;
-          if (node < 0) p = -1;  // alone in its cell: nothing to find
+        const unsigned r = __popc(need & lt);
+        const unsigned long long q = r < have ? q_next + r : nb + (r - have);
+        if (q < nq) {
+          p = (uint32_t)q;
+          ldg_box(a.sbox + p, qlo, qhi);
+          cend = (uint32_t)nbox;
+          if (!kRefine && a.dkind != SCD_DECOMP_NONE)
+            cend = (uint32_t)__ldg(a.cellend + __ldg(a.scell + p));
+          if (p + 1u < cend) {
+            // start at the smallest node that holds p and the last position
+            const int h = (kWideBits + 31 - __clz((int)(p ^ (cend - 1u)))) / kWideBits;
+            const uint32_t top = p >> (kWideBits * h);
+            mine[h * kTvThreads] = (top >> kWideBits) << 8 | 1u << (top & 7u);
+            lv = 1u << h;
+          }
         } else {
           exhausted = true;
         }
@@ -514,17 +398,23 @@ __global__ void __launch_bounds__(kT2Threads, 8) k_traverse2(TravArgs a) {
         q_next += cnt;
       }
     }
-    // Once the queue is empty, a lane without a query takes the oldest
-    // deferred subtree (the largest) of a lane that has one, with its query:
-    // one long query then spreads over the warp instead of holding it.
+    // Once the queue is empty, a lane without a query takes pending nodes of
+    // a lane that has some to spare, with its query: the whole word of its
+    // highest level, or the last child of its only one; one long query then
+    // spreads over the warp instead of holding it.
     if (__ballot_sync(0xffffffffu, exhausted)) {
-      const unsigned idle = __ballot_sync(0xffffffffu, p < 0);
-      const unsigned donors = __ballot_sync(0xffffffffu, p >= 0 && sp > sb);
+      const int hl = lv ? 31 - __clz((int)lv) : 0;
+      const uint32_t word = lv ? mine[hl * kTvThreads] : 0u;
+      const bool more = (lv & (lv - 1u)) != 0u;  // a lower level has some too
+      const unsigned idle = __ballot_sync(0xffffffffu, lv == 0u);
+      const unsigned donors =
+          __ballot_sync(0xffffffffu, more || __popc(word & 0xffu) > 1);
       const int moves = min(__popc(idle), __popc(donors));
       if (moves > 0) {
         const bool is_idle = (idle >> lane) & 1u, is_donor = (donors >> lane) & 1u;
         const int ri = __popc(idle & lt), rd = __popc(donors & lt);
-        const int32_t give = is_donor ? stack[sb] : 0;
+        const uint32_t top = 0x80u >> (__clz((int)(word & 0xffu)) - 24);  // last child's bit
+        const uint32_t give = more ? word : (word & ~0xffu) | top;
         // the receiver of rank k takes from the donor of rank k
         int src = lane;
         if (is_idle && ri < moves) {
@@ -532,129 +422,85 @@ __global__ void __launch_bounds__(kT2Threads, 8) k_traverse2(TravArgs a) {
           for (int k = 0; k < ri; ++k) m &= m - 1u;
           src = __ffs(m) - 1;
         }
-        const int32_t gnode = __shfl_sync(0xffffffffu, give, src);
-        const uint32_t gp = __shfl_sync(0xffffffffu, (uint32_t)p, src);
-        QBox gq;
-        gq.lo_xy = __shfl_sync(0xffffffffu, q.lo_xy, src);
-        gq.lo_zt = __shfl_sync(0xffffffffu, q.lo_zt, src);
-        gq.hi_xy = __shfl_sync(0xffffffffu, q.hi_xy, src);
-        gq.hi_zt = __shfl_sync(0xffffffffu, q.hi_zt, src);
+        const uint32_t gword = __shfl_sync(0xffffffffu, give, src);
+        const int glevel = __shfl_sync(0xffffffffu, hl, src);
+        const uint32_t gp = __shfl_sync(0xffffffffu, p, src);
+        const uint32_t gend = __shfl_sync(0xffffffffu, cend, src);
+        float4 glo, ghi;
+        glo.x = __shfl_sync(0xffffffffu, qlo.x, src);
+        glo.y = __shfl_sync(0xffffffffu, qlo.y, src);
+        glo.z = __shfl_sync(0xffffffffu, qlo.z, src);
+        glo.w = __shfl_sync(0xffffffffu, qlo.w, src);
+        ghi.x = __shfl_sync(0xffffffffu, qhi.x, src);
+        ghi.y = __shfl_sync(0xffffffffu, qhi.y, src);
+        ghi.z = __shfl_sync(0xffffffffu, qhi.z, src);
+        ghi.w = __shfl_sync(0xffffffffu, qhi.w, src);
+        if (is_donor && rd < moves) {
+          if (more) lv ^= 1u << hl;
+          else mine[hl * kTvThreads] = word ^ top;
+        }
         if (is_idle && ri < moves) {
-          p = (int64_t)gp;
-          q = gq;
-          node = gnode;
-          node2 = -1;
-          sp = sb = 0;
+          p = gp;
+          cend = gend;
+          qlo = glo;
+          qhi = ghi;
+          mine[glevel * kTvThreads] = gword;
+          lv = 1u << glevel;
         }
-        if (is_donor && rd < moves) ++sb;
       }
     }
-    bool active = p >= 0;
-    if (__ballot_sync(0xffffffffu, active) == 0) break;
-    const uint32_t pq = (uint32_t)p;  // this step's query, before p may end
-    bool hl = false, hr = false, hl2 = false, hr2 = false;
-    int32_t cl = 0, cl2 = 0;
-    // the subtrees to visit next: the first one (two) are this lane's next
-    // node(s), the rest go on the stack
-    int32_t first = -1, second = -1;
-    bool overflow = false;
-    auto take = [&](bool go, int32_t c) {
-      if (!go) return;
-      if (first < 0) {
-        first = c;
-      } else if (kTwo && second < 0) {
-        second = c;
-      } else if (sp < kDepth) {
-        stack[sp++] = c;
-      } else {
-        overflow = true;
-      }
-    };
-    // four-wide: the leaf slots that pass, with their leaf indices
-    bool h4[4] = {false, false, false, false};
-    uint32_t c4[4] = {0u, 0u, 0u, 0u};
+    const bool active = lv != 0u;
+    if (__ballot_sync(0xffffffffu, active) == 0u) {
+      if (__ballot_sync(0xffffffffu, exhausted) == 0xffffffffu) break;
+      continue;  // every query taken was alone in its cell
+    }
+    uint32_t mask = 0, node = 0;
+    bool leaf = false;
     if (active) {
-      if constexpr (kW4) {
-        const W4Node *nd = a.w4 + node;
-        uint4 b0, b1, b2, b3, la, lb;
-        ldg_qbox_pair(nd->box, b0, b1);
-        ldg_qbox_pair(nd->box + 2, b2, b3);
-        ldg_w4_links(nd->link, la, lb);
-        nt += 4;
-        const uint32_t lx[4] = {la.x, la.z, lb.x, lb.z};
-        const bool ok[4] = {w4_slot(q, p, b0, la.y), w4_slot(q, p, b1, la.w),
-                            w4_slot(q, p, b2, lb.y), w4_slot(q, p, b3, lb.w)};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const bool leaf = (lx[k] & kW4Leaf) != 0u;
-          h4[k] = ok[k] && leaf;
-          c4[k] = lx[k] & kW4Index;
-          take(ok[k] && !leaf, (int32_t)c4[k]);
-        }
-      } else {
-        if (kTwo && node2 < 0 && sp > sb) node2 = stack[--sp];
-        bool gl, gr, gl2 = false, gr2 = false;
-        test_children(a, q, p, node, gl, gr, hl, hr, cl);
-        if (kTwo && node2 >= 0) {
-          test_children(a, q, p, node2, gl2, gr2, hl2, hr2, cl2);
-          nt += 2;
-        }
-        nt += 2;
-        take(gl, cl);
-        take(gr, cl + 1);
-        if (kTwo) {
-          take(gl2, cl2);
-          take(gr2, cl2 + 1);
-        }
-      }
-      if (overflow) {
-        atomicOr(&a.ctr->trav_flags, ERR_STACK);
-        p = -1;
-      } else if (first >= 0) {
-        node = first;
-        node2 = second;
-      } else if (sp > sb) {
-        node = stack[--sp];
-        node2 = -1;
-      } else {
-        p = -1;  // query (or the subtree taken from another lane) done
+      // the next pending node of the lowest level
+      const int l = __ffs(lv) - 1;
+      const uint32_t word = mine[l * kTvThreads];
+      const uint32_t rest = word & (word - 1u);
+      node = (word >> 8) * kWide + (__ffs(word) - 1);
+      mine[l * kTvThreads] = rest;
+      if (!(rest & 0xffu)) lv &= lv - 1u;
+      mask = meet_mask(a.nodes + off[l] + node, qlo, qhi);
+      nt += kWide;
+      // only children that hold a position in (p, cend)
+      const int sh = kWideBits * (l - 1);
+      const int lo = (int)((p + 1u) >> sh) - (int)(node * kWide);
+      const int hi = (int)((cend - 1u) >> sh) - (int)(node * kWide);
+      mask &= (0xffu << min(max(lo, 0), 8)) & ((2u << min(hi, 7)) - 1u);
+      leaf = l == 1;
+      if (!leaf && mask) {
+        mine[(l - 1) * kTvThreads] = node << 8 | mask;
+        lv |= 1u << (l - 1);
       }
     }
-    // append this step's hits to the warp buffer
-    auto append = [&](bool h, int32_t c) {
-      unsigned v = __ballot_sync(0xffffffffu, h);
-      if (h) buf[nhit + __popc(v & lt)] = make_uint2(pq, (uint32_t)c);
-      nhit += __popc(v);
-    };
-    if constexpr (kW4) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) append(h4[k], (int32_t)c4[k]);
-    } else {
-      append(hl, cl);
-      append(hr, cl + 1);
-      if (kTwo) {
-        append(hl2, cl2);
-        append(hr2, cl2 + 1);
+    // leaf nodes with boxes that meet go to the warp's buffer
+    const bool put = leaf && mask;
+    const unsigned v = __ballot_sync(0xffffffffu, put);
+    if (v) {
+      if (put) {
+        const int k = nent + __popc(v & lt);
+        buf.p[k] = p;
+        buf.n[k] = node;
+        buf.mask[k] = (uint8_t)mask;
       }
-    }
-    __syncwarp();
-    if (nhit > kHitCap - (kTwo || kW4 ? 128 : 64)) {
-      if constexpr (kRefine) drain_round_hits(a, buf, nhit);
-      else drain_hits(a, buf, nhit, we);
-      __syncwarp();
-      ntests += nhit;  // exact box tests, counted once per warp
-      nhit = 0;
+      nent += __popc(v);
+      if (nent > kEntryCap - 32) {
+        __syncwarp();
+        ntests += drain<kRefine>(a, buf, nent, we);  // exact box tests
+        nent = 0;
+      }
     }
   }
   __syncwarp();
-  if constexpr (kRefine) {
-    if (nhit > 0) drain_round_hits(a, buf, nhit);
-  } else {
-    if (nhit > 0) drain_hits(a, buf, nhit, we);
+  if (nent > 0) ntests += drain<kRefine>(a, buf, nent, we);
+  if constexpr (!kRefine) {
     chunk_fill_holes(we.s, a.starts, a.cap);
     if (!a.raw) chunk_fill_holes(we.e, a.ends, a.cap);
   }
-  ntests += nhit;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nt += __shfl_down_sync(0xffffffffu, nt, o);
   if (lane == 0) {
@@ -671,34 +517,39 @@ __global__ void __launch_bounds__(kT2Threads, 8) k_traverse2(TravArgs a) {
 }
 
 // persistent: as many blocks as fit on the GPU at once
-template <int kDepth, bool kTwo, bool kW4>
-static void launch_t2(const TravArgs &a, int sms, cudaStream_t st) {
-  static int per_sm = 0;
-  if (!per_sm)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse2<kDepth, kTwo, kW4>,
-                                                  kT2Threads, 0);
-  k_traverse2<kDepth, kTwo, kW4><<<(unsigned)(sms * std::max(per_sm, 1)), kT2Threads, 0, st>>>(
-      a);
+template <bool kRefine>
+static int launch_traverse(const TravArgs &a, cudaStream_t st) {
+  static int wave = 0;
+  if (!wave) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<kRefine>, kTvThreads, 0);
+    wave = std::max(sms, 1) * std::max(per_sm, 1);
+  }
+  // sorted boxes and nodes are read with 32-byte loads
+  if ((reinterpret_cast<uintptr_t>(a.sbox) | reinterpret_cast<uintptr_t>(a.nodes)) & 31)
+    return SCD_ERR_INTERNAL;
+  k_traverse<kRefine><<<(unsigned)wave, kTvThreads, 0, st>>>(a);
+  note_launch();
+  return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
 
 // One refinement round's traversal over up to cap sorted boxes (their count
-// on the device): one box per leaf, binary nodes, two nodes per step.
-int traverse_round(const QBox *qbox, const uint32_t *qlink, const SBox *sbox,
-                   const uint32_t *sobj, const uint32_t *sid, int64_t cap,
-                   const unsigned long long *d_N, int64_t T, DevCounters *ctr, uint32_t *rflags,
-                   unsigned long long *rcand, unsigned long long *rncand, unsigned long long rcap,
-                   int spans, int deep, cudaStream_t st) {
+// on the device).
+int traverse_round(const WideNode *nodes, const SBox *sbox, const uint32_t *sobj,
+                   const uint32_t *sid, int64_t cap, const unsigned long long *d_N, int64_t T,
+                   DevCounters *ctr, uint32_t *rflags, unsigned long long *rcand,
+                   unsigned long long *rncand, unsigned long long rcap, int spans,
+                   cudaStream_t st) {
   if (cap < 2) return SCD_OK;
-  if ((reinterpret_cast<uintptr_t>(sbox) | reinterpret_cast<uintptr_t>(qbox)) & 31)
-    return SCD_ERR_INTERNAL;
   TravArgs a{};
-  a.qbox = qbox;
-  a.qlink = qlink;
+  a.nodes = nodes;
+  a.lv = tree_levels(cap);
   a.sbox = sbox;
   a.sobj = sobj;
   a.sid = sid;
   a.N = cap;
-  a.L = 1;
   a.T = (int)T;
   a.ctr = ctr;
   a.dkind = SCD_DECOMP_NONE;
@@ -708,41 +559,19 @@ int traverse_round(const QBox *qbox, const uint32_t *qlink, const SBox *sbox,
   a.rncand = rncand;
   a.rcap = rcap;
   a.rspans = spans;
-  static int sms = 0, per64 = 0, per128 = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per64, k_traverse2<64, true, false, true>,
-                                                  kT2Threads, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per128, k_traverse2<128, true, false, true>,
-                                                  kT2Threads, 0);
-  }
-  if (deep)
-    k_traverse2<128, true, false, true>
-        <<<(unsigned)(sms * std::max(per128, 1)), kT2Threads, 0, st>>>(a);
-  else
-    k_traverse2<64, true, false, true>
-        <<<(unsigned)(sms * std::max(per64, 1)), kT2Threads, 0, st>>>(a);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
+  return launch_traverse<true>(a, st);
 }
 
-int traverse(scd_scene *s, int64_t n_leaves, int raw_mode, int obj_bits, int t_bits) {
+int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   TravArgs a{};
   a.nodes = s->d_nodes.p;
-  a.qbox = s->d_qbox.p;
-  a.qlink = s->d_qlink.p;
-  a.w4 = s->d_w4.p;
   a.sbox = s->s_box.p;
   a.sobj = s->s_obj.p;
   a.nb = s->s_nb.p;
   a.sid = s->d_id.p;
-  a.lo = s->d_lo.p;
-  a.hi = s->d_hi.p;
-  a.N = s->N;
-  a.L = s->tune.leaf_size;
-  a.M = n_leaves;
+  // one query per sorted reference
+  a.N = s->dkind != SCD_DECOMP_NONE ? s->n_refs : s->N;
+  a.lv = tree_levels(a.N);
   a.T = (int)s->T;
   a.raw = raw_mode;
   a.obj_bits = obj_bits;
@@ -758,45 +587,11 @@ int traverse(scd_scene *s, int64_t n_leaves, int raw_mode, int obj_bits, int t_b
   a.n_slabs = s->n_slabs;
   a.p_bands = s->p_bands;
   a.scell = s->s_cell.p;
-  a.cellroot = s->d_cellroot.p;
+  a.cellend = s->d_cellend.p;
   a.rr = s->d_rr.p;
   a.edges = s->d_edges.p;
   a.objT = s->n_scenes > 0 ? s->d_objT.p : nullptr;
-  if (a.dkind != SCD_DECOMP_NONE) a.N = s->n_refs;  // one query per reference
-  // sorted boxes (and node pairs) are read with 32-byte loads
-  if (reinterpret_cast<uintptr_t>(a.sbox) & 31) return SCD_ERR_INTERNAL;
-  if (a.L == 1) {
-    if (reinterpret_cast<uintptr_t>(a.qbox) & 31) return SCD_ERR_INTERNAL;
-    // persistent: as many blocks as fit on the GPU at once
-    static int sms = 0;
-    if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-    const bool two = s->tune.nodes_per_step == 2, w4 = s->tune.node_width == 4;
-    if (w4 && (reinterpret_cast<uintptr_t>(a.w4) & 127)) return SCD_ERR_INTERNAL;
-    auto go = [&](auto depth) {
-      constexpr int D = decltype(depth)::value;
-      if (w4) launch_t2<D, false, true>(a, sms, s->stream);
-      else if (two) launch_t2<D, true, false>(a, sms, s->stream);
-      else launch_t2<D, false, false>(a, sms, s->stream);
-    };
-    switch (s->tune.stack_depth) {
-      case 32: go(std::integral_constant<int, 32>()); break;
-      case 128: go(std::integral_constant<int, 128>()); break;
-      default: go(std::integral_constant<int, 64>()); break;
-    }
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
-  }
-  int bs = s->tune.block_threads;
-  if (bs < 32 || bs > 256 || bs % 32) bs = 128;
-  int64_t g = (s->N + bs - 1) / bs;
-  if (g == 0) return SCD_OK;
-  switch (s->tune.stack_depth) {
-    case 32: k_traverse<32><<<(unsigned)g, bs, 0, s->stream>>>(a); break;
-    case 128: k_traverse<128><<<(unsigned)g, bs, 0, s->stream>>>(a); break;
-    default: k_traverse<64><<<(unsigned)g, bs, 0, s->stream>>>(a); break;
-  }
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
+  return launch_traverse<false>(a, s->stream);
 }
 
 // ---------------------------------------------------------------------------
