@@ -48,7 +48,7 @@ class StepNet:
 
     def grad(self, x, t):
         import torch
-        g = torch.zeros(B.SCD_STEPNET_PARAMS, dtype=torch.float32, device=x.device)
+        g = torch.empty(B.SCD_STEPNET_PARAMS, dtype=torch.float32, device=x.device)
         loss = B.scd_stepnet_grad(self.handle, x.contiguous().data_ptr(),
                                   t.contiguous().data_ptr(), len(x), g.data_ptr())
         return loss, g
