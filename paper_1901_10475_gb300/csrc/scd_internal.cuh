@@ -432,7 +432,19 @@ int scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, DevBuf<int64_
 
 // the scene (opaque in the ABI)
 namespace scd {
-constexpr int kStreamBuckets = 16;  // buckets of a canonical list streamed to the host
+// Buckets of a canonical list streamed to the host; 1 = the list is sorted
+// whole and copied.  A bucket costs its own sorts' launches (about 40 kernels,
+// 140 us) and hides the sorting of the others under its copy (83 us a million
+// pairs): below 8 M pairs the launches cost more than they hide (7.1 M pairs:
+// 2.9 ms whole, 3.2 ms in 3 buckets), then four to five buckets are best (19.8 M
+// pairs 6.0 ms against 6.1 whole and 8.3 in 16, 47 M 10.9 ms in 5 against 12.5
+// in 2 or 16), and the longest lists take 16 (164 M 29.8 ms).
+constexpr int kStreamBuckets = 16;
+inline int stream_buckets(int64_t pairs) {
+  const int64_t few = pairs >> 22, many = pairs / 10000000;
+  const int64_t b = few < 5 ? few : many > 5 ? many : 5;
+  return b < 1 ? 1 : b > kStreamBuckets ? kStreamBuckets : (int)b;
+}
 struct RfCache;  // the refinement's buffers and captured rounds (refine.cu)
 }
 

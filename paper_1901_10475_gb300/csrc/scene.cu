@@ -422,19 +422,21 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
   // A9: canonical list (into host memory: streamed out bucket by bucket)
   s->host_done = false;
   int crc = SCD_ERR_STATE;
-  if (s->host_dst && !raw_mode && (int64_t)s->h_ctr.v_starts <= s->host_cap)
+  if (s->host_dst && !raw_mode && (int64_t)s->h_ctr.v_starts <= s->host_cap &&
+      stream_buckets((int64_t)s->h_ctr.v_starts) > 1)
     crc = canonicalize_streamed(s, ob, tb, s->host_dst);
   if (crc == SCD_OK) s->host_done = true;
   else if (crc != SCD_ERR_STATE) return crc;
   else TRY(canonicalize(s, raw_mode, ob, tb));
   if (s->events_ready) cudaEventRecord(s->ev[6], st);
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SCD_ERR_CUDA;
+  // the sorts' and the zip's error bits: one copy before the one wait
+  if (cudaMemcpyAsync(s->h_ctr_pinned, s->d_ctr.p, sizeof(DevCounters), cudaMemcpyDeviceToHost,
+                      st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return SCD_ERR_CUDA;
   if (s->host_done && cudaStreamSynchronize(s->cstream) != cudaSuccess) return SCD_ERR_CUDA;
-  unsigned int flags[2] = {0, 0};
-  cudaMemcpy(&flags[0], &s->d_ctr.p->trav_flags, sizeof(unsigned int), cudaMemcpyDeviceToHost);
-  cudaMemcpy(&flags[1], &s->d_ctr.p->sort_flags, sizeof(unsigned int), cudaMemcpyDeviceToHost);
-  if (flags[1] & ERR_SORT) return SCD_ERR_TIMEOUT;
-  if (flags[0] & ERR_ZIP) return SCD_ERR_INTERNAL;
+  if (s->h_ctr_pinned->sort_flags & ERR_SORT) return SCD_ERR_TIMEOUT;
+  if (s->h_ctr_pinned->trav_flags & ERR_ZIP) return SCD_ERR_INTERNAL;
   finish_metrics(s, raw_mode);
   return SCD_OK;
 }

@@ -897,14 +897,15 @@ int canonicalize_streamed(scd_scene *s, int obj_bits, int t_bits, scd_pair *host
   if (vs[255] < 0 || ve[255] < 0 || sum_s != n || sum_e != ne) return SCD_ERR_INTERNAL;
   int64_t out_at = 0;
   int d0 = 0;
-  for (int b = 0; b < kStreamBuckets && d0 < 256; ++b) {
+  const int nb = stream_buckets(n);
+  for (int b = 0; b < nb && d0 < 256; ++b) {
     // whole digits up to about an equal share of the starts still left; the
     // first bucket small, so that the copies (the slower stream) start early
-    const int64_t share = b == 0 ? (n + 63) / 64
-                                 : (n - out_at + (kStreamBuckets - b) - 1) / (kStreamBuckets - b);
+    const int64_t share = b == 0 ? (n + 4 * nb - 1) / (4 * nb)
+                                 : (n - out_at + (nb - b) - 1) / (nb - b);
     int d1 = d0;
     int64_t m = 0, me = 0;
-    while (d1 < 256 && (m < share || b == kStreamBuckets - 1)) {
+    while (d1 < 256 && (m < share || b == nb - 1)) {
       m += vs[d1];
       me += ve[d1];
       ++d1;
