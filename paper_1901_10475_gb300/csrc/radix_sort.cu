@@ -419,6 +419,288 @@ __global__ void __launch_bounds__(kRsThreads, 4) k_rs_downsweep(
   }
 }
 
+// ---------------------------------------------------------------------------
+// Small sorts: every pass in one launch, by one cluster of 16 blocks (16 SMs).
+// A block ranks its sixteenth of the keys in registers and stages them by
+// digit in shared memory; the blocks exchange their digit counts through
+// distributed shared memory and write their runs to global memory (L2 at
+// these sizes); the cluster's hardware barrier separates the steps.  Up to
+// kSoloMax keys one block does it alone, the keys in shared memory throughout.
+// A pass of three kernels takes about 18 us of launches and latency however
+// few the keys.  Five passes of (key, value) pairs: 1,204 keys 16 us (86 in
+// three kernels a pass), 3,913 26 (97), 15,050 42 (96), 45,150 51 (98), 90,300 68
+// (97), 154,112 92 (97), 210,700 108 (101): the SMs' ranking takes over.
+// ---------------------------------------------------------------------------
+constexpr int kClBlocks = 16, kClThreads = 1024, kClWarps = kClThreads / 32;
+constexpr int kClItems = 16;  // keys per thread at most
+constexpr int kSoloItems = 4;
+constexpr int64_t kSoloMax = (int64_t)kSoloItems * kClThreads;
+// up to 163,840 keys; where the count is on the device and the host knows only
+// a capacity, up to the most that fits (the refinement's first round is its
+// largest by far: 512 objects 192,512, then 2,594 and fewer)
+constexpr int64_t kClusterHost = (int64_t)10 * kClBlocks * kClThreads;
+constexpr int64_t kClusterMax = (int64_t)kClItems * kClBlocks * kClThreads;
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a word of another block's shared memory, by the address of one's own
+__device__ __forceinline__ uint32_t ld_cluster(const uint32_t *own, uint32_t rank) {
+  uint32_t v, addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_addr(own)), "r"(rank));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+struct ClusterSmem {
+  uint16_t wcnt[kClWarps][256];  // per warp and digit: counts, then tile positions
+  uint32_t total[256];           // the block's digit counts (read by the others)
+  uint32_t part[4][256];         // digit counts of eight warps each
+  uint32_t scan[256];
+  uint32_t gbase[256];           // a digit's global position less its tile position
+};
+template <class K>
+constexpr size_t cluster_smem(bool vals) {
+  return sizeof(ClusterSmem) + (size_t)kClItems * kClThreads * (sizeof(K) + (vals ? 4 : 0));
+}
+
+// exclusive scan of one value per digit (threads 0 .. 255; all threads call)
+__device__ __forceinline__ uint32_t digits_excl(uint32_t v, uint32_t *buf) {
+  const int t = threadIdx.x, lane = t & 31;
+  uint32_t x = v;
+  if (t < 256) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    buf[t] = x;
+  }
+  __syncthreads();
+  uint32_t add = 0;
+  if (t < 256)
+    for (int q = 0; q < (t >> 5); ++q) add += buf[q * 32 + 31];
+  __syncthreads();
+  return x + add - v;
+}
+
+// Stable ranks of the warp's kItems x 32 keys by digit (items up to `items`,
+// positions from first in steps of 32, below n), the block's digit counts,
+// and the keys (and values) staged at their tile positions.  Returns the
+// count of digit t and its first tile position (threads 0 .. 255).
+template <int kItems, class K, bool kVals, class LoadVal>
+__device__ __forceinline__ void stage_tile(ClusterSmem &sm, const K (&key)[kItems], uint32_t items,
+                                           uint32_t first, uint32_t n, int shift, K *kst,
+                                           uint32_t *vst, LoadVal load_val, uint32_t &count,
+                                           uint32_t &at0) {
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  for (int i = t; i < kClWarps * 128; i += kClThreads)
+    reinterpret_cast<uint32_t *>(&sm.wcnt[0][0])[i] = 0;
+  __syncthreads();
+  uint16_t rnk[kItems];
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    if ((uint32_t)k < items) {  // uniform
+      const bool valid = first + 32u * (uint32_t)k < n;
+      const uint32_t dg = valid ? digit_of(key[k], shift) : 256u;
+      const unsigned peers = __match_any_sync(0xffffffffu, dg);
+      const uint32_t before = valid ? sm.wcnt[w][dg] : 0u;
+      rnk[k] = (uint16_t)(before + __popc(peers & lt));
+      __syncwarp();
+      if (valid && lane == __ffs(peers) - 1) sm.wcnt[w][dg] = (uint16_t)(before + __popc(peers));
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  // a digit's counts over the warps: four threads of eight warps each
+  const int d = t & 255, q = t >> 8;
+  {
+    uint32_t run = 0;
+#pragma unroll
+    for (int j = 0; j < kClWarps / 4; ++j) {
+      const uint32_t c = sm.wcnt[q * (kClWarps / 4) + j][d];
+      sm.wcnt[q * (kClWarps / 4) + j][d] = (uint16_t)run;
+      run += c;
+    }
+    sm.part[q][d] = run;
+  }
+  __syncthreads();
+  count = t < 256 ? sm.part[0][t] + sm.part[1][t] + sm.part[2][t] + sm.part[3][t] : 0u;
+  if (t < 256) sm.total[t] = count;
+  at0 = digits_excl(count, sm.scan);
+  if (t < 256) sm.scan[t] = at0;
+  __syncthreads();
+  {
+    uint32_t b = sm.scan[d];
+    for (int j = 0; j < q; ++j) b += sm.part[j][d];
+#pragma unroll
+    for (int j = 0; j < kClWarps / 4; ++j)
+      sm.wcnt[q * (kClWarps / 4) + j][d] = (uint16_t)(sm.wcnt[q * (kClWarps / 4) + j][d] + b);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kItems; ++k) {
+    const uint32_t i = first + 32u * (uint32_t)k;
+    if ((uint32_t)k < items && i < n) {
+      const uint32_t r = (uint32_t)sm.wcnt[w][digit_of(key[k], shift)] + rnk[k];
+      kst[r] = key[k];
+      if (kVals) vst[r] = load_val(k, i);
+    }
+  }
+}
+
+template <class K, bool kVals>
+__global__ void __launch_bounds__(kClThreads, 1) k_rs_cluster(
+    K *__restrict__ keys, uint32_t *__restrict__ vals, K *__restrict__ keys_alt,
+    uint32_t *__restrict__ vals_alt, int64_t n_cap, const unsigned long long *__restrict__ d_n,
+    int lo, int bits) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(smem);
+  K *kst = reinterpret_cast<K *>(smem + sizeof(ClusterSmem));
+  uint32_t *vst = reinterpret_cast<uint32_t *>(kst + (size_t)kClItems * kClThreads);
+  const uint32_t n = (uint32_t)sort_count(n_cap, d_n);
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  uint32_t rank;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+
+  if (n <= (uint32_t)kSoloMax) {  // the whole cluster decides alike
+    if (rank != 0u || n == 0u) return;
+    const uint32_t items = (n + kClThreads - 1) / kClThreads;
+    const uint32_t first = (uint32_t)w * 32u * items + (uint32_t)lane;
+    K key[kSoloItems];
+    uint32_t val[kSoloItems];
+#pragma unroll
+    for (int k = 0; k < kSoloItems; ++k) {
+      const uint32_t i = first + 32u * (uint32_t)k;
+      const bool in = (uint32_t)k < items && i < n;
+      key[k] = in ? keys[i] : (K)0;
+      val[k] = kVals && in ? vals[i] : 0u;
+    }
+    for (int shift = lo; shift < bits; shift += 8) {
+      uint32_t c, a;
+      stage_tile<kSoloItems, K, kVals>(sm, key, items, first, n, shift, kst, vst,
+                                       [&](int k, uint32_t) { return val[k]; }, c, a);
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kSoloItems; ++k) {
+        const uint32_t i = first + 32u * (uint32_t)k;
+        if ((uint32_t)k < items && i < n) {
+          key[k] = kst[i];
+          if (kVals) val[k] = vst[i];
+        }
+      }
+      // (stage_tile writes the staging area only after its own barriers)
+    }
+#pragma unroll
+    for (int k = 0; k < kSoloItems; ++k) {
+      const uint32_t i = first + 32u * (uint32_t)k;
+      if ((uint32_t)k < items && i < n) {
+        keys[i] = key[k];
+        if (kVals) vals[i] = val[k];
+      }
+    }
+    return;
+  }
+
+  const uint32_t items = (n + kClBlocks * kClThreads - 1) / (kClBlocks * kClThreads);
+  // the warp's keys: items x 32 consecutive ones, item k of a lane at
+  // first + 32 k, so (item, lane) order is input order and ranks are stable
+  const uint32_t tile0 = rank * kClThreads * items;
+  const uint32_t first = tile0 + (uint32_t)w * 32u * items + (uint32_t)lane;
+  const uint32_t cnt = tile0 < n ? min(n - tile0, (uint32_t)kClThreads * items) : 0u;
+  const K *ks = keys;
+  K *kd = keys_alt;
+  const uint32_t *vs = vals;
+  uint32_t *vd = vals_alt;
+  for (int shift = lo; shift < bits; shift += 8) {
+    K key[kClItems];
+    // (read past L1: another block wrote them in the pass before)
+#pragma unroll
+    for (int k = 0; k < kClItems; ++k) {
+      const uint32_t i = first + 32u * (uint32_t)k;
+      key[k] = (uint32_t)k < items && i < n ? __ldcg(ks + i) : (K)0;
+    }
+    uint32_t count, at0;
+    stage_tile<kClItems, K, kVals>(sm, key, items, first, n, shift, kst, vst,
+                                   [&](int, uint32_t i) { return __ldcg(vs + i); }, count, at0);
+    cluster_arrive();
+    cluster_wait();
+    // the digit's keys in the blocks before this one, and in all of them
+    uint32_t before = 0, all = 0;
+    if (t < 256) {
+#pragma unroll
+      for (uint32_t r = 0; r < kClBlocks; ++r) {
+        const uint32_t c = ld_cluster(&sm.total[t], r);
+        before += r < rank ? c : 0u;
+        all += c;
+      }
+    }
+    const uint32_t g0 = digits_excl(all, sm.scan);
+    if (t < 256) sm.gbase[t] = g0 + before - at0;
+    __syncthreads();
+    for (uint32_t r = t; r < cnt; r += kClThreads) {
+      const K k = kst[r];
+      const uint32_t pos = sm.gbase[digit_of(k, shift)] + r;
+      kd[pos] = k;
+      if (kVals) vd[pos] = vst[r];
+    }
+    cluster_arrive();
+    cluster_wait();  // every key is in place, and every count has been read
+    K *kt = const_cast<K *>(ks);
+    ks = kd;
+    kd = kt;
+    uint32_t *vt = const_cast<uint32_t *>(vs);
+    vs = vd;
+    vd = vt;
+  }
+  if (ks != keys) {  // an odd number of passes
+    for (uint32_t r = t; r < cnt; r += kClThreads) {
+      keys[tile0 + r] = __ldcg(ks + tile0 + r);
+      if (kVals) vals[tile0 + r] = __ldcg(vs + tile0 + r);
+    }
+  }
+}
+
+// one launch of the cluster sort; SCD_ERR_STATE where the device cannot run
+// a cluster of 16 such blocks
+template <class K, bool kVals>
+static int rs_cluster(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
+                      const unsigned long long *d_n, int lo, int bits, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kClBlocks);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = cluster_smem<K>(kVals);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kClBlocks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  static int fits = -1;
+  if (fits < 0) {
+    int clusters = 0;
+    const bool ok =
+        cudaFuncSetAttribute(k_rs_cluster<K, kVals>,
+                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_rs_cluster<K, kVals>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)cfg.dynamicSmemBytes) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, k_rs_cluster<K, kVals>, &cfg) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    fits = ok && clusters > 0;
+  }
+  if (!fits) return SCD_ERR_STATE;
+  if (cudaLaunchKernelEx(&cfg, k_rs_cluster<K, kVals>, keys, vals, keys_alt, vals_alt, n, d_n, lo,
+                         bits) != cudaSuccess)
+    return SCD_ERR_CUDA;
+  note_launch();
+  return SCD_OK;
+}
+
 template <class K>
 static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long *d_n, int lo,
                    int bits, SortScratch &sc, cudaStream_t st, const PairEmit *pe = nullptr) {
@@ -431,6 +713,12 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
   int64_t nblk = (n + kRsTile - 1) / kRsTile;
   if (!sc.keys_alt.ensure(sizeof(K) * (size_t)n, st)) return SCD_ERR_OOM;
   if (vals && !sc.vals_alt.ensure((size_t)n, st)) return SCD_ERR_OOM;
+  if (!pe && n <= (d_n ? kClusterMax : kClusterHost)) {
+    K *alt = (K *)sc.keys_alt.p;
+    const int rc = vals ? rs_cluster<K, true>(keys, vals, alt, sc.vals_alt.p, n, d_n, lo, bits, st)
+                        : rs_cluster<K, false>(keys, nullptr, alt, nullptr, n, d_n, lo, bits, st);
+    if (rc != SCD_ERR_STATE) return rc;
+  }
   if (!sc.counts.ensure((size_t)(256 * nblk + 256), st)) return SCD_ERR_OOM;
   uint32_t *counts = sc.counts.p;
   uint32_t *totals = sc.counts.p + 256 * nblk;

@@ -534,7 +534,7 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int r
                                                      B.tcap);
       note_launch();
     }
-    int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, 0, kb, B.sc, st);
+    int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, sort_key_skip(kb, cap), kb, B.sc, st);
     if (rc != SCD_OK) return rc;
     rc = build_round_tree(B.idx.p, B.lo.p, B.hi.p, B.obj[cur].p, cap, dM, B.sbox.p, B.sobj.p,
                           B.nodes.p, B.nbox.p, st);

@@ -256,6 +256,13 @@ __host__ __device__ inline unsigned long long sort_key(unsigned long long curve,
   if (bits >= 12) return (curve >> 1) | (unsigned long long)group << (4 * bits - 1);
   return curve | (unsigned long long)group << (4 * bits);
 }
+// Lowest key bits left out of the sort (boxes of equal higher bits stay in
+// input order): up to 2^20 boxes the top 40 bits order them as well as 48
+// (3001 objects, 7 h, 0.9 M boxes: 32.4 nodes a query either way on the CPU
+// model), one pass fewer.
+inline int sort_key_skip(int key_bits, int64_t boxes) {
+  return boxes <= (1 << 20) && key_bits > 40 ? key_bits - 40 : 0;
+}
 inline int sort_key_bits(const scd_tuning &t) {
   const bool split = split_of(t) != 0.0f;
   return 4 * t.morton_bits + (split && t.morton_bits < 12 ? 1 : 0);

@@ -376,7 +376,7 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
     // A5: sort box ids along the Hilbert curve
     int kb = sort_key_bits(s->tune);
     if (s->tune.morton_bits > 8) {
-      TRY(radix_sort_u64(s->d_key64.p, s->d_id.p, N, kb, s->sort_sc, st));
+      TRY(radix_sort_u64(s->d_key64.p, s->d_id.p, N, sort_key_skip(kb, N), kb, s->sort_sc, st));
     } else {
       TRY(radix_sort_u32(s->d_key32.p, s->d_id.p, N, kb, s->sort_sc, st));
     }
@@ -450,7 +450,8 @@ static int enqueue_find(scd_scene *s, const scd_decomp *d, int dkind, int ob, in
   if (dkind == SCD_DECOMP_NONE) {
     int kb = sort_key_bits(s->tune);
     if (s->tune.morton_bits > 8) {
-      TRY(radix_sort_u64(s->d_key64.p, s->d_id.p, s->N, kb, s->sort_sc, st));
+      TRY(radix_sort_u64(s->d_key64.p, s->d_id.p, s->N, sort_key_skip(kb, s->N), kb, s->sort_sc,
+                         st));
     } else {
       TRY(radix_sort_u32(s->d_key32.p, s->d_id.p, s->N, kb, s->sort_sc, st));
     }
