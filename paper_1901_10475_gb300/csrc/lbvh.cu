@@ -49,16 +49,18 @@ __device__ __forceinline__ float4 f4_xor_lane(float4 a, int d) {
                      __shfl_xor_sync(0xffffffffu, a.z, d), __shfl_xor_sync(0xffffffffu, a.w, d));
 }
 
-// One axis of a node's frame.  Space: the node's own extent onto [0, 1].
-// Ticks (whole numbers): half a tick of room on both sides, and one cell per
-// tick while the node spans at most 128 of them, so that consecutive
-// segments, which touch without overlapping, stay apart.
+// One axis of a node's frame: its own extent onto cells 1.25 to 126.25 of 127
+// (whole cells 1 to 126; 0 and 127 are outside).  Ticks (whole numbers): onto
+// the middles of cells, one cell per tick while the node spans at most 125 of
+// them, so that consecutive segments, which touch without overlapping, stay
+// apart.
 __device__ __forceinline__ void axis_frame(float lo, float hi, bool tick, float &scale,
                                            float &off) {
   const float ext = hi - lo;
-  scale = tick ? 1.0f / fmaxf(ext + 1.0f, 128.0f) : 1.0f / ext;
-  off = (tick ? 0.5f - lo : -lo) * scale;
-  if (!isfinite(scale) || !isfinite(off)) scale = off = 0.0f;
+  scale = tick ? (125.0f / kCellTop) / fmaxf(ext, 125.0f) : (125.0f / kCellTop) / ext;
+  off = (tick ? 1.5f : 1.25f) / kCellTop - lo * scale;
+  // (an infinite extent would map finite faces to a cell above infinite ones)
+  if (!isfinite(ext) || !isfinite(scale) || !isfinite(off)) scale = off = 0.0f;
 }
 
 // Eight neighbouring lanes hold a node's children (valid: the child exists);
@@ -84,7 +86,7 @@ __device__ __forceinline__ void make_node(float4 &lo, float4 &hi, bool valid, Wi
   axis_frame(lo.w, hi.w, true, s.w, o.w);
   unsigned char *bl = reinterpret_cast<unsigned char *>(dst->lo) + c;
   unsigned char *bh = reinterpret_cast<unsigned char *>(dst->hi) + c;
-  // a child that does not exist: lower faces at the top, upper ones at 0
+  // a child that does not exist: lower faces above all, upper ones below
   bl[0] = valid ? (unsigned char)node_coord(cl.x, s.x, o.x, false) : 127;
   bl[8] = valid ? (unsigned char)node_coord(cl.y, s.y, o.y, false) : 127;
   bl[16] = valid ? (unsigned char)node_coord(cl.z, s.z, o.z, false) : 127;

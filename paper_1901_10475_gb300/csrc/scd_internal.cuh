@@ -77,7 +77,8 @@ struct DevCounters {
 // m of level k covers the sorted boxes [m 8^k, (m + 1) 8^k), so there are no
 // links and no depth to discover; its children are the nodes 8 m .. 8 m + 7
 // of level k - 1 (the boxes themselves below level 1).  A node holds its
-// frame (per axis a scale and an offset that map its own box onto [0, 127])
+// frame (per axis a scale and an offset that map its own box onto the cells
+// 1 to 126 of 0 to 127, so that a face outside it is told apart from one on it)
 // and its children's faces in that frame, one byte each, axis by axis with
 // the eight children side by side: a query is brought into the frame once
 // and then tested against four children per instruction.  The upper faces
@@ -123,8 +124,10 @@ inline TreeLevels tree_levels(int64_t cap) {
 // [0, 1], then added to 2^23 with rounding down, where one unit is the last
 // place.  Both steps are monotone in x for a fixed frame, so order
 // relations survive (a NaN clamps to 0: a frame that is not finite has scale
-// and offset 0, and every coordinate becomes 0).
-constexpr float kCellTop = 127.9f;
+// and offset 0, and every coordinate becomes 0).  A query wholly above the
+// node has a lower face in cell 127, one wholly below it an upper face in cell
+// 0: no child reaches either, so the node's children all fail at once.
+constexpr float kCellTop = 127.0f;
 __device__ __forceinline__ uint32_t node_coord(float x, float scale, float off, bool guard) {
   float s, u;
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(s) : "f"(x), "f"(scale), "f"(off));

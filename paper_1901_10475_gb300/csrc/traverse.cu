@@ -39,7 +39,8 @@ struct TravArgs {
   uint32_t open_tag;          // last tick of an open run start
   unsigned long long *starts, *ends;
   uint32_t *rawval;           // raw cells' (or unpacked run starts') last tick
-  unsigned long long cap;
+  uint32_t cap;               // record slots (at most 2^32 - 1025)
+  uint32_t chunk;             // slots reserved at a time
   DevCounters *ctr;
   // static decomposition (kind SCD_DECOMP_NONE: one tree over all boxes)
   int dkind;
@@ -86,38 +87,45 @@ __device__ __forceinline__ bool reports_here(const TravArgs &a, uint32_t cell, f
 constexpr unsigned long long kHole = ~0ull;
 
 // Whole-warp emission into a chunk of slots reserved by the warp (one atomic
-// per kChunk records).  A chunk's unused tail is filled with holes.  Every
-// lane of the warp calls put() together; the chunk state is warp-uniform.
-constexpr unsigned kChunk = 512;
+// per chunk).  A chunk's unused tail is filled with holes, which the record
+// sorts carry along, so small screens take small chunks: at most as many
+// slots as boxes a warp (3001 objects, 2 h: 2.5 M slots of 512 for 0.46 M
+// records).  Every lane of the warp calls put() together; the chunk state is
+// warp-uniform.
+constexpr unsigned kMinChunk = 32, kMaxChunk = 512;
+// (slot numbers in 32 bits: the record sorts take no more, and a list that
+// would need more is refused)
 struct ChunkCursor {
-  unsigned long long next = 0, end = 0, count = 0;
+  uint32_t next = 0, end = 0, count = 0;
 };
 
 __device__ __forceinline__ void chunk_fill_holes(ChunkCursor &c, unsigned long long *buf,
-                                                 unsigned long long cap) {
+                                                 uint32_t cap) {
   const int lane = threadIdx.x & 31;
-  for (unsigned long long k = c.next + lane; k < c.end; k += 32)
+  for (uint32_t k = c.next + lane; k < c.end; k += 32)
     if (k < cap) buf[k] = kHole;
   c.next = c.end;
 }
 
 __device__ __forceinline__ void chunk_put(ChunkCursor &c, unsigned long long *buf, uint32_t *vbuf,
-                                          unsigned long long *slots, unsigned long long cap,
+                                          unsigned long long *slots, uint32_t cap, uint32_t chunk,
                                           bool pred, unsigned long long key, uint32_t v) {
   const int lane = threadIdx.x & 31;
-  unsigned vote = __ballot_sync(0xffffffffu, pred);
-  unsigned cnt = __popc(vote);
+  const unsigned vote = __ballot_sync(0xffffffffu, pred);
+  const uint32_t cnt = __popc(vote);
   if (cnt == 0) return;
   if (c.next + cnt > c.end) {
     chunk_fill_holes(c, buf, cap);
     unsigned long long b = 0;
-    if (lane == 0) b = atomicAdd(slots, (unsigned long long)kChunk);
-    b = __shfl_sync(0xffffffffu, b, 0);
-    c.next = b;
-    c.end = b + kChunk;
+    if (lane == 0) {
+      b = atomicAdd(slots, (unsigned long long)chunk);
+      if (b > 0xffffffffull - 2 * kMaxChunk) b = 0xffffffffull - 2 * kMaxChunk;  // past any cap
+    }
+    c.next = __shfl_sync(0xffffffffu, (uint32_t)b, 0);
+    c.end = c.next + chunk;
   }
   if (pred) {
-    unsigned long long idx = c.next + __popc(vote & ((1u << lane) - 1u));
+    const uint32_t idx = c.next + __popc(vote & ((1u << lane) - 1u));
     if (idx < cap) {
       buf[idx] = key;
       if (vbuf) vbuf[idx] = v;
@@ -169,24 +177,32 @@ __device__ __forceinline__ unsigned long long start_key(const TravArgs &a, unsig
 // lane whose query is done takes the next one from a pool its warp claims in
 // blocks; leaf nodes with overlapping boxes go to a per-warp buffer and the
 // records of their pairs are worked out by the whole warp together, into
-// output chunks the warp reserves kChunk slots at a time.
+// output chunks the warp reserves.
 //
-// The lane's pending nodes are one 32-bit word per level (the parent's index
-// and a mask of its children still to visit): at most ten words in shared
-// memory, whatever the query, so no stack can overflow.
+// kGroup neighbouring lanes walk together: their queries are consecutive along
+// the curve and visit nearly the same nodes, so the group visits the union of
+// them and one load serves its lanes.  A group's pending nodes are one 32-bit
+// word per level (the parent's index and a mask of its children still to
+// visit): at most ten words in shared memory, whatever the query, so no stack
+// can overflow.
 //
-// Measured on the 24 h catalog screen (17.4 M boxes): 12.0 ms and 40 nodes a
-// query with SPEED boxes, 6.5 ms and 35 with INTERVAL boxes; two-child nodes
-// of 36 bytes along a Morton curve, with 64-entry stacks in local memory,
-// took 18.4 ms and 91, 10.7 ms and 65.  Bound by the L1's load wavefronts
-// (87% of its peak while active: 32 lanes on 32 different nodes take one
-// wavefront for each of the three loads of a node).
+// Bound by the L1's wavefronts: a node's three 32-byte loads take one each per
+// distinct line, and a pair's exact boxes, objects and neighbouring segments
+// about 135 per 32 pairs.  Measured on the 24 h catalog screen (17.4 M boxes,
+// 164 M runs; SPEED / INTERVAL boxes): lanes alone 12.2 / 6.5 ms, groups of two
+// 11.3 / 5.9, of four 11.6 / 6.1, of eight 14.1 / 7.7; with groups of two, 256
+// buffered leaf nodes instead of 160 take SPEED from 11.5 to 11.3; fetching the
+// children ahead into L1 costs more wavefronts than it hides (17.7 / 15.8).
+// Two-child nodes of 36 bytes along a Morton curve, with 64-entry stacks in
+// local memory, took 18.4 / 10.7 ms and 91 nodes a query.
 // ---------------------------------------------------------------------------
 constexpr int kTvThreads = 128;
 constexpr int kTvWarps = kTvThreads / 32;
+// lanes that walk together (their queries are consecutive)
+constexpr int kGroup = 2;
 // leaf nodes (query, node, mask of its boxes) buffered per warp, drained when
 // fewer than one step's worth (32) of slots remain
-constexpr int kEntryCap = 160;
+constexpr int kEntryCap = 256;
 // entries expanded into single pairs at a time, two per lane
 constexpr int kExpand = 64;
 // queries claimed per warp atomic; small, so that the queries in flight stay
@@ -244,8 +260,8 @@ __device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint3
   int s = max((int)ql.w, (int)bl.w), e = min((int)qh.w, (int)bh.w);
   unsigned long long pk = pair_key(a, qo, bo);
   if (a.raw) {
-    chunk_put(we.s, a.starts, a.rawval, &a.ctr->n_raw, a.cap, valid, pk | (unsigned long long)s,
-              (uint32_t)e);
+    chunk_put(we.s, a.starts, a.rawval, &a.ctr->n_raw, a.cap, a.chunk, valid,
+              pk | (unsigned long long)s, (uint32_t)e);
     return;
   }
   bool start = valid, end = valid;
@@ -253,9 +269,10 @@ __device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint3
     run_ends_sorted(a, ql, qh, __ldg(a.nb + p), bl, bh, __ldg(a.nb + b), s, e,
                     a.objT ? __ldg(a.objT + qo) : a.T, start, end);
   const uint32_t last = end ? (uint32_t)e : a.open_tag;
-  chunk_put(we.s, a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, a.cap, start,
+  chunk_put(we.s, a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, a.cap,
+            a.chunk, start,
             start_key(a, pk, s, last), last);
-  chunk_put(we.e, a.ends, nullptr, &a.ctr->n_ends, a.cap, end && !start,
+  chunk_put(we.e, a.ends, nullptr, &a.ctr->n_ends, a.cap, a.chunk, end && !start,
             pk | (unsigned long long)e, 0u);
 }
 
@@ -339,147 +356,169 @@ __device__ __forceinline__ uint32_t meet_mask(const WideNode *nd, float4 qlo, fl
 template <bool kRefine>
 __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
   __shared__ HitBuf hits[kTvWarps];
-  __shared__ uint32_t pend[kMaxLevels][kTvThreads];  // [level - 1]: parent << 8 | children mask
+  __shared__ uint32_t pend[kMaxLevels][kTvThreads / kGroup];  // [level - 1]: parent << 8 | mask
   __shared__ uint32_t off[kMaxLevels + 1];
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr int kStride = kTvThreads / kGroup;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int sub = lane & (kGroup - 1);
   const unsigned lt = (1u << lane) - 1u;
+  constexpr unsigned kLead = 0x55555555u;  // the groups' first lanes
+  static_assert(kGroup == 2, "kLead and the group reduction are for pairs of lanes");
   HitBuf &buf = hits[w];
-  uint32_t *const mine = &pend[0][threadIdx.x] - kTvThreads;  // level l at mine[l * kTvThreads]
+  uint32_t *const mine = &pend[0][threadIdx.x / kGroup] - kStride;  // level l at mine[l * kStride]
   if (threadIdx.x <= kMaxLevels) off[threadIdx.x] = a.lv.off[threadIdx.x];
   __syncthreads();
   int nent = 0;  // warp-uniform
-  unsigned long long nt = 0, ntests = 0;
+  uint32_t visits = 0;
+  uint32_t ntests = 0;
   uint32_t p = 0;     // current query (sorted position)
-  uint32_t cend = 0;  // one past the last position it may meet
-  uint32_t lv = 0;    // levels with pending nodes; 0 = no query
+  uint32_t cend = 0;  // one past the last position it may meet (0: no query)
+  uint32_t lv = 0;    // the group's levels with pending nodes; 0 = no query
   float4 qlo = make_float4(0.f, 0.f, 0.f, 0.f), qhi = qlo;
-  bool exhausted = false;
+  bool dry = false;   // warp-uniform: the queue is empty
   // the last box has no later partner: queries are 0 .. N-2
   const int64_t nbox = kRefine && a.d_N && *a.d_N < (unsigned long long)a.N ? (int64_t)*a.d_N
                                                                             : a.N;
-  const unsigned long long nq = nbox > 1 ? (unsigned long long)(nbox - 1) : 0ull;
-  unsigned long long q_next = 0, q_end = 0;  // the warp's query pool
+  const uint32_t nq = nbox > 1 ? (uint32_t)(nbox - 1) : 0u;
+  // the warp's query pool: the first chunk by the warp's place in the grid,
+  // the later ones by the counter (no atomics where a few warps do it all)
+  uint32_t q_next = min((blockIdx.x * kTvWarps + w) * kQueryChunk, nq);
+  uint32_t q_end = q_next + kQueryChunk;
   WarpEmit we;
   for (;;) {
-    // lanes without a query take the next ones from the warp's pool
-    const unsigned need = __ballot_sync(0xffffffffu, lv == 0u && !exhausted);
-    if (need) {
-      const unsigned cnt = __popc(need);
-      const unsigned long long have = q_end - q_next;
-      unsigned long long nb = 0;
-      if (have < cnt) {
-        if (lane == 0) nb = atomicAdd(&a.ctr->work_next, (unsigned long long)kQueryChunk);
-        nb = __shfl_sync(0xffffffffu, nb, 0);
-      }
-      if (need & (1u << lane)) {
-        const unsigned r = __popc(need & lt);
-        const unsigned long long q = r < have ? q_next + r : nb + (r - have);
-        if (q < nq) {
-          p = (uint32_t)q;
-          ldg_box(a.sbox + p, qlo, qhi);
-          cend = (uint32_t)nbox;
-          if (!kRefine && a.dkind != SCD_DECOMP_NONE)
-            cend = (uint32_t)__ldg(a.cellend + __ldg(a.scell + p));
-          if (p + 1u < cend) {
-            // start at the smallest node that holds p and the last position
-            const int h = (kWideBits + 31 - __clz((int)(p ^ (cend - 1u)))) / kWideBits;
-            const uint32_t top = p >> (kWideBits * h);
-            mine[h * kTvThreads] = (top >> kWideBits) << 8 | 1u << (top & 7u);
-            lv = 1u << h;
+    unsigned idle = __ballot_sync(kFull, lv == 0u);
+    if (idle) {
+      if (!dry) {
+        // groups without queries take the next ones from the warp's pool
+        const uint32_t cnt = (uint32_t)__popc(idle);  // whole groups are idle
+        const uint32_t have = q_end - q_next;
+        uint32_t nb = 0;
+        if (have < cnt) {
+          const unsigned long long later = (unsigned long long)gridDim.x * kTvWarps * kQueryChunk;
+          unsigned long long c = 0;
+          if (later < (unsigned long long)nq) {
+            if (lane == 0) c = atomicAdd(&a.ctr->work_next, (unsigned long long)kQueryChunk);
+            c = __shfl_sync(kFull, c, 0);
           }
+          c += later;
+          dry = c >= (unsigned long long)nq;
+          nb = dry ? nq : (uint32_t)c;
+        }
+        const uint32_t r = (uint32_t)__popc(idle & lt);
+        const uint32_t q = r < have ? q_next + r : nb + (r - have);
+        uint32_t gend = 0;
+        if (lv == 0u) {
+          cend = 0;
+          if (q < nq) {
+            p = q;
+            ldg_box(a.sbox + p, qlo, qhi);
+            cend = (uint32_t)nbox;
+            if (!kRefine && a.dkind != SCD_DECOMP_NONE)
+              cend = (uint32_t)__ldg(a.cellend + __ldg(a.scell + p));
+            if (p + 1u >= cend) cend = 0;  // the last of its cell
+          }
+          gend = cend;
+        }
+        // the group's end (its queries may lie in several cells) and start
+        gend = max(gend, __shfl_xor_sync(kFull, gend, 1));
+        const uint32_t p0 = q - (uint32_t)sub;
+        if (lv == 0u && gend > 0u) {
+          // start at the smallest node that holds p0 and the last position
+          const int h = (kWideBits + 31 - __clz((int)(p0 ^ (gend - 1u)))) / kWideBits;
+          const uint32_t top = p0 >> (kWideBits * h);
+          mine[h * kStride] = (top >> kWideBits) << 8 | 1u << (top & 7u);
+          lv = 1u << h;
+        }
+        if (have < cnt) {
+          q_next = nb + (cnt - have);
+          q_end = nb + kQueryChunk;
         } else {
-          exhausted = true;
+          q_next += cnt;
         }
-      }
-      if (have < cnt) {
-        q_next = nb + (cnt - have);
-        q_end = nb + kQueryChunk;
+        __syncwarp();
       } else {
-        q_next += cnt;
-      }
-    }
-    // Once the queue is empty, a lane without a query takes pending nodes of
-    // a lane that has some to spare, with its query: the whole word of its
-    // highest level, or the last child of its only one; one long query then
-    // spreads over the warp instead of holding it.
-    if (__ballot_sync(0xffffffffu, exhausted)) {
-      const int hl = lv ? 31 - __clz((int)lv) : 0;
-      const uint32_t word = lv ? mine[hl * kTvThreads] : 0u;
-      const bool more = (lv & (lv - 1u)) != 0u;  // a lower level has some too
-      const unsigned idle = __ballot_sync(0xffffffffu, lv == 0u);
-      const unsigned donors =
-          __ballot_sync(0xffffffffu, more || __popc(word & 0xffu) > 1);
-      const int moves = min(__popc(idle), __popc(donors));
-      if (moves > 0) {
-        const bool is_idle = (idle >> lane) & 1u, is_donor = (donors >> lane) & 1u;
-        const int ri = __popc(idle & lt), rd = __popc(donors & lt);
-        const uint32_t top = 0x80u >> (__clz((int)(word & 0xffu)) - 24);  // last child's bit
-        const uint32_t give = more ? word : (word & ~0xffu) | top;
-        // the receiver of rank k takes from the donor of rank k
-        int src = lane;
-        if (is_idle && ri < moves) {
-          unsigned m = donors;
-          for (int k = 0; k < ri; ++k) m &= m - 1u;
-          src = __ffs(m) - 1;
-        }
-        const uint32_t gword = __shfl_sync(0xffffffffu, give, src);
-        const int glevel = __shfl_sync(0xffffffffu, hl, src);
-        const uint32_t gp = __shfl_sync(0xffffffffu, p, src);
-        const uint32_t gend = __shfl_sync(0xffffffffu, cend, src);
-        float4 glo, ghi;
-        glo.x = __shfl_sync(0xffffffffu, qlo.x, src);
-        glo.y = __shfl_sync(0xffffffffu, qlo.y, src);
-        glo.z = __shfl_sync(0xffffffffu, qlo.z, src);
-        glo.w = __shfl_sync(0xffffffffu, qlo.w, src);
-        ghi.x = __shfl_sync(0xffffffffu, qhi.x, src);
-        ghi.y = __shfl_sync(0xffffffffu, qhi.y, src);
-        ghi.z = __shfl_sync(0xffffffffu, qhi.z, src);
-        ghi.w = __shfl_sync(0xffffffffu, qhi.w, src);
-        if (is_donor && rd < moves) {
-          if (more) lv ^= 1u << hl;
-          else mine[hl * kTvThreads] = word ^ top;
-        }
-        if (is_idle && ri < moves) {
-          p = gp;
-          cend = gend;
-          qlo = glo;
-          qhi = ghi;
-          mine[glevel * kTvThreads] = gword;
-          lv = 1u << glevel;
+        // The queue is empty: an idle group takes pending nodes of a group
+        // that has some to spare, with its queries: the whole word of its
+        // highest level, or the last child of its only one; long queries then
+        // spread over the warp instead of holding it.
+        if (idle == kFull) break;
+        const int hl = lv ? 31 - __clz((int)lv) : 0;
+        const uint32_t word = lv ? mine[hl * kStride] : 0u;
+        const bool more = (lv & (lv - 1u)) != 0u;  // a lower level has some too
+        idle &= kLead;
+        const unsigned donors =
+            __ballot_sync(kFull, more || __popc(word & 0xffu) > 1) & kLead;
+        const int moves = min(__popc(idle), __popc(donors));
+        if (moves > 0) {
+          const int lead = lane - sub;  // the group's first lane
+          const unsigned lb = (1u << lead) - 1u;
+          const int ri = __popc(idle & lb), rd = __popc(donors & lb);
+          const bool take = ((idle >> lead) & 1u) && ri < moves;
+          const bool give = ((donors >> lead) & 1u) && rd < moves;
+          const uint32_t top = 0x80u >> (__clz((int)(word & 0xffu)) - 24);  // last child's bit
+          const uint32_t part = more ? word : (word & ~0xffu) | top;
+          // the receiver of rank k takes from the donor of rank k
+          int src = lane;
+          if (take) {
+            unsigned m = donors;
+            for (int k = 0; k < ri; ++k) m &= m - 1u;
+            src = __ffs(m) - 1 + sub;
+          }
+          const uint32_t gword = __shfl_sync(kFull, part, src);
+          const int glevel = __shfl_sync(kFull, hl, src);
+          p = __shfl_sync(kFull, p, src);
+          cend = __shfl_sync(kFull, cend, src);
+          qlo.x = __shfl_sync(kFull, qlo.x, src);
+          qlo.y = __shfl_sync(kFull, qlo.y, src);
+          qlo.z = __shfl_sync(kFull, qlo.z, src);
+          qlo.w = __shfl_sync(kFull, qlo.w, src);
+          qhi.x = __shfl_sync(kFull, qhi.x, src);
+          qhi.y = __shfl_sync(kFull, qhi.y, src);
+          qhi.z = __shfl_sync(kFull, qhi.z, src);
+          qhi.w = __shfl_sync(kFull, qhi.w, src);
+          if (give) {
+            if (more) lv ^= 1u << hl;
+            else mine[hl * kStride] = word ^ top;
+          }
+          if (take) {
+            mine[glevel * kStride] = gword;
+            lv = 1u << glevel;
+          }
+          __syncwarp();
         }
       }
     }
-    const bool active = lv != 0u;
-    if (__ballot_sync(0xffffffffu, active) == 0u) {
-      if (__ballot_sync(0xffffffffu, exhausted) == 0xffffffffu) break;
-      continue;  // every query taken was alone in its cell
-    }
+    // the next pending node of the lowest level
+    const bool on = lv != 0u;
+    const int l = on ? __ffs(lv) - 1 : 1;
+    const uint32_t word = mine[l * kStride];
+    __syncwarp();  // read by the whole group before any lane rewrites it
     uint32_t mask = 0, node = 0;
-    bool leaf = false;
-    if (active) {
-      // the next pending node of the lowest level
-      const int l = __ffs(lv) - 1;
-      const uint32_t word = mine[l * kTvThreads];
+    if (on) {
       const uint32_t rest = word & (word - 1u);
       node = (word >> 8) * kWide + (__ffs(word) - 1);
-      mine[l * kTvThreads] = rest;
+      mine[l * kStride] = rest;
       if (!(rest & 0xffu)) lv &= lv - 1u;
       mask = meet_mask(a.nodes + off[l] + node, qlo, qhi);
-      nt += kWide;
+      ++visits;
       // only children that hold a position in (p, cend)
       const int sh = kWideBits * (l - 1);
       const int lo = (int)((p + 1u) >> sh) - (int)(node * kWide);
       const int hi = (int)((cend - 1u) >> sh) - (int)(node * kWide);
-      mask &= (0xffu << min(max(lo, 0), 8)) & ((2u << min(hi, 7)) - 1u);
-      leaf = l == 1;
-      if (!leaf && mask) {
-        mine[(l - 1) * kTvThreads] = node << 8 | mask;
-        lv |= 1u << (l - 1);
-      }
+      mask &= (0xffu << min(max(lo, 0), 8)) & ((1u << min(max(hi + 1, 0), 8)) - 1u);
+      if (cend == 0u) mask = 0u;
     }
+    // the children that a query of the group meets
+    const uint32_t any = mask | __shfl_xor_sync(kFull, mask, 1);
+    if (on && l > 1 && any) {
+      mine[(l - 1) * kStride] = node << 8 | any;
+      lv |= 1u << (l - 1);
+    }
+    __syncwarp();
     // leaf nodes with boxes that meet go to the warp's buffer
-    const bool put = leaf && mask;
-    const unsigned v = __ballot_sync(0xffffffffu, put);
+    const bool put = on && l == 1 && mask;
+    const unsigned v = __ballot_sync(kFull, put);
     if (v) {
       if (put) {
         const int k = nent + __popc(v & lt);
@@ -492,6 +531,8 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
         __syncwarp();
         ntests += drain<kRefine>(a, buf, nent, we);  // exact box tests
         nent = 0;
+        // (read again rather than kept in registers across the drain)
+        ldg_box(a.sbox + p, qlo, qhi);
       }
     }
   }
@@ -501,24 +542,34 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
     chunk_fill_holes(we.s, a.starts, a.cap);
     if (!a.raw) chunk_fill_holes(we.e, a.ends, a.cap);
   }
+  // the block's totals, one atomic each where there is something to add
+  unsigned long long nt = (unsigned long long)visits * kWide;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nt += __shfl_down_sync(0xffffffffu, nt, o);
+  __shared__ unsigned long long sums[kTvWarps][4];
   if (lane == 0) {
-    atomicAdd(&a.ctr->node_tests, nt);
-    atomicAdd(&a.ctr->leaf_tests, ntests);
-    if (kRefine) {
-    } else if (a.raw) {
-      atomicAdd(&a.ctr->v_raw, we.s.count);
-    } else {
-      atomicAdd(&a.ctr->v_starts, we.s.count);
-      atomicAdd(&a.ctr->v_ends, we.e.count);
-    }
+    sums[w][0] = nt;
+    sums[w][1] = ntests;
+    sums[w][2] = we.s.count;
+    sums[w][3] = we.e.count;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    unsigned long long v = 0;
+#pragma unroll
+    for (int q = 0; q < kTvWarps; ++q) v += sums[q][threadIdx.x];
+    unsigned long long *to = threadIdx.x == 0   ? &a.ctr->node_tests
+                             : threadIdx.x == 1 ? &a.ctr->leaf_tests
+                             : threadIdx.x == 3 ? &a.ctr->v_ends
+                             : a.raw            ? &a.ctr->v_raw
+                                                : &a.ctr->v_starts;
+    if (v) atomicAdd(to, v);
   }
 }
 
 // persistent: as many blocks as fit on the GPU at once
 template <bool kRefine>
-static int launch_traverse(const TravArgs &a, cudaStream_t st) {
+static int launch_traverse(TravArgs &a, cudaStream_t st) {
   static int wave = 0;
   if (!wave) {
     int dev = 0, sms = 0, per_sm = 0;
@@ -530,6 +581,8 @@ static int launch_traverse(const TravArgs &a, cudaStream_t st) {
   // sorted boxes and nodes are read with 32-byte loads
   if ((reinterpret_cast<uintptr_t>(a.sbox) | reinterpret_cast<uintptr_t>(a.nodes)) & 31)
     return SCD_ERR_INTERNAL;
+  a.chunk = kMinChunk;
+  while (a.chunk < kMaxChunk && (int64_t)a.chunk * wave * kTvWarps < a.N) a.chunk *= 2;
   k_traverse<kRefine><<<(unsigned)wave, kTvThreads, 0, st>>>(a);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
@@ -581,7 +634,7 @@ int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   a.starts = s->d_starts.p;
   a.ends = s->d_ends.p;
   a.rawval = s->d_rawval.p;
-  a.cap = (unsigned long long)s->pair_cap;
+  a.cap = (uint32_t)std::min<int64_t>(s->pair_cap, 0xffffffffll - 2 * kMaxChunk);
   a.ctr = s->d_ctr.p;
   a.dkind = s->dkind;
   a.n_slabs = s->n_slabs;
