@@ -12,7 +12,8 @@ namespace scd {
 
 // One block takes 512 nodes of level k0 (the sorted boxes when k0 = 0) and
 // builds the three levels above them: 64 nodes, 8 nodes, one node.  The
-// boxes of its topmost node go to the next launch (k0 + 3), 1/512 of the size.  Bound
+// boxes of the topmost nodes go to the next launch (k0 + 3), 1/512 of the size,
+// or, where they fit one tile, to the last block to finish.  Bound
 // by the gather's loads: 32 bytes a box read at random (two 16-byte halves, a
 // sector each) and 32 + 4 written, 14 bytes of nodes.  With the neighbour
 // positions 0.73 ms for 17.4 M boxes (a binary radix tree with its gather and
@@ -36,6 +37,9 @@ struct TreeArgs {
   int k0;
   int64_t n;                       // boxes (a capacity when d_n is set)
   const unsigned long long *d_n;
+  // set: the levels above k0 + 3 fit one tile, and the last block to finish
+  // builds them (zero before and after the launch)
+  uint32_t *finish;
 };
 
 __device__ __forceinline__ float4 f4min(float4 a, float4 b) {
@@ -101,79 +105,105 @@ __device__ __forceinline__ void make_node(float4 &lo, float4 &hi, bool valid, Wi
   }
 }
 
+struct TreeSmem {
+  WideNode s1[kWide * kWide], s2[kWide], s3;
+  SBox u1[kWide * kWide], u2[kWide];
+};
+
+// The three levels above 512 nodes of level k0 (tile of them), whose boxes
+// are gathered by id (k0 = 0) or read from `in`; the topmost node's box goes
+// to `out`.
 template <bool kGather>
-__global__ void __launch_bounds__(kTreeThreads) k_tree(TreeArgs a) {
-  __shared__ WideNode s1[kWide * kWide], s2[kWide], s3;
-  __shared__ SBox u1[kWide * kWide], u2[kWide];
-  int64_t n = a.n;
-  if (a.d_n && *a.d_n < (unsigned long long)n) n = (int64_t)*a.d_n;
-  // nodes of level k0 and of the three above
-  const int s0 = kWideBits * a.k0;
-  const int64_t c0 = (n + (1ll << s0) - 1) >> s0, c1 = (c0 + 7) >> 3, c2 = (c1 + 7) >> 3,
-                c3 = (c2 + 7) >> 3;
+__device__ __forceinline__ void tree_tile(const TreeArgs &a, TreeSmem &sm, int k0, int64_t n,
+                                          int64_t tile, const SBox *in, SBox *out) {
+  // nodes of level k0 and of the two above
+  const int s0 = kWideBits * k0;
+  const int64_t c0 = (n + (1ll << s0) - 1) >> s0, c1 = (c0 + 7) >> 3, c2 = (c1 + 7) >> 3;
   const int tid = threadIdx.x;
-  for (int64_t tile = blockIdx.x; tile < c3; tile += gridDim.x) {
-    const int64_t i = tile * kTreeThreads + tid;
-    const bool valid = i < c0;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (valid) {
-      if (kGather) {
-        const uint32_t b = a.id[i];
-        lo = __ldg(a.lo + b);
-        hi = __ldg(a.hi + b);
-        a.sbox[i].lo = lo;
-        a.sbox[i].hi = hi;
-        a.sobj[i] = __ldg(a.obj + b);
-        // a box referenced from several cells: any copy will do, their data agree
-        if (a.posof) a.posof[b] = (uint32_t)i;
-        if (a.scell) a.scell[i] = (uint32_t)(a.keys[i] >> a.cell_shift);
-      } else {
-        lo = a.in[i].lo;
-        hi = a.in[i].hi;
-      }
+  const int64_t i = tile * kTreeThreads + tid;
+  const bool valid = i < c0;
+  float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+  if (valid) {
+    if (kGather) {
+      const uint32_t b = a.id[i];
+      lo = __ldg(a.lo + b);
+      hi = __ldg(a.hi + b);
+      a.sbox[i].lo = lo;
+      a.sbox[i].hi = hi;
+      a.sobj[i] = __ldg(a.obj + b);
+      // a box referenced from several cells: any copy will do, their data agree
+      if (a.posof) a.posof[b] = (uint32_t)i;
+      if (a.scell) a.scell[i] = (uint32_t)(a.keys[i] >> a.cell_shift);
+    } else {  // (past L1: other blocks may have written it in this launch)
+      lo = __ldcg(&in[i].lo);
+      hi = __ldcg(&in[i].hi);
     }
-    make_node(lo, hi, valid, &s1[tid >> 3]);
-    if ((tid & 7) == 0) {
-      u1[tid >> 3].lo = lo;
-      u1[tid >> 3].hi = hi;
+  }
+  make_node(lo, hi, valid, &sm.s1[tid >> 3]);
+  if ((tid & 7) == 0) {
+    sm.u1[tid >> 3].lo = lo;
+    sm.u1[tid >> 3].hi = hi;
+  }
+  __syncthreads();
+  // whole nodes out, 16 bytes a thread
+  auto store = [&](const WideNode *src, int level, int64_t first, int64_t count) {
+    uint4 *dst = reinterpret_cast<uint4 *>(a.nodes + a.lv.off[level] + first);
+    const uint4 *from = reinterpret_cast<const uint4 *>(src);
+    for (int k = tid; k < (int)count * 6; k += kTreeThreads) dst[k] = from[k];
+  };
+  store(sm.s1, k0 + 1, tile * 64, c1 - tile * 64 < 64 ? c1 - tile * 64 : 64);
+  if (k0 + 2 <= a.lv.levels) {
+    if (tid < kWide * kWide) {
+      lo = sm.u1[tid].lo;
+      hi = sm.u1[tid].hi;
+      make_node(lo, hi, tile * 64 + tid < c1, &sm.s2[tid >> 3]);
+      if ((tid & 7) == 0) {
+        sm.u2[tid >> 3].lo = lo;
+        sm.u2[tid >> 3].hi = hi;
+      }
     }
     __syncthreads();
-    // whole nodes out, 16 bytes a thread
-    auto store = [&](const WideNode *src, int level, int64_t first, int64_t count) {
-      uint4 *dst = reinterpret_cast<uint4 *>(a.nodes + a.lv.off[level] + first);
-      const uint4 *from = reinterpret_cast<const uint4 *>(src);
-      for (int k = tid; k < (int)count * 6; k += kTreeThreads) dst[k] = from[k];
-    };
-    store(s1, a.k0 + 1, tile * 64, c1 - tile * 64 < 64 ? c1 - tile * 64 : 64);
-    if (a.k0 + 2 <= a.lv.levels) {
-      if (tid < kWide * kWide) {
-        lo = u1[tid].lo;
-        hi = u1[tid].hi;
-        make_node(lo, hi, tile * 64 + tid < c1, &s2[tid >> 3]);
-        if ((tid & 7) == 0) {
-          u2[tid >> 3].lo = lo;
-          u2[tid >> 3].hi = hi;
-        }
-      }
-      __syncthreads();
-      store(s2, a.k0 + 2, tile * 8, c2 - tile * 8 < 8 ? c2 - tile * 8 : 8);
-    }
-    if (a.k0 + 3 <= a.lv.levels) {
-      if (tid < 32) {
-        // every eight lanes put together the same node
-        lo = u2[tid & 7].lo;
-        hi = u2[tid & 7].hi;
-        make_node(lo, hi, tile * 8 + (tid & 7) < c2, &s3);
-        if (tid == 0) {
-          a.out[tile].lo = lo;
-          a.out[tile].hi = hi;
-        }
-      }
-      __syncthreads();
-      store(&s3, a.k0 + 3, tile, 1);
-    }
-    __syncthreads();  // the next tile reuses the shared nodes
+    store(sm.s2, k0 + 2, tile * 8, c2 - tile * 8 < 8 ? c2 - tile * 8 : 8);
   }
+  if (k0 + 3 <= a.lv.levels) {
+    if (tid < 32) {
+      // every eight lanes put together the same node
+      lo = sm.u2[tid & 7].lo;
+      hi = sm.u2[tid & 7].hi;
+      make_node(lo, hi, tile * 8 + (tid & 7) < c2, &sm.s3);
+      if (tid == 0) {
+        out[tile].lo = lo;
+        out[tile].hi = hi;
+      }
+    }
+    __syncthreads();
+    store(&sm.s3, k0 + 3, tile, 1);
+  }
+  __syncthreads();  // the next tile reuses the shared nodes
+}
+
+template <bool kGather>
+__global__ void __launch_bounds__(kTreeThreads) k_tree(TreeArgs a) {
+  __shared__ TreeSmem sm;
+  __shared__ bool last;
+  int64_t n = a.n;
+  if (a.d_n && *a.d_n < (unsigned long long)n) n = (int64_t)*a.d_n;
+  const int s3 = kWideBits * (a.k0 + 3);
+  const int64_t tiles = (n + (1ll << s3) - 1) >> s3;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x)
+    tree_tile<kGather>(a, sm, a.k0, n, tile, a.in, a.out);
+  if (!a.finish) return;
+  // the last block to get here sees every block's topmost boxes
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(a.finish, 1u) == gridDim.x - 1u;
+    if (last) {
+      *a.finish = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (last && tiles > 0) tree_tile<false>(a, sm, a.k0 + 3, n, 0, a.out, a.out + tiles);
 }
 
 // Sorted positions of each box's previous and next segment of the same
@@ -212,14 +242,20 @@ static int launch_tree(TreeArgs a, SBox *nbox, cudaStream_t st) {
   if (a.n > kMaxTreeBoxes) return SCD_ERR_CAPACITY;
   a.lv = tree_levels(a.n);
   int64_t tiles = (a.n + kTreeThreads - 1) / kTreeThreads;
+  uint32_t *const finish = a.finish;
   a.in = nullptr;
   a.out = nbox;
   for (a.k0 = 0; a.k0 < a.lv.levels; a.k0 += 3) {
+    // one tile of topmost nodes (up to 2^18 boxes at the first launch, 2^27 at
+    // the second): the same launch builds the levels above them
+    const bool ends = a.k0 + 3 < a.lv.levels && tiles <= kTreeThreads;
+    a.finish = ends ? finish : nullptr;
     // with a device count, one resident wave loops over the tiles there are
     const unsigned grid = (unsigned)(a.d_n ? std::min<int64_t>(tiles, wave) : tiles);
     if (a.k0 == 0) k_tree<true><<<grid, kTreeThreads, 0, st>>>(a);
     else k_tree<false><<<grid, kTreeThreads, 0, st>>>(a);
     note_launch();
+    if (ends) break;
     a.in = a.out;
     a.out += tiles;
     tiles = (tiles + kTreeThreads - 1) / kTreeThreads;
@@ -249,6 +285,7 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
   a.scell = cells ? s->s_cell.p : nullptr;
   a.nodes = s->d_nodes.p;
   a.n = Nq;
+  a.finish = &s->d_ctr.p->tree_done;
   if (int rc = launch_tree(a, s->d_nbox.p, st)) return rc;
   const int bs = 256;
   k_neighbors<<<(unsigned)((Nq + bs - 1) / bs), bs, 0, st>>>(ids_sorted, s->d_obj.p, s->d_posof.p,
@@ -261,7 +298,8 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
 // boxes, their count on the device.
 int build_round_tree(const uint32_t *ids_sorted, const float4 *lo, const float4 *hi,
                      const uint32_t *obj, int64_t cap, const unsigned long long *d_M, SBox *sbox,
-                     uint32_t *sobj, WideNode *nodes, SBox *nbox, cudaStream_t st) {
+                     uint32_t *sobj, WideNode *nodes, SBox *nbox, DevCounters *ctr,
+                     cudaStream_t st) {
   TreeArgs a{};
   a.id = ids_sorted;
   a.lo = lo;
@@ -272,6 +310,7 @@ int build_round_tree(const uint32_t *ids_sorted, const float4 *lo, const float4 
   a.nodes = nodes;
   a.n = cap;
   a.d_n = d_M;
+  a.finish = &ctr->tree_done;
   return launch_tree(a, nbox, st);
 }
 

@@ -357,8 +357,9 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
   k_narrow_init<<<1, 32, 0, s->stream>>>(s->d_narrow.p);
   note_launch();
   if (n_pairs > 0) {
-    k_np_objects<<<(unsigned)((s->n + 255) / 256), 256, 0, s->stream>>>(s->d_par.p, s->n,
-                                                                         s->tick_s, obj);
+    // (FP64: one warp a block, spread over the SMs)
+    k_np_objects<<<(unsigned)((s->n + 31) / 32), 32, 0, s->stream>>>(s->d_par.p, s->n, s->tick_s,
+                                                                      obj);
     note_launch();
     static int per_sm = 0, sms = 0;
     if (!per_sm) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_narrow, kNpThreads, 0);

@@ -112,7 +112,10 @@ int launch_prepare_objects(scd_scene *s) {
   sa.n_bands = (int)s->band_fracs.size();
   sa.learned_k = s->step_kind == SCD_STEP_LEARNED ? s->d_learned.p : nullptr;
   sa.objT = s->n_scenes > 0 ? s->d_objT.p : nullptr;
-  int bs = 256;
+  // one warp a block: about 500 FP64 operations an object at two per SM and
+  // clock, so a few hundred objects must spread over many SMs (512 objects in
+  // blocks of 256: 17 us, of 32: 6)
+  int bs = 32;
   int64_t g = (s->n + bs - 1) / bs;
   k_prepare_objects<<<(unsigned)g, bs, 0, s->stream>>>(s->d_el.p, s->n, sa, s->d_par.p,
                                                         s->d_k.p, s->d_segcnt.p, s->d_ctr.p);
@@ -274,7 +277,7 @@ int launch_propagate(const scd_element *d_el, int64_t n, const uint32_t *obj, co
   ObjParams *par = (ObjParams *)dev_alloc(sizeof(ObjParams) * (size_t)n, st);
   if (!par) return SCD_ERR_OOM;
   int bs = 256;
-  k_prepare_params_only<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(d_el, n, par);
+  k_prepare_params_only<<<(unsigned)((n + 31) / 32), 32, 0, st>>>(d_el, n, par);
   if (m > 0) k_propagate<<<(unsigned)((m + bs - 1) / bs), bs, 0, st>>>(par, obj, t, m, out);
   cudaError_t e = cudaGetLastError();
   cudaStreamSynchronize(st);
@@ -363,10 +366,43 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const int64_t *in, i
   }
 }
 
+// The whole scan by one block, tile after tile: up to kScanSmall values one
+// launch of a few microseconds instead of three.
+constexpr int64_t kScanSmall = 8 * kScanTile;
+__global__ void __launch_bounds__(kScanThreads) k_scan_small(const int64_t *in, int64_t n,
+                                                             int64_t *out) {
+  int64_t carry = 0;
+  for (int64_t base = 0; base < n; base += kScanTile) {
+    int64_t v[kScanItems];
+    int64_t s = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      const int64_t idx = base + (int64_t)threadIdx.x * kScanItems + k;
+      v[k] = idx < n ? in[idx] : 0;
+      s += v[k];
+    }
+    int64_t tot;
+    int64_t ex = carry + block_scan_excl(s, tot);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      const int64_t idx = base + (int64_t)threadIdx.x * kScanItems + k;
+      if (idx < n) out[idx] = ex;
+      ex += v[k];
+    }
+    carry += tot;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
 int scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, DevBuf<int64_t> &tmp,
                        cudaStream_t st) {
   if (n <= 0) {
     cudaMemsetAsync(out, 0, sizeof(int64_t), st);
+    return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
+  }
+  if (n <= kScanSmall) {
+    k_scan_small<<<1, kScanThreads, 0, st>>>(in, n, out);
+    note_launch();
     return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
   }
   int64_t nb = (n + kScanTile - 1) / kScanTile;
@@ -440,7 +476,7 @@ extern "C" SCD_API int scd_propagate_noalloc(const scd_element *d_elems, int64_t
   const int bs = 256;
   // every entry the second kernel reads is written by the first, so the
   // array needs no clearing between calls
-  scd::k_prepare_params_only<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(d_elems, n, par);
+  scd::k_prepare_params_only<<<(unsigned)((n + 31) / 32), 32, 0, st>>>(d_elems, n, par);
   if (m > 0) scd::k_propagate<<<(unsigned)((m + bs - 1) / bs), bs, 0, st>>>(par, d_obj, d_t_s, m, d_out);
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }

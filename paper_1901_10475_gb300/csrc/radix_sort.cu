@@ -703,7 +703,9 @@ static int rs_cluster(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
 
 template <class K>
 static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long *d_n, int lo,
-                   int bits, SortScratch &sc, cudaStream_t st, const PairEmit *pe = nullptr) {
+                   int bits, SortScratch &sc, cudaStream_t st, const PairEmit *pe = nullptr,
+                   const uint32_t **vals_out = nullptr) {
+  if (vals_out) *vals_out = vals;
   if (!pe && (n <= 1 || bits <= lo)) return SCD_OK;
   if (pe && (n < 1 || bits <= lo || vals || sizeof(K) != 8)) return SCD_ERR_INTERNAL;
   if (n >= (1ll << 32) - 1) return SCD_ERR_CAPACITY;  // positions are 32-bit
@@ -786,7 +788,9 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
     K *t = ka; ka = kb; kb = t;
     uint32_t *tv = va; va = vb; vb = tv;
   }
-  if (passes & 1) {
+  if (vals_out) {
+    *vals_out = va;
+  } else if (passes & 1) {
     cudaMemcpyAsync(keys, ka, sizeof(K) * (size_t)n, cudaMemcpyDeviceToDevice, st);
     if (vals) cudaMemcpyAsync(vals, va, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st);
   }
@@ -873,8 +877,8 @@ int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, const unsigned lon
 
 int radix_sort_u64_dev(unsigned long long *keys, uint32_t *vals, int64_t n_cap,
                        const unsigned long long *d_n, int lo, int bits, SortScratch &sc,
-                       cudaStream_t st) {
-  return rs_impl<unsigned long long>(keys, vals, n_cap, d_n, lo, bits, sc, st);
+                       cudaStream_t st, const uint32_t **vals_out) {
+  return rs_impl<unsigned long long>(keys, vals, n_cap, d_n, lo, bits, sc, st, nullptr, vals_out);
 }
 
 }  // namespace scd

@@ -59,21 +59,21 @@ constexpr int kRfThreads = 256;
 constexpr int kRfMaxRounds = 64;
 // object indices take 20 bits and ticks 24 in a packed candidate key
 constexpr int64_t kRfMaxObjects = 1ll << 20;
-// device state words: tick candidates, next intervals, error bits, unique
-// candidates, witnesses, this round's intervals, the largest next-round
-// count asked for
-enum {
-  RF_NCAND = 0, RF_NNEXT = 1, RF_ERR = 2, RF_NUNIQ = 3, RF_NWIT = 4, RF_M = 5, RF_OVER = 6,
-  RF_LMAX = 7, RF_WORDS = 8
-};
+// device state words: tick candidates, error bits, unique candidates,
+// witnesses, the longest first interval
+enum { RF_NCAND = 0, RF_ERR = 1, RF_NUNIQ = 2, RF_NWIT = 3, RF_LMAX = 4, RF_WORDS = 8 };
+// ... followed by the intervals asked for by every round (kRfMaxRounds of
+// them, then the ones left after the last)
+constexpr int kRfCounts = kRfMaxRounds + 1;
 // the rounds' 4D curve keys: 10 bits per axis, time weighed 4x against
 // space (24 h catalog rounds 552 -> 522 ms against equal weights; 12-bit axes
 // with weight 8, the screen's choice, 519 ms but slower on small rounds)
 constexpr int kRfCurveBits = 10;
 constexpr float kRfTimeScale = 4.0f;
 
-__device__ __forceinline__ int64_t rf_count(const unsigned long long *state, int64_t cap) {
-  const unsigned long long m = state[RF_M];
+// a round's intervals: those asked for, at most the capacity
+__device__ __forceinline__ int64_t rf_count(const unsigned long long *asked, int64_t cap) {
+  const unsigned long long m = *asked;
   return m < (unsigned long long)cap ? (int64_t)m : cap;
 }
 
@@ -108,12 +108,8 @@ __global__ void k_rf_start_count(const ObjParams *__restrict__ par, int64_t n, i
 __global__ void k_rf_init_start(const ObjParams *__restrict__ par, int64_t n, int32_t T,
                                 double unit, const int64_t *__restrict__ off, int64_t cap,
                                 uint32_t *obj, int32_t *t0, int32_t *t1,
-                                unsigned long long *state) {
-  const int64_t total = off[n];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    state[RF_M] = (unsigned long long)(total < cap ? total : cap);
-    if (total > cap) atomicMax(&state[RF_OVER], (unsigned long long)total);
-  }
+                                unsigned long long *asked) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *asked = (unsigned long long)off[n];
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; o < n; o += nw) {
@@ -129,9 +125,9 @@ __global__ void k_rf_init_start(const ObjParams *__restrict__ par, int64_t n, in
 }
 
 __global__ void k_rf_init(int64_t n, int32_t T, uint32_t *obj, int32_t *t0, int32_t *t1,
-                          unsigned long long *state) {
+                          unsigned long long *asked) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) state[RF_M] = (unsigned long long)n;
+  if (i == 0) *asked = (unsigned long long)n;
   if (i >= n) return;
   obj[i] = (uint32_t)i;
   t0[i] = 0;
@@ -144,15 +140,14 @@ struct RfBoxArgs {
   const uint32_t *obj;
   const int32_t *t0, *t1;
   int64_t cap;
-  const unsigned long long *state;
-  unsigned long long *round_count;  // this round's entry of the per-round counts
+  const unsigned long long *asked;  // the round's intervals
   double tick_s;                // the length of one unit of t0, t1 [s]
-  const DevCounters *ctr;       // the scene's extent (key frame)
+  DevCounters *ctr;             // the scene's extent (key frame); the query queue
   int64_t Tf;                   // the time extent of the key frame [units]
   float split_km;
   float4 *lo, *hi;
   unsigned long long *key;
-  uint32_t *idx;
+  uint32_t *idx, *flags;
   unsigned long long *err;
 };
 
@@ -181,12 +176,16 @@ __device__ __forceinline__ void rf_box(const RfBoxArgs &a, int64_t i) {
   k |= (unsigned long long)split_bit(L, H, a.split_km) << (4 * kRfCurveBits);
   a.key[i] = k;
   a.idx[i] = (uint32_t)i;
+  a.flags[i] = 0;
 }
 
-__global__ void __launch_bounds__(kRfThreads) k_rf_boxes(RfBoxArgs a) {
-  const int64_t M = rf_count(a.state, a.cap);
+// (blocks of two warps: the FP64 work of a nearly empty round spreads over
+// many SMs)
+constexpr int kRfBoxThreads = 64;
+__global__ void __launch_bounds__(kRfBoxThreads) k_rf_boxes(RfBoxArgs a) {
+  const int64_t M = rf_count(a.asked, a.cap);
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i0 == 0) *a.round_count = (unsigned long long)M;
+  if (i0 == 0) a.ctr->work_next = 0;  // the round's traversal starts from its first query
   for (int64_t i = i0; i < M; i += (int64_t)gridDim.x * blockDim.x) rf_box(a, i);
 }
 
@@ -217,8 +216,8 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_split(const uint32_t *__restr
                                                          const uint32_t *__restrict__ flags,
                                                          int64_t cap, uint32_t *nobj,
                                                          int32_t *nt0, int32_t *nt1,
-                                                         unsigned long long *state) {
-  const int64_t M = rf_count(state, cap);
+                                                         unsigned long long *asked) {
+  const int64_t M = rf_count(asked, cap);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // whole warps walk the intervals (rf_claim needs every lane)
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < M;
@@ -236,7 +235,7 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_split(const uint32_t *__restr
         need = a1 > a0 ? 2u : ((f & kRfHitLong) ? 1u : 0u);
       }
     }
-    const unsigned long long q = rf_claim(&state[RF_NNEXT], need);
+    const unsigned long long q = rf_claim(asked + 1, need);
     // every slot below the capacity is written, also by the lane whose two
     // slots straddle it: a round cut short still reads all of its intervals
     if (need == 0 || q >= (unsigned long long)cap) continue;
@@ -259,14 +258,14 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_split_cont(const uint32_t *__
                                                               const uint32_t *__restrict__ flags,
                                                               int64_t cap, uint32_t *nobj,
                                                               int32_t *nt0, int32_t *nt1,
-                                                              unsigned long long *state) {
-  const int64_t M = rf_count(state, cap);
+                                                              unsigned long long *asked) {
+  const int64_t M = rf_count(asked, cap);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < M;
        base += stride) {
     const int64_t i = base + (threadIdx.x & 31);
     const uint32_t need = (i < M && (flags[i] & kRfHit)) ? 2u : 0u;
-    const unsigned long long q = rf_claim(&state[RF_NNEXT], need);
+    const unsigned long long q = rf_claim(asked + 1, need);
     if (need == 0 || q >= (unsigned long long)cap) continue;  // (slots below cap all written)
     const int32_t k = t0[i];
     nobj[q] = obj[i];
@@ -286,13 +285,12 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_trace(const float4 *__restric
                                                          const float4 *__restrict__ hi,
                                                          const uint32_t *__restrict__ obj,
                                                          int64_t cap,
-                                                         const unsigned long long *state,
                                                          const unsigned long long *rounds, int r,
                                                          float4 *tlo, float4 *thi,
                                                          uint32_t *tobj, int64_t tcap) {
-  const int64_t M = rf_count(state, cap);
+  const int64_t M = rf_count(rounds + r, cap);
   unsigned long long off = 0;
-  for (int q = 0; q < r; ++q) off += rounds[q];
+  for (int q = 0; q < r; ++q) off += (unsigned long long)rf_count(rounds + q, cap);
   if (off + (unsigned long long)M > (unsigned long long)tcap) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -300,15 +298,6 @@ __global__ void __launch_bounds__(kRfThreads) k_rf_trace(const float4 *__restric
     thi[off + i] = hi[i];
     tobj[off + i] = obj[i];
   }
-}
-
-// the next round's count becomes the current one (at most the capacity; the
-// largest count asked for is kept)
-__global__ void k_rf_advance(unsigned long long *state, int64_t cap) {
-  const unsigned long long nx = state[RF_NNEXT];
-  if (nx > state[RF_OVER]) state[RF_OVER] = nx;
-  state[RF_M] = nx < (unsigned long long)cap ? nx : (unsigned long long)cap;
-  state[RF_NNEXT] = 0;
 }
 
 // distinct span keys (sorted) appended to out (in any order)
@@ -377,7 +366,7 @@ struct RfBuffers {
   DevBuf<uint32_t> obj[2], idx, flags, sobj;
   DevBuf<int32_t> t0[2], t1[2], first;
   DevBuf<float4> lo, hi;
-  DevBuf<unsigned long long> key, cand, state, wkey, rounds;
+  DevBuf<unsigned long long> key, cand, state, wkey;
   DevBuf<SBox> sbox, nbox;
   DevBuf<WideNode> nodes;
   DevBuf<DevCounters> ctr;
@@ -403,7 +392,7 @@ struct RfBuffers {
     }
     idx.release(st); flags.release(st); sobj.release(st); first.release(st);
     lo.release(st); hi.release(st); key.release(st); cand.release(st); state.release(st);
-    wkey.release(st); rounds.release(st); sbox.release(st); nbox.release(st); nodes.release(st);
+    wkey.release(st); sbox.release(st); nbox.release(st); nodes.release(st);
     ctr.release(st); sort_err.release(st); pairs.release(st);
     wit.release(st); span.release(st); tlo.release(st); thi.release(st); tobj.release(st);
     scnt.release(st); soff.release(st); stmp.release(st);
@@ -494,8 +483,8 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int r
                     int levels) {
   cudaStream_t st = B.st;
   const int64_t n = s->n;
-  if (cudaMemsetAsync(B.state.p, 0, sizeof(unsigned long long) * RF_WORDS, st) != cudaSuccess ||
-      cudaMemsetAsync(B.rounds.p, 0, sizeof(unsigned long long) * kRfMaxRounds, st) !=
+  unsigned long long *const asked = B.state.p + RF_WORDS;
+  if (cudaMemsetAsync(B.state.p, 0, sizeof(unsigned long long) * (RF_WORDS + kRfCounts), st) !=
           cudaSuccess ||
       cudaMemsetAsync(B.sort_err.p, 0, sizeof(uint32_t), st) != cudaSuccess ||
       cudaMemsetAsync(B.ctr.p, 0, sizeof(DevCounters), st) != cudaSuccess ||
@@ -505,72 +494,77 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int r
   const bool cont = levels >= 0;
   const double T_s = (double)s->T * s->tick_s;
   if (cont)
-    k_rf_init<<<grid_of(n), kRfThreads, 0, st>>>(n, 1, B.obj[0].p, B.t0[0].p, B.t1[0].p,
-                                                  B.state.p);
+    k_rf_init<<<grid_of(n), kRfThreads, 0, st>>>(n, 1, B.obj[0].p, B.t0[0].p, B.t1[0].p, asked);
   else
     k_rf_init_start<<<wave_of(32 * n), kRfThreads, 0, st>>>(s->d_par.p, n, (int32_t)s->T,
                                                              rf_start_unit(s), B.soff.p, cap,
                                                              B.obj[0].p, B.t0[0].p, B.t1[0].p,
-                                                             B.state.p);
+                                                             asked);
   note_launch();
   const float split = split_of(s->tune);
   const int kb = 4 * kRfCurveBits + (split != 0.0f);
-  unsigned long long *dM = B.state.p + RF_M;
   const int nr = cont ? levels + 1 : rounds;
   int cur = 0;
   for (int r = 0; r < nr; ++r) {
     const int nx = cur ^ 1;
+    unsigned long long *const dM = asked + r;  // this round's intervals; the next one's follow
     // the unit of t0, t1 and the time extent of the key frame
     const double unit = cont ? ldexp(T_s, -r) : s->tick_s;
     const int64_t Tf = cont ? (1ll << r) : s->T;
     RfBoxArgs ba{s->d_par.p, s->box_mode, B.obj[cur].p, B.t0[cur].p, B.t1[cur].p, cap,
-                 B.state.p, B.rounds.p + r, unit, B.ctr.p, Tf, split, B.lo.p, B.hi.p,
-                 B.key.p, B.idx.p, B.state.p + RF_ERR};
-    k_rf_boxes<<<wave_of(cap), kRfThreads, 0, st>>>(ba);
+                 dM, unit, B.ctr.p, Tf, split, B.lo.p, B.hi.p, B.key.p, B.idx.p, B.flags.p,
+                 B.state.p + RF_ERR};
+    k_rf_boxes<<<wave_of(cap) * (kRfThreads / kRfBoxThreads), kRfBoxThreads, 0, st>>>(ba);
     note_launch();
     if (B.tcap > 0) {
-      k_rf_trace<<<wave_of(cap), kRfThreads, 0, st>>>(B.lo.p, B.hi.p, B.obj[cur].p, cap, B.state.p,
-                                                     B.rounds.p, r, B.tlo.p, B.thi.p, B.tobj.p,
-                                                     B.tcap);
+      k_rf_trace<<<wave_of(cap), kRfThreads, 0, st>>>(B.lo.p, B.hi.p, B.obj[cur].p, cap, asked, r,
+                                                     B.tlo.p, B.thi.p, B.tobj.p, B.tcap);
       note_launch();
     }
-    int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, sort_key_skip(kb, cap), kb, B.sc, st);
+    const uint32_t *idx = nullptr;  // (by the keys' top 40 bits: five passes)
+    int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, kb - 4 * kRfCurveBits, kb, B.sc, st,
+                                &idx);
     if (rc != SCD_OK) return rc;
-    rc = build_round_tree(B.idx.p, B.lo.p, B.hi.p, B.obj[cur].p, cap, dM, B.sbox.p, B.sobj.p,
-                          B.nodes.p, B.nbox.p, st);
+    rc = build_round_tree(idx, B.lo.p, B.hi.p, B.obj[cur].p, cap, dM, B.sbox.p, B.sobj.p,
+                          B.nodes.p, B.nbox.p, B.ctr.p, st);
     if (rc != SCD_OK) return rc;
-    // the flags, and the traversal's counters (its error bits, which follow
-    // them, stay set across the rounds)
-    if (cudaMemsetAsync(B.flags.p, 0, sizeof(uint32_t) * (size_t)cap, st) != cudaSuccess ||
-        cudaMemsetAsync(B.ctr.p, 0, offsetof(DevCounters, trav_flags), st) != cudaSuccess)
-      return SCD_ERR_CUDA;
     const int spans = cont && r == levels;
-    rc = traverse_round(B.nodes.p, B.sbox.p, B.sobj.p, B.idx.p, cap, dM, Tf, B.ctr.p, B.flags.p,
+    rc = traverse_round(B.nodes.p, B.sbox.p, B.sobj.p, idx, cap, dM, Tf, B.ctr.p, B.flags.p,
                         B.cand.p, B.state.p + RF_NCAND, (unsigned long long)ccap, spans, st);
     if (rc != SCD_OK) return rc;
     if (spans) break;
     if (cont)
       k_rf_split_cont<<<wave_of(cap), kRfThreads, 0, st>>>(B.obj[cur].p, B.t0[cur].p, B.flags.p,
                                                           cap, B.obj[nx].p, B.t0[nx].p,
-                                                          B.t1[nx].p, B.state.p);
+                                                          B.t1[nx].p, dM);
     else
       k_rf_split<<<wave_of(cap), kRfThreads, 0, st>>>(B.obj[cur].p, B.t0[cur].p, B.t1[cur].p,
                                                      B.flags.p, cap, B.obj[nx].p, B.t0[nx].p,
-                                                     B.t1[nx].p, B.state.p);
-    k_rf_advance<<<1, 1, 0, st>>>(B.state.p, cap);
-    note_launch(2);
+                                                     B.t1[nx].p, dM);
+    note_launch();
     cur = nx;
   }
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
 
-// the rounds' sizes and the state words, after the queue
-static int rf_collect(RfBuffers &B, unsigned long long h[RF_WORDS],
-                      unsigned long long *round_counts) {
-  if (cudaMemcpyAsync(round_counts, B.rounds.p, sizeof(unsigned long long) * kRfMaxRounds,
-                      cudaMemcpyDeviceToHost, B.st) != cudaSuccess)
+// The state words after the queue, the intervals of every round (at most the
+// capacity), and over all rounds the most asked for.
+static int rf_collect(RfBuffers &B, int64_t cap, int nr, unsigned long long h[RF_WORDS],
+                      unsigned long long *round_counts, unsigned long long &most,
+                      unsigned long long &left) {
+  unsigned long long w[RF_WORDS + kRfCounts];
+  if (cudaMemcpyAsync(w, B.state.p, sizeof(w), cudaMemcpyDeviceToHost, B.st) != cudaSuccess ||
+      cudaStreamSynchronize(B.st) != cudaSuccess)
     return SCD_ERR_CUDA;
-  return rf_read_state(B, h);
+  std::copy(w, w + RF_WORDS, h);
+  most = 0;
+  for (int r = 0; r < kRfCounts; ++r) {
+    most = std::max(most, w[RF_WORDS + r]);
+    if (r < kRfMaxRounds)
+      round_counts[r] = std::min<unsigned long long>(w[RF_WORDS + r], (unsigned long long)cap);
+  }
+  left = w[RF_WORDS + nr];
+  return SCD_OK;
 }
 
 // The rounds' queue captured as one CUDA graph, replayed while the call's
@@ -617,7 +611,8 @@ static void rf_key(const scd_scene *s, const RfBuffers &B, int64_t cap, int64_t 
 // eagerly
 static int rf_rounds(scd_scene *s, RfBuffers &B, RfCache *gc, int64_t cap, int64_t ccap,
                      int rounds, int levels, unsigned long long h[RF_WORDS],
-                     unsigned long long *round_counts) {
+                     unsigned long long *round_counts, unsigned long long &most,
+                     unsigned long long &left) {
   int64_t k[11];
   rf_key(s, B, cap, ccap, rounds, levels, k);
   if (gc && gc->exec && memcmp(k, gc->key, sizeof(k)) == 0) {
@@ -632,7 +627,7 @@ static int rf_rounds(scd_scene *s, RfBuffers &B, RfCache *gc, int64_t cap, int64
     int rc = rf_queue(s, B, cap, ccap, rounds, levels);
     if (rc != SCD_OK) return rc;
   }
-  return rf_collect(B, h, round_counts);
+  return rf_collect(B, cap, levels >= 0 ? levels + 1 : rounds, h, round_counts, most, left);
 }
 
 // capture the queue of a shape that has just run eagerly (nothing is
@@ -683,10 +678,11 @@ namespace scd {
 // its next call.
 // Discrete rounds (levels < 0) set `rounds` from their first intervals.
 static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int levels,
-                  unsigned long long h[RF_WORDS], unsigned long long *round_counts) {
+                  unsigned long long h[RF_WORDS], unsigned long long *round_counts,
+                  unsigned long long &left) {
   cudaStream_t st = B.st;
-  if (!B.state.ensure(RF_WORDS, st) || !B.sort_err.ensure(1, st) ||
-      !B.rounds.ensure(kRfMaxRounds, st) || !B.ctr.ensure(1, st))
+  if (!B.state.ensure(RF_WORDS + kRfCounts, st) || !B.sort_err.ensure(1, st) ||
+      !B.ctr.ensure(1, st))
     return SCD_ERR_OOM;
   B.sc.err = B.sort_err.p;
   B.sc_post.err = B.sort_err.p;
@@ -700,11 +696,12 @@ static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int leve
   int64_t ccap = std::max<int64_t>(s->rf_ccap, 1 << 16);
   for (int attempt = 0; attempt < 8; ++attempt) {
     if (!B.size(cap, ccap)) return SCD_ERR_OOM;
-    int rc = rf_rounds(s, B, gc, cap, ccap, rounds, levels, h, round_counts);
+    unsigned long long most = 0;
+    int rc = rf_rounds(s, B, gc, cap, ccap, rounds, levels, h, round_counts, most, left);
     if (rc != SCD_OK) return rc;
     bool again = false;
-    if (h[RF_OVER] > (unsigned long long)cap) {
-      cap = (int64_t)std::max<unsigned long long>(2ull * (unsigned long long)cap, 2ull * h[RF_OVER]);
+    if (most > (unsigned long long)cap) {
+      cap = (int64_t)std::max<unsigned long long>(2ull * (unsigned long long)cap, 2ull * most);
       again = true;
     }
     if (h[RF_NCAND] > (unsigned long long)ccap) {
@@ -762,7 +759,8 @@ extern "C" SCD_API int scd_refine_witnesses(scd_scene *s, scd_witness *host_out,
   // interval
   int nr = 0;
   unsigned long long h[RF_WORDS], rc_[kRfMaxRounds];
-  int rc = rf_run(s, B, &gc, nr, -1, h, rc_);
+  unsigned long long left = 0;
+  int rc = rf_run(s, B, &gc, nr, -1, h, rc_, left);
   if (rc != SCD_OK) return rc;
   int r = 0;
   while (r < nr && rc_[r] > 0) {
@@ -770,7 +768,7 @@ extern "C" SCD_API int scd_refine_witnesses(scd_scene *s, scd_witness *host_out,
     ++r;
   }
   if (rounds) *rounds = r;
-  if (h[RF_M] > 0) return SCD_ERR_INTERNAL;  // more rounds than the halvings allow
+  if (left > 0) return SCD_ERR_INTERNAL;  // more rounds than the halvings allow
   if (h[RF_ERR]) return SCD_ERR_KEPLER_NOCONV;
   const int64_t ncand = (int64_t)h[RF_NCAND];
   // distinct tick candidates, then Alg 1's test at each tick
@@ -798,21 +796,19 @@ extern "C" SCD_API int scd_refine_witnesses(scd_scene *s, scd_witness *host_out,
       note_launch();
     }
   }
+  // the sorts' error bit and, where they fit, the witnesses: one wait
   uint32_t serr = 0;
   if (cudaMemcpyAsync(&serr, B.sort_err.p, sizeof(serr), cudaMemcpyDeviceToHost, st) !=
           cudaSuccess ||
+      (nw > 0 && nw <= cap &&
+       cudaMemcpyAsync(host_out, B.wit.p, sizeof(scd_witness) * (size_t)nw,
+                       cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return SCD_ERR_CUDA;
   if (serr) return SCD_ERR_TIMEOUT;
   s->last_launches = launch_count() - mark;
   *n_out = nw;
-  if (nw > cap) return SCD_ERR_BUFFER_TOO_SMALL;
-  if (nw > 0 &&
-      (cudaMemcpyAsync(host_out, B.wit.p, sizeof(scd_witness) * (size_t)nw, cudaMemcpyDeviceToHost,
-                       st) != cudaSuccess ||
-       cudaStreamSynchronize(st) != cudaSuccess))
-    return SCD_ERR_CUDA;
-  return SCD_OK;
+  return nw > cap ? SCD_ERR_BUFFER_TOO_SMALL : SCD_OK;
 }
 
 namespace scd {
@@ -836,7 +832,8 @@ extern "C" SCD_API int scd_refine_continuous(scd_scene *s, double eps_s, scd_spa
   RfBuffers &B = gc.B;
   unsigned long long h[RF_WORDS], rc_[kRfMaxRounds];
   int nr = 0;
-  int rc = rf_run(s, B, &gc, nr, L, h, rc_);
+  unsigned long long left = 0;
+  int rc = rf_run(s, B, &gc, nr, L, h, rc_, left);
   if (rc != SCD_OK) return rc;
   int r = 0;
   while (r <= L && rc_[r] > 0) {
@@ -896,7 +893,8 @@ extern "C" SCD_API int scd_refine_trace(scd_scene *s, double eps_s, float *lo4, 
       !B.tobj.ensure((size_t)B.tcap, st))
     return SCD_ERR_OOM;
   unsigned long long h[RF_WORDS], rc_[kRfMaxRounds];
-  int rc = rf_run(s, B, nullptr, nr, L, h, rc_);
+  unsigned long long left = 0;
+  int rc = rf_run(s, B, nullptr, nr, L, h, rc_, left);
   if (rc != SCD_OK) return rc;
   const int nrounds = L >= 0 ? L + 1 : nr;
   int r = 0;

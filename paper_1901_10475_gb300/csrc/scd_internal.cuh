@@ -70,7 +70,7 @@ struct DevCounters {
   unsigned long long n_boxes;      // seg_off[n]
   unsigned long long refs_total;   // references of the last decomposed build
   unsigned int sort_flags;         // ERR_SORT (set by any sort since the box build)
-  unsigned int pad1;
+  unsigned int tree_done;          // blocks finished of a tree launch (0 between launches)
 };
 
 // The 4D box hierarchy: an implicit 8-wide tree over the sorted boxes.  Node
@@ -404,9 +404,12 @@ int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaSt
 // in an unspecified order.
 int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, const unsigned long long *d_n,
                          int lo, int bits, SortScratch &sc, const PairEmit &pe, cudaStream_t st);
+// vals_out: only the sorted values are wanted; set to where they are (vals or
+// the scratch, by the number of passes; the keys are left in any order), which
+// saves the copy back of an odd number of passes over the whole capacity.
 int radix_sort_u64_dev(unsigned long long *keys, uint32_t *vals, int64_t n_cap,
                        const unsigned long long *d_n, int lo, int bits, SortScratch &sc,
-                       cudaStream_t st);
+                       cudaStream_t st, const uint32_t **vals_out = nullptr);
 
 // Run starts carry their last tick below the (i, j, first tick) key when
 // both fit in 64 bits and the all-ones tick field is free to tag open runs
@@ -581,7 +584,8 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
 // the same for one refinement round (up to cap boxes, their count on the device)
 int build_round_tree(const uint32_t *ids_sorted, const float4 *lo, const float4 *hi,
                      const uint32_t *obj, int64_t cap, const unsigned long long *d_M, SBox *sbox,
-                     uint32_t *sobj, WideNode *nodes, SBox *nbox, cudaStream_t st);
+                     uint32_t *sobj, WideNode *nodes, SBox *nbox, DevCounters *ctr,
+                     cudaStream_t st);
 // node boxes between the tree build's launches, for up to cap boxes
 int64_t tree_scratch_boxes(int64_t cap);
 // decomposed screen: references, their sort, the tree and each cell's end
