@@ -36,7 +36,7 @@
 
 namespace scd {
 
-constexpr int kNpThreads = 256, kNpBlocksPerSm = 3;
+constexpr int kNpThreads = 256, kNpBlocksPerSm = 4;
 // margin of the FP64 skip bound [km] (the FP64 propagation is good to
 // 1e-7 km)
 constexpr double kNpMarginKm = 1e-5;
@@ -88,6 +88,7 @@ struct NarrowArgs {
   int32_t *first;   // per candidate, may be null
   uint32_t *count;  // per candidate, may be null
   unsigned long long *state;
+  unsigned claim;   // candidates a warp takes per atomic
 };
 
 // The velocity bound: v = (B cos E - A sin E) n / (1 - e cos E) changes by
@@ -160,27 +161,40 @@ __device__ __forceinline__ float mean_anomaly32(const float4 m, float tf) {
 }
 
 // FP32 position [km] and velocity [km/s] at tick t with bounds of their
-// errors.  The Newton steps start as the FP32 stage of kepler_E_sc and use
-// the fast hardware sine, cosine and division: their accuracy does not
-// matter, because the bounds come from the residual of Kepler's equation at
-// the final E, evaluated with the accurate sincosf (within 2 ulp).
+// errors.  Newton's method with the fast hardware sine and cosine (within 4.3e-7
+// on [-pi, pi], where E lies) and division; a correction d of at most
+// kNpNewton leaves the next one below 1.5e-7 (e d^2 / 2 (1 - e) at e <= 0.75;
+// for larger e the residual shows what is left), so it is the last: the sine
+// and cosine of the corrected E come from those before it to second order (the
+// third is below 5e-12), together within 7e-7 of the true ones.  The error
+// bounds take the residual of Kepler's equation at the result; their
+// allowances, kNpResidualSlack rad and 4e-6 a of the position, are four times
+// what the sine's error and the rounding of the terms amount to.
+constexpr float kNpNewton = 3e-4f;
+
 __device__ __forceinline__ void pv32(const NpTick &o, float tf, float x[3], float v[3],
                                      float &perr, float &verr) {
   const float Mf = mean_anomaly32(o.m, tf), ef = o.b.w;
-  float E = (ef <= 0.5f) ? Mf + ef * sinf(Mf)
-                         : Mf + 0.85f * ef * (sinf(Mf) >= 0.f ? 1.f : -1.f);
-  for (int it = 0; it < kFp32Steps; ++it) {
-    const float d = __fdividef(E - ef * __sinf(E) - Mf, 1.0f - ef * __cosf(E));
-    E -= d;
-    if (fabsf(d) <= 1e-6f) break;
+  float E = (ef <= 0.5f) ? fmaf(ef, __sinf(Mf), Mf) : Mf + copysignf(0.85f * ef, Mf);
+  float s = 0.f, c = 1.f, d = 0.f;
+  bool last = false;
+  for (int it = 0; it <= kFp32Steps && !last; ++it) {
+    __sincosf(E, &s, &c);
+    d = __fdividef(E - ef * s - Mf, 1.0f - ef * c);
+    last = fabsf(d) <= kNpNewton;
+    if (!last && it < kFp32Steps) E -= d;
   }
-  float s, c;
-  sincosf(E, &s, &c);
+  if (last) {
+    const float h = 0.5f * d * d, s0 = s;
+    E -= d;
+    s = fmaf(-d, c, fmaf(-h, s, s));
+    c = fmaf(d, s0, fmaf(-h, c, c));
+  }
   const float r = fabsf(E - ef * s - Mf) + kNpResidualSlack;
   perr = fmaf(o.err.x, r, o.err.y);
   verr = fmaf(o.err.z, r, o.err.w);
   const float ce = c - ef;
-  const float edot = o.a.w / (1.0f - ef * c);
+  const float edot = __fdividef(o.a.w, 1.0f - ef * c);
   const float A[3] = {o.a.x, o.a.y, o.a.z}, B[3] = {o.b.x, o.b.y, o.b.z};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -195,6 +209,7 @@ struct NpLane {
   int32_t t = 0, thi = 0;  // ticks (T < 2^24)
   uint32_t oi = 0, oj = 0, cnt = 0;
   int32_t f = -1;
+  bool shared = false;  // the candidate's interval is split over several lanes
   float Rf = 0.f, slack = 0.f, V = 0.f, Acc = 0.f;  // r_i + r_j [km], decision slack, skip bounds
 };
 
@@ -246,15 +261,23 @@ __device__ __forceinline__ void np_tick(const NarrowArgs &a, NpLane &L,
   } else if (D > 0.f) {
     // the largest s with min(V s, w s + Acc s^2 / 2) < D, in whole ticks
     const float wm = w + wi + wj + 1e-5f;
-    const float s1 = D / L.V;
-    const float s2 = 2.f * D / (wm + sqrtf(wm * wm + 2.f * L.Acc * D));
+    float root;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(wm, wm, 2.f * L.Acc * D)));
+    const float s1 = __fdividef(D, L.V);
+    const float s2 = __fdividef(2.f * D, wm + root);
     const float ks = floorf(fmaxf(s1, s2) * a.inv_tick * kNpSkipShrink);
     if (ks >= 1.f) next = L.t + 1 + (int32_t)fminf(ks, (float)(L.thi - L.t));
   }
   L.t = next;
   if (L.t > L.thi) {
-    if (a.first) a.first[L.q] = L.f;
-    if (a.count) a.count[L.q] = L.cnt;
+    if (!L.shared) {
+      if (a.first) a.first[L.q] = L.f;
+      if (a.count) a.count[L.q] = L.cnt;
+    } else {  // (-1, no witness, is the largest first tick as an unsigned word)
+      if (a.first && L.f >= 0)
+        atomicMin(reinterpret_cast<unsigned *>(a.first) + L.q, (unsigned)L.f);
+      if (a.count && L.cnt) atomicAdd(a.count + L.q, L.cnt);
+    }
     if (L.f >= 0)
       atomicMin(&a.state[NP_EARLIEST],
                 ((unsigned long long)L.f << 32) | (unsigned long long)L.q);
@@ -262,29 +285,52 @@ __device__ __forceinline__ void np_tick(const NarrowArgs &a, NpLane &L,
   }
 }
 
+// candidates a warp claims per atomic at most (a lane takes the next one of
+// them every second step or so); short lists are dealt out 32 at a time
+constexpr unsigned kNpClaim = 256, kNpMinClaim = 32;
+// ticks left of an interval worth splitting (24 h INTERVAL candidates: never
+// 1.72 ms, from 128 ticks 1.13, 32 0.80, 16 0.77)
+constexpr int32_t kNpSplitTicks = 16;
+
 // Persistent: every lane holds one candidate and walks its ticks; lanes that
-// finish claim the next candidates (one atomic per warp and refill), so
-// consecutive lanes share object i and its constants stay in L1.  Claims run
-// from the end of the list: candidates of the highest object indices, which
-// in catalog order are the eccentric and geosynchronous orbits with the
-// longest intervals, start first instead of forming a tail.
+// finish take the next ones of their warp's claim, so consecutive lanes share
+// object i and its constants stay in L1.  Claims run from the end of the list:
+// candidates of the highest object indices, which in catalog order are the
+// eccentric and geosynchronous orbits with the longest intervals, start first.
+// Bound by instruction issue: two FP32 Kepler solves a tick, 1.4 ticks a
+// candidate.  24 h catalog screen (164 M candidates, 229 M ticks): one Newton
+// correction with the fast sine and cosine instead of two or three and the
+// accurate ones, claims of 256 candidates instead of one atomic a step, and four
+// blocks of 64 registers instead of three of 76 took it from 6.1 to 3.4 ms (5
+// blocks spill: 3.9), sharing the last long intervals to 3.1; INTERVAL
+// candidates 2.0 -> 0.77 ms, a list with one pair of twins 60 -> 1.4.
 __global__ void __launch_bounds__(kNpThreads, kNpBlocksPerSm) k_narrow(NarrowArgs a) {
   constexpr unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   NpLane L;
   bool drained = false;
+  unsigned long long next = 0, end = 0;  // the warp's claim
   unsigned long long evals = 0, evals64 = 0, err = 0;
   for (;;) {
     const unsigned idle = __ballot_sync(kFull, L.q < 0);
     if (idle && !drained) {
-      const int leader = __ffs(idle) - 1;
+      const unsigned cnt = __popc(idle);
+      const unsigned long long have = end - next;
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(&a.state[NP_NEXT], (unsigned long long)__popc(idle));
-      base = __shfl_sync(kFull, base, leader);
-      if (base + (unsigned long long)__popc(idle) >= (unsigned long long)a.m) drained = true;
+      if (have < cnt) {
+        if (lane == 0) base = atomicAdd(&a.state[NP_NEXT], (unsigned long long)a.claim);
+        base = __shfl_sync(kFull, base, 0);
+      }
+      const unsigned r = __popc(idle & ((1u << lane) - 1u));
+      const unsigned long long mine = r < have ? next + r : base + (r - have);
+      if (have < cnt) {
+        next = base + (cnt - have);
+        end = base + a.claim;
+      } else {
+        next += cnt;
+      }
+      if (next >= (unsigned long long)a.m) drained = true;
       if (L.q < 0) {
-        const unsigned long long mine =
-            base + (unsigned long long)__popc(idle & ((1u << lane) - 1u));
         if (mine < (unsigned long long)a.m) {
           const int64_t qq = a.m - 1 - (int64_t)mine;
           const scd_pair c = a.pairs[qq];
@@ -301,6 +347,7 @@ __global__ void __launch_bounds__(kNpThreads, kNpBlocksPerSm) k_narrow(NarrowArg
             L.thi = c.thi;
             L.f = -1;
             L.cnt = 0;
+            L.shared = false;
             const float4 si = __ldg(reinterpret_cast<const float4 *>(a.obj + c.i) + 4);
             const float4 sj = __ldg(reinterpret_cast<const float4 *>(a.obj + c.j) + 4);
             L.V = si.x + sj.x;
@@ -308,6 +355,55 @@ __global__ void __launch_bounds__(kNpThreads, kNpBlocksPerSm) k_narrow(NarrowArg
             L.Rf = si.z + sj.z;
             L.slack = kNpSlackKm + kNpSlackRel * L.Rf;
           }
+        }
+      }
+    }
+    // The list is used up: an idle lane takes the later half of the interval of
+    // a lane that has a long way to go, so that a few long candidates spread
+    // over their warp instead of forming a tail.
+    if (drained && idle) {
+      const bool far = L.q >= 0 && L.thi - L.t >= kNpSplitTicks;
+      const unsigned donors = __ballot_sync(kFull, far);
+      const unsigned takers = __ballot_sync(kFull, L.q < 0);
+      const int moves = min(__popc(donors), __popc(takers));
+      if (moves > 0) {
+        const unsigned lt = (1u << lane) - 1u;
+        const bool give = far && __popc(donors & lt) < moves;
+        const int rank = __popc(takers & lt);
+        const bool take = L.q < 0 && rank < moves;
+        int src = lane;  // the taker of rank k takes from the donor of rank k
+        if (take) {
+          unsigned d = donors;
+          for (int k = 0; k < rank; ++k) d &= d - 1u;
+          src = __ffs(d) - 1;
+        }
+        if (give && !L.shared) {
+          if (a.first) a.first[L.q] = -1;
+          if (a.count) a.count[L.q] = 0;
+          __threadfence();  // before any lane's atomics on them
+          L.shared = true;
+        }
+        __syncwarp();
+        const long long q = __shfl_sync(kFull, (long long)L.q, src);
+        const int32_t t = __shfl_sync(kFull, L.t, src), thi = __shfl_sync(kFull, L.thi, src);
+        const uint32_t oi = __shfl_sync(kFull, L.oi, src), oj = __shfl_sync(kFull, L.oj, src);
+        const float Rf = __shfl_sync(kFull, L.Rf, src), V = __shfl_sync(kFull, L.V, src);
+        const float Acc = __shfl_sync(kFull, L.Acc, src);
+        const float slack = __shfl_sync(kFull, L.slack, src);
+        if (give) L.thi = L.t + (L.thi - L.t) / 2;
+        if (take) {
+          L.q = q;
+          L.oi = oi;
+          L.oj = oj;
+          L.t = t + (thi - t) / 2 + 1;
+          L.thi = thi;
+          L.f = -1;
+          L.cnt = 0;
+          L.shared = true;
+          L.Rf = Rf;
+          L.V = V;
+          L.Acc = Acc;
+          L.slack = slack;
         }
       }
     }
@@ -379,6 +475,9 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
     a.first = d_first;
     a.count = d_count;
     a.state = s->d_narrow.p;
+    a.claim = kNpMinClaim;
+    while (a.claim < kNpClaim && (int64_t)a.claim * 8 * blocks * (kNpThreads / 32) < n_pairs)
+      a.claim *= 2;
     k_narrow<<<(unsigned)blocks, kNpThreads, 0, s->stream>>>(a);
     note_launch();
   }
