@@ -52,8 +52,12 @@ constexpr float kNpSkipShrink = 1.0f - 1e-4f;
 constexpr float kNpResidualSlack = 3.5e-6f;
 
 // narrow-phase state words (device): earliest witness as t << 32 | candidate,
-// next candidate to claim, error bits, tick evaluations, FP64 evaluations
-enum { NP_EARLIEST = 0, NP_NEXT = 1, NP_ERR = 2, NP_EVALS = 3, NP_EVALS64 = 4, NP_WORDS = 5 };
+// next candidate to claim, error bits, tick evaluations, FP64 evaluations,
+// blocks finished, and the earliest witness' objects as i << 32 | j
+enum {
+  NP_EARLIEST = 0, NP_NEXT = 1, NP_ERR = 2, NP_EVALS = 3, NP_EVALS64 = 4, NP_DONE = 5,
+  NP_PAIR = 6, NP_WORDS = 7
+};
 enum : unsigned long long { NP_ERR_PAIR = 1, NP_ERR_KEPLER = 2 };
 
 // Per-object FP32 constants of the narrow phase (80 bytes, five 16-byte
@@ -95,8 +99,9 @@ struct NarrowArgs {
 // at most 2 a n / (1 - e)^2 per radian of E, and the FP32 solution's E is
 // within (residual) / (1 - e) of the true one; four times over.
 __global__ void k_np_objects(const ObjParams *__restrict__ par, int64_t n, double tick_s,
-                             NpObj *__restrict__ out) {
+                             NpObj *__restrict__ out, unsigned long long *state) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < NP_WORDS) state[i] = i == NP_EARLIEST ? ~0ull : 0ull;
   if (i >= n) return;
   const ObjParams p = par[i];
   const double a = sqrt(p.A[0] * p.A[0] + p.A[1] * p.A[1] + p.A[2] * p.A[2]);  // |A| = a
@@ -286,8 +291,10 @@ __device__ __forceinline__ void np_tick(const NarrowArgs &a, NpLane &L,
 }
 
 // candidates a warp claims per atomic at most (a lane takes the next one of
-// them every second step or so); short lists are dealt out 32 at a time
-constexpr unsigned kNpClaim = 256, kNpMinClaim = 32;
+// them every second step or so); short lists are dealt out 8 at a time to more
+// warps, whose idle lanes take halves of their intervals (43,851 candidates 133
+// us -> 59 for the call, 839 candidates 59 -> 37)
+constexpr unsigned kNpClaim = 256, kNpMinClaim = 8;
 // ticks left of an interval worth splitting (24 h INTERVAL candidates: never
 // 1.72 ms, from 128 ticks 1.13, 32 0.80, 16 0.77)
 constexpr int32_t kNpSplitTicks = 16;
@@ -323,15 +330,16 @@ __global__ void __launch_bounds__(kNpThreads, kNpBlocksPerSm) k_narrow(NarrowArg
       }
       const unsigned r = __popc(idle & ((1u << lane) - 1u));
       const unsigned long long mine = r < have ? next + r : base + (r - have);
+      const unsigned got = have < cnt ? a.claim : 0u;  // a claim may be less than was missing
       if (have < cnt) {
-        next = base + (cnt - have);
-        end = base + a.claim;
+        next = base + min((unsigned)(cnt - have), got);
+        end = base + got;
       } else {
         next += cnt;
       }
       if (next >= (unsigned long long)a.m) drained = true;
       if (L.q < 0) {
-        if (mine < (unsigned long long)a.m) {
+        if (r < have + got && mine < (unsigned long long)a.m) {
           const int64_t qq = a.m - 1 - (int64_t)mine;
           const scd_pair c = a.pairs[qq];
           if ((int64_t)c.i >= a.n || (int64_t)c.j >= a.n || c.tlo < 0 || c.tlo > c.thi ||
@@ -425,15 +433,18 @@ __global__ void __launch_bounds__(kNpThreads, kNpBlocksPerSm) k_narrow(NarrowArg
     if (evals64) atomicAdd(&a.state[NP_EVALS64], evals64);
     if (err) atomicOr(&a.state[NP_ERR], err);
   }
-}
-
-__global__ void k_narrow_init(unsigned long long *state) {
+  // the last block looks up the earliest witness' objects, so that the host
+  // reads everything with one copy
+  __syncthreads();
   if (threadIdx.x == 0) {
-    state[NP_EARLIEST] = ~0ull;
-    state[NP_NEXT] = 0;
-    state[NP_ERR] = 0;
-    state[NP_EVALS] = 0;
-    state[NP_EVALS64] = 0;
+    __threadfence();
+    if (atomicAdd(&a.state[NP_DONE], 1ull) == gridDim.x - 1ull) {
+      const unsigned long long w = atomicOr(&a.state[NP_EARLIEST], 0ull);
+      if (w != ~0ull) {
+        const scd_pair c = a.pairs[w & 0xffffffffull];
+        a.state[NP_PAIR] = (unsigned long long)c.i << 32 | c.j;
+      }
+    }
   }
 }
 
@@ -450,18 +461,18 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
   if (!s->d_narrow.ensure(NP_WORDS, s->stream)) return SCD_ERR_OOM;
   if (!s->d_npobj.ensure((size_t)s->n * sizeof(NpObj), s->stream)) return SCD_ERR_OOM;
   NpObj *obj = reinterpret_cast<NpObj *>(s->d_npobj.p);
-  k_narrow_init<<<1, 32, 0, s->stream>>>(s->d_narrow.p);
-  note_launch();
+  unsigned long long h[NP_WORDS] = {~0ull};
   if (n_pairs > 0) {
     // (FP64: one warp a block, spread over the SMs)
     k_np_objects<<<(unsigned)((s->n + 31) / 32), 32, 0, s->stream>>>(s->d_par.p, s->n, s->tick_s,
-                                                                      obj);
+                                                                      obj, s->d_narrow.p);
     note_launch();
     static int per_sm = 0, sms = 0;
     if (!per_sm) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_narrow, kNpThreads, 0);
     if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
     int64_t blocks = (int64_t)std::max(sms, 1) * std::max(per_sm, 1);
-    const int64_t need = (n_pairs + kNpThreads - 1) / kNpThreads;
+    constexpr int kPerBlock = kNpMinClaim * (kNpThreads / 32);
+    const int64_t need = (n_pairs + kPerBlock - 1) / kPerBlock;
     if (need < blocks) blocks = need;
     NarrowArgs a;
     a.par = s->d_par.p;
@@ -476,15 +487,14 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
     a.count = d_count;
     a.state = s->d_narrow.p;
     a.claim = kNpMinClaim;
-    while (a.claim < kNpClaim && (int64_t)a.claim * 8 * blocks * (kNpThreads / 32) < n_pairs)
+    while (a.claim < kNpClaim && (int64_t)a.claim * 2 * blocks * (kNpThreads / 32) < n_pairs)
       a.claim *= 2;
     k_narrow<<<(unsigned)blocks, kNpThreads, 0, s->stream>>>(a);
     note_launch();
   }
   if (cudaGetLastError() != cudaSuccess) return SCD_ERR_CUDA;
-  unsigned long long h[NP_WORDS];
-  if (cudaMemcpyAsync(h, s->d_narrow.p, sizeof(h), cudaMemcpyDeviceToHost, s->stream) !=
-          cudaSuccess ||
+  if ((n_pairs > 0 && cudaMemcpyAsync(h, s->d_narrow.p, sizeof(h), cudaMemcpyDeviceToHost,
+                                      s->stream) != cudaSuccess) ||
       cudaStreamSynchronize(s->stream) != cudaSuccess)
     return SCD_ERR_CUDA;
   s->last_np_evals = h[NP_EVALS];
@@ -496,14 +506,8 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
     earliest->j = 0;
     earliest->t = -1;
     if (h[NP_EARLIEST] != ~0ull) {
-      scd_pair p;
-      const int64_t q = (int64_t)(h[NP_EARLIEST] & 0xffffffffull);
-      if (cudaMemcpyAsync(&p, d_pairs + q, sizeof(p), cudaMemcpyDeviceToHost, s->stream) !=
-              cudaSuccess ||
-          cudaStreamSynchronize(s->stream) != cudaSuccess)
-        return SCD_ERR_CUDA;
-      earliest->i = p.i;
-      earliest->j = p.j;
+      earliest->i = (uint32_t)(h[NP_PAIR] >> 32);
+      earliest->j = (uint32_t)h[NP_PAIR];
       earliest->t = (int32_t)(h[NP_EARLIEST] >> 32);
     }
   }
