@@ -521,9 +521,10 @@ static int rf_queue(scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int r
                                                      B.tlo.p, B.thi.p, B.tobj.p, B.tcap);
       note_launch();
     }
-    const uint32_t *idx = nullptr;  // (by the keys' top 40 bits: five passes)
+    SortOut so;  // (by the keys' top 40 bits: five passes)
     int rc = radix_sort_u64_dev(B.key.p, B.idx.p, cap, dM, kb - 4 * kRfCurveBits, kb, B.sc, st,
-                                &idx);
+                                &so);
+    const uint32_t *idx = so.vals;
     if (rc != SCD_OK) return rc;
     rc = build_round_tree(idx, B.lo.p, B.hi.p, B.obj[cur].p, cap, dM, B.sbox.p, B.sobj.p,
                           B.nodes.p, B.nbox.p, B.ctr.p, st);

@@ -391,8 +391,15 @@ int radix_sort_u32(uint32_t *keys, uint32_t *vals, int64_t n, int bits, SortScra
 int radix_sort_u64(unsigned long long *keys, uint32_t *vals, int64_t n, int bits,
                    SortScratch &sc, cudaStream_t st);
 // the same by key bits [lo, bits) only (the bits below lo are payload)
+// so: the sorted arrays are left where the last pass put them (keys and vals, or
+// the scratch, by the number of passes) and named there, which saves the copy
+// back of an odd number of passes.
+struct SortOut {
+  const void *keys;
+  const uint32_t *vals;
+};
 int radix_sort_u64(unsigned long long *keys, uint32_t *vals, int64_t n, int lo, int bits,
-                   SortScratch &sc, cudaStream_t st);
+                   SortScratch &sc, cudaStream_t st, SortOut *so = nullptr);
 // size the scratch for sorts of up to n elements (nothing allocated later)
 int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaStream_t st);
 // the same with the element count read on the device (min(*d_n, n_cap)), for
@@ -404,12 +411,10 @@ int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaSt
 // in an unspecified order.
 int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, const unsigned long long *d_n,
                          int lo, int bits, SortScratch &sc, const PairEmit &pe, cudaStream_t st);
-// vals_out: only the sorted values are wanted; set to where they are (vals or
-// the scratch, by the number of passes; the keys are left in any order), which
-// saves the copy back of an odd number of passes over the whole capacity.
+// (without so the copy back takes the whole capacity)
 int radix_sort_u64_dev(unsigned long long *keys, uint32_t *vals, int64_t n_cap,
                        const unsigned long long *d_n, int lo, int bits, SortScratch &sc,
-                       cudaStream_t st, const uint32_t **vals_out = nullptr);
+                       cudaStream_t st, SortOut *so = nullptr);
 
 // Run starts carry their last tick below the (i, j, first tick) key when
 // both fit in 64 bits and the all-ones tick field is free to tag open runs
@@ -553,6 +558,7 @@ struct scd_scene {
   scd::DevBuf<scd_pair> d_out;
   int64_t n_out = 0;
   scd::SortScratch sort_sc;
+  scd::SortScratch ends_sc;  // the run ends' (the starts' sorted list may lie in sort_sc)
 
   // narrow phase: device state words, tick evaluations of the last call
   scd::DevBuf<unsigned long long> d_narrow;

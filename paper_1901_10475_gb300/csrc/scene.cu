@@ -201,7 +201,7 @@ extern "C" SCD_API int scd_scene_create(const scd_element *elems, int64_t n, dou
     scd_scene_destroy(s);
     return SCD_ERR_OOM;
   }
-  s->sort_sc.err = &s->d_ctr.p->sort_flags;
+  s->sort_sc.err = s->ends_sc.err = &s->d_ctr.p->sort_flags;
   cudaError_t e = cudaMemcpyAsync(s->d_el.p, elems, sizeof(scd_element) * (size_t)n,
                                   cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !s->band_fracs.empty()) {
@@ -531,7 +531,7 @@ static int find_graph(scd_scene *s, const scd_decomp *d, int dkind, int ob, int 
   if (!s->d_out.grow_keep(s->pair_cap, s->n_out, st) ||
       sort_reserve(s->sort_sc, s->pair_cap, sizeof(unsigned long long),
                    !runs_packed(ob, tb, s->T), st) != SCD_OK ||
-
+      sort_reserve(s->ends_sc, s->pair_cap, sizeof(unsigned long long), false, st) != SCD_OK ||
       !s->d_tilecnt.ensure((size_t)(s->pair_cap / 2048 + 2), st) ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return SCD_OK;  // no graph this time; the eager result stands
@@ -761,6 +761,7 @@ extern "C" SCD_API void scd_scene_destroy(scd_scene *s) {
   s->d_narrow.release(st);
   s->d_npobj.release(st);
   s->sort_sc.release(st);
+  s->ends_sc.release(st);
   s->s_cell.release(st);
   s->d_refcnt.release(st); s->d_refoff.release(st); s->d_refkey.release(st);
   s->d_refid.release(st); s->d_rr.release(st); s->d_edges.release(st);
