@@ -16,7 +16,7 @@ namespace scd {
 // or, where they fit one tile, to the last block to finish.  Bound
 // by the gather's loads: 32 bytes a box read at random (two 16-byte halves, a
 // sector each) and 32 + 4 written, 14 bytes of nodes.  With the neighbour
-// positions 0.73 ms for 17.4 M boxes (a binary radix tree with its gather and
+// links 0.69 ms for 17.4 M boxes (a binary radix tree with its gather and
 // bottom-up refit took 2.34 ms).
 constexpr int kTreeThreads = kWide * kWide * kWide;
 
@@ -88,17 +88,17 @@ __device__ __forceinline__ void make_node(float4 &lo, float4 &hi, bool valid, Wi
   axis_frame(lo.y, hi.y, false, s.y, o.y);
   axis_frame(lo.z, hi.z, false, s.z, o.z);
   axis_frame(lo.w, hi.w, true, s.w, o.w);
-  unsigned char *bl = reinterpret_cast<unsigned char *>(dst->lo) + c;
-  unsigned char *bh = reinterpret_cast<unsigned char *>(dst->hi) + c;
+  unsigned char *bl = reinterpret_cast<unsigned char *>(dst->half[c >> 2].lo) + (c & 3);
+  unsigned char *bh = reinterpret_cast<unsigned char *>(dst->half[c >> 2].hi) + (c & 3);
   // a child that does not exist: lower faces above all, upper ones below
   bl[0] = valid ? (unsigned char)node_coord(cl.x, s.x, o.x, false) : 127;
-  bl[8] = valid ? (unsigned char)node_coord(cl.y, s.y, o.y, false) : 127;
-  bl[16] = valid ? (unsigned char)node_coord(cl.z, s.z, o.z, false) : 127;
-  bl[24] = valid ? (unsigned char)node_coord(cl.w, s.w, o.w, false) : 127;
+  bl[4] = valid ? (unsigned char)node_coord(cl.y, s.y, o.y, false) : 127;
+  bl[8] = valid ? (unsigned char)node_coord(cl.z, s.z, o.z, false) : 127;
+  bl[12] = valid ? (unsigned char)node_coord(cl.w, s.w, o.w, false) : 127;
   bh[0] = valid ? (unsigned char)node_coord(ch.x, s.x, o.x, true) : 128;
-  bh[8] = valid ? (unsigned char)node_coord(ch.y, s.y, o.y, true) : 128;
-  bh[16] = valid ? (unsigned char)node_coord(ch.z, s.z, o.z, true) : 128;
-  bh[24] = valid ? (unsigned char)node_coord(ch.w, s.w, o.w, true) : 128;
+  bh[4] = valid ? (unsigned char)node_coord(ch.y, s.y, o.y, true) : 128;
+  bh[8] = valid ? (unsigned char)node_coord(ch.z, s.z, o.z, true) : 128;
+  bh[12] = valid ? (unsigned char)node_coord(ch.w, s.w, o.w, true) : 128;
   if (c == 0) {
     *reinterpret_cast<float4 *>(dst->scale) = s;
     *reinterpret_cast<float4 *>(dst->off) = o;
@@ -130,7 +130,7 @@ __device__ __forceinline__ void tree_tile(const TreeArgs &a, TreeSmem &sm, int k
       hi = __ldg(a.hi + b);
       a.sbox[i].lo = lo;
       a.sbox[i].hi = hi;
-      a.sobj[i] = __ldg(a.obj + b);
+      if (a.sobj) a.sobj[i] = __ldg(a.obj + b);
       // a box referenced from several cells: any copy will do, their data agree
       if (a.posof) a.posof[b] = (uint32_t)i;
       if (a.scell) a.scell[i] = (uint32_t)(a.keys[i] >> a.cell_shift);
@@ -182,8 +182,10 @@ __device__ __forceinline__ void tree_tile(const TreeArgs &a, TreeSmem &sm, int k
   __syncthreads();  // the next tile reuses the shared nodes
 }
 
+// (three blocks an SM: at 58 registers two fit, 0.77 ms instead of 0.69 for the
+// tree and the links)
 template <bool kGather>
-__global__ void __launch_bounds__(kTreeThreads) k_tree(TreeArgs a) {
+__global__ void __launch_bounds__(kTreeThreads, 3) k_tree(TreeArgs a) {
   __shared__ TreeSmem sm;
   __shared__ bool last;
   int64_t n = a.n;
@@ -206,19 +208,21 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree(TreeArgs a) {
   if (last && tiles > 0) tree_tile<false>(a, sm, a.k0 + 3, n, 0, a.out, a.out + tiles);
 }
 
-// Sorted positions of each box's previous and next segment of the same
-// object (-1 at the ends of the horizon).  Adjacent segments lie close in
-// space and time, so these positions stay near p along the curve.
-__global__ void k_neighbors(const uint32_t *__restrict__ id, const uint32_t *__restrict__ obj,
-                            const uint32_t *__restrict__ posof, int64_t Nq, int64_t nbox,
-                            int2 *__restrict__ nb) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Each sorted box's object and the sorted positions of that object's previous
+// and next segments (-1 at the ends of the horizon).  Adjacent segments lie
+// close in space and time, so these positions stay near p along the curve.
+// (In object order everything read lies in order, but 16 bytes written at
+// random cost more than the reads: 0.5 ms against 0.17 for 17.4 M boxes.)
+__global__ void k_links(const uint32_t *__restrict__ id, const uint32_t *__restrict__ obj,
+                        const uint32_t *__restrict__ posof, int64_t Nq, int64_t nbox,
+                        int4 *__restrict__ out) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= Nq) return;
-  uint32_t u = id[p];
-  uint32_t o = obj[u];
-  int prev = (u > 0 && obj[u - 1] == o) ? (int)posof[u - 1] : -1;
-  int next = ((int64_t)u + 1 < nbox && obj[u + 1] == o) ? (int)posof[u + 1] : -1;
-  nb[p] = make_int2(prev, next);
+  const int64_t u = (int64_t)id[p];
+  const uint32_t o = obj[u];
+  const int prev = u > 0 && obj[u - 1] == o ? (int)posof[u - 1] : -1;
+  const int next = u + 1 < nbox && obj[u + 1] == o ? (int)posof[u + 1] : -1;
+  out[p] = make_int4(prev, next, (int)o, 0);
 }
 
 int64_t tree_scratch_boxes(int64_t cap) {
@@ -268,8 +272,8 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
   cudaStream_t st = s->stream;
   const bool cells = cell_shift >= 0;
   if (Nq > kMaxTreeBoxes) return SCD_ERR_CAPACITY;
-  if (!s->s_box.ensure(Nq, st) || !s->s_obj.ensure(Nq, st) || !s->d_posof.ensure(s->N, st) ||
-      !s->s_nb.ensure(Nq, st) || !s->d_nodes.ensure(tree_levels(Nq).total, st) ||
+  if (!s->s_box.ensure(Nq, st) || !s->d_posof.ensure(s->N, st) || !s->s_link.ensure(Nq, st) ||
+      !s->d_nodes.ensure(tree_levels(Nq).total, st) ||
       !s->d_nbox.ensure(tree_scratch_boxes(Nq), st) || (cells && !s->s_cell.ensure(Nq, st)))
     return SCD_ERR_OOM;
   TreeArgs a{};
@@ -280,7 +284,6 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
   a.keys = keys_sorted;
   a.cell_shift = cells ? cell_shift : 0;
   a.sbox = s->s_box.p;
-  a.sobj = s->s_obj.p;
   a.posof = s->d_posof.p;
   a.scell = cells ? s->s_cell.p : nullptr;
   a.nodes = s->d_nodes.p;
@@ -288,8 +291,8 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
   a.finish = &s->d_ctr.p->tree_done;
   if (int rc = launch_tree(a, s->d_nbox.p, st)) return rc;
   const int bs = 256;
-  k_neighbors<<<(unsigned)((Nq + bs - 1) / bs), bs, 0, st>>>(ids_sorted, s->d_obj.p, s->d_posof.p,
-                                                             Nq, s->N, s->s_nb.p);
+  k_links<<<(unsigned)((Nq + bs - 1) / bs), bs, 0, st>>>(ids_sorted, s->d_obj.p, s->d_posof.p, Nq,
+                                                         s->N, s->s_link.p);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }

@@ -86,11 +86,13 @@ struct DevCounters {
 // (at most 127) never borrows from its neighbour and its top bit says
 // whether upper >= lower.  Children and queries go through the same monotone
 // map (node_coord), so a test in the frame never rejects a pair that overlaps
-// in FP32.  96 bytes, three 32-byte loads for eight child boxes (12 bytes a
-// child).
+// in FP32.  96 bytes for eight child boxes (12 bytes a child): three 32-byte
+// loads.
 struct __align__(32) WideNode {
-  float scale[4], off[4];       // x, y, z, tick
-  uint32_t lo[4][2], hi[4][2];  // per axis: children 0-3, children 4-7
+  float scale[4], off[4];  // x, y, z, tick
+  struct Half {
+    uint32_t lo[4], hi[4];  // per axis: a byte for each of four children
+  } half[2];                // children 0-3, children 4-7
 };
 static_assert(sizeof(WideNode) == 96, "three 32-byte sectors per node");
 constexpr int kWide = 8, kWideBits = 3;
@@ -501,9 +503,9 @@ struct scd_scene {
 
   // sorted leaves and hierarchy
   scd::DevBuf<scd::SBox> s_box;
-  scd::DevBuf<uint32_t> s_obj;
   scd::DevBuf<uint32_t> d_posof;  // sorted position of each box id
-  scd::DevBuf<int2> s_nb;         // sorted positions of the previous / next segment (-1: none)
+  scd::DevBuf<int4> s_link;       // sorted positions of the previous / next segment (-1: none),
+                                  // object, 0
   scd::DevBuf<uint32_t> s_cell;   // decomposition cell of each sorted reference
 
   // static decomposition: references (cell, box) and per-cell subtrees

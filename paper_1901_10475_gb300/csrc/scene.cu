@@ -752,8 +752,8 @@ extern "C" SCD_API void scd_scene_destroy(scd_scene *s) {
   s->d_band.release(st); s->d_ctr.release(st);
   s->d_lo.release(st); s->d_hi.release(st); s->d_obj.release(st);
   s->d_key64.release(st); s->d_key32.release(st); s->d_id.release(st);
-  s->s_box.release(st); s->s_obj.release(st);
-  s->d_posof.release(st); s->s_nb.release(st);
+  s->s_box.release(st);
+  s->d_posof.release(st); s->s_link.release(st);
   s->d_nodes.release(st); s->d_nbox.release(st);
   s->d_starts.release(st); s->d_ends.release(st); s->d_rawval.release(st);
   s->d_tilecnt.release(st);

@@ -29,8 +29,8 @@ struct TravArgs {
   const WideNode *nodes;      // the tree (all levels, lv.off)
   TreeLevels lv;
   const SBox *sbox;           // sorted boxes
-  const uint32_t *sobj, *sid; // object and unsorted id of each sorted box
-  const int2 *nb;             // sorted positions of the previous / next segment
+  const uint32_t *sobj, *sid; // (rounds) object and unsorted id of each sorted box
+  const int4 *link;           // (screens) previous / next segment (-1: none), object, 0
   int64_t N;
   int T;
   int raw;
@@ -96,7 +96,7 @@ constexpr unsigned kMinChunk = 32, kMaxChunk = 512;
 // (slot numbers in 32 bits: the record sorts take no more, and a list that
 // would need more is refused)
 struct ChunkCursor {
-  uint32_t next = 0, end = 0, count = 0;
+  uint32_t next, end, count;
 };
 
 __device__ __forceinline__ void chunk_fill_holes(ChunkCursor &c, unsigned long long *buf,
@@ -104,7 +104,6 @@ __device__ __forceinline__ void chunk_fill_holes(ChunkCursor &c, unsigned long l
   const int lane = threadIdx.x & 31;
   for (uint32_t k = c.next + lane; k < c.end; k += 32)
     if (k < cap) buf[k] = kHole;
-  c.next = c.end;
 }
 
 __device__ __forceinline__ void chunk_put(ChunkCursor &c, unsigned long long *buf, uint32_t *vbuf,
@@ -114,25 +113,30 @@ __device__ __forceinline__ void chunk_put(ChunkCursor &c, unsigned long long *bu
   const unsigned vote = __ballot_sync(0xffffffffu, pred);
   const uint32_t cnt = __popc(vote);
   if (cnt == 0) return;
-  if (c.next + cnt > c.end) {
+  uint32_t next = c.next;
+  if (next + cnt > c.end) {
     chunk_fill_holes(c, buf, cap);
     unsigned long long b = 0;
     if (lane == 0) {
       b = atomicAdd(slots, (unsigned long long)chunk);
       if (b > 0xffffffffull - 2 * kMaxChunk) b = 0xffffffffull - 2 * kMaxChunk;  // past any cap
     }
-    c.next = __shfl_sync(0xffffffffu, (uint32_t)b, 0);
-    c.end = c.next + chunk;
+    next = __shfl_sync(0xffffffffu, (uint32_t)b, 0);
+    if (lane == 0) c.end = next + chunk;
   }
   if (pred) {
-    const uint32_t idx = c.next + __popc(vote & ((1u << lane) - 1u));
+    const uint32_t idx = next + __popc(vote & ((1u << lane) - 1u));
     if (idx < cap) {
       buf[idx] = key;
       if (vbuf) vbuf[idx] = v;
     }
   }
-  c.next += cnt;
-  c.count += cnt;
+  __syncwarp();
+  if (lane == 0) {
+    c.next = next + cnt;
+    c.count += cnt;
+  }
+  __syncwarp();
 }
 
 // Is (q, b) the first / last cell of its run?  Both need the neighbouring
@@ -186,20 +190,30 @@ __device__ __forceinline__ unsigned long long start_key(const TravArgs &a, unsig
 // visit): at most ten words in shared memory, whatever the query, so no stack
 // can overflow.
 //
-// Bound by the L1's wavefronts: a node's three 32-byte loads take one each per
-// distinct line, and a pair's exact boxes, objects and neighbouring segments
-// about 135 per 32 pairs.  Measured on the 24 h catalog screen (17.4 M boxes,
-// 164 M runs; SPEED / INTERVAL boxes): lanes alone 12.2 / 6.5 ms, groups of two
-// 11.3 / 5.9, of four 11.6 / 6.1, of eight 14.1 / 7.7; with groups of two, 256
-// buffered leaf nodes instead of 160 take SPEED from 11.5 to 11.3; fetching the
-// children ahead into L1 costs more wavefronts than it hides (17.7 / 15.8).
-// Two-child nodes of 36 bytes along a Morton curve, with 64-entry stacks in
-// local memory, took 18.4 / 10.7 ms and 91 nodes a query.
+// Bound by the L1's wavefronts (its data pipe is busy 90% of the time, the
+// schedulers 66%): a node's three 32-byte loads take one each per distinct
+// line, and so do a pair's exact boxes, links and neighbouring segments.
+// 24 h catalog screen (17.4 M boxes, 164 M runs; SPEED / INTERVAL boxes):
+// 10.1 / 5.15 ms.  What led here, measured at one stage or another: lanes alone
+// 12.2 / 6.5, groups of two 11.3 / 5.9, of four 11.6 / 6.1, of eight 14.1 / 7.7;
+// 256 buffered leaf nodes instead of 160, SPEED 11.5 to 11.3; a pair's object
+// and links in one load, with the registers it takes, 11.2 / 5.9 to 10.6 /
+// 5.3; the pairs left over by one expansion joining the next, 10.4 / 5.26; the
+// record chunks' state in shared memory, so that eight blocks of 64 registers
+// fit without spills, 10.1 / 5.15.  Slower: fetching the children ahead into
+// L1 (17.7 / 15.8), the neighbours' rounded boxes beside the links (12.9 /
+// 5.8), two lanes testing half the children each for both (a sixth fewer
+// wavefronts, 18% more instructions; 10.4 / 5.36).  Two-child nodes of 36 bytes
+// along a Morton curve, with 64-entry stacks in local memory, took 18.4 / 10.7
+// and 91 nodes a query.
 // ---------------------------------------------------------------------------
 constexpr int kTvThreads = 128;
 constexpr int kTvWarps = kTvThreads / 32;
 // lanes that walk together (their queries are consecutive)
 constexpr int kGroup = 2;
+// lanes without a query before the warp hands out new ones, a step of the whole
+// warp (INTERVAL 5.31 -> 5.25 ms; SPEED the same; 2 and 8 lie between)
+constexpr int kMinRefill = 4;
 // leaf nodes (query, node, mask of its boxes) buffered per warp, drained when
 // fewer than one step's worth (32) of slots remain
 constexpr int kEntryCap = 256;
@@ -212,6 +226,7 @@ constexpr unsigned kQueryChunk = 32;
 // one new chunk: a chunk smaller than a warp would leave lanes without one
 static_assert(kQueryChunk >= 32, "a query chunk covers at least one warp's refill");
 
+// (in shared memory: the registers go to the pairs)
 struct WarpEmit {
   ChunkCursor s, e;  // start and end record chunks (raw cells use s)
 };
@@ -248,11 +263,14 @@ __device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint3
                                             WarpEmit &we) {
   float4 ql = make_float4(0.f, 0.f, 0.f, 0.f), qh = ql, bl = ql, bh = ql;
   uint32_t qo = 0, bo = 0;
+  int4 qk = make_int4(0, 0, 0, 0), bk = qk;
   if (valid) {
     ldg_box(a.sbox + p, ql, qh);
-    qo = __ldg(a.sobj + p);
+    qk = __ldg(a.link + p);
     ldg_box(a.sbox + b, bl, bh);
-    bo = __ldg(a.sobj + b);
+    bk = __ldg(a.link + b);
+    qo = (uint32_t)qk.z;
+    bo = (uint32_t)bk.z;
     valid = bo != qo && box_overlap(ql, qh, bl, bh);
     if (valid && a.dkind != SCD_DECOMP_NONE)
       valid = reports_here(a, __ldg(a.scell + p), ql, bl, qo, bo);
@@ -266,7 +284,7 @@ __device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint3
   }
   bool start = valid, end = valid;
   if (valid)
-    run_ends_sorted(a, ql, qh, __ldg(a.nb + p), bl, bh, __ldg(a.nb + b), s, e,
+    run_ends_sorted(a, ql, qh, make_int2(qk.x, qk.y), bl, bh, make_int2(bk.x, bk.y), s, e,
                     a.objT ? __ldg(a.objT + qo) : a.T, start, end);
   const uint32_t last = end ? (uint32_t)e : a.open_tag;
   chunk_put(we.s, a.starts, a.packed ? nullptr : a.rawval, &a.ctr->n_starts, a.cap,
@@ -280,17 +298,18 @@ __device__ __forceinline__ void screen_pair(const TravArgs &a, bool valid, uint3
 struct HitBuf {
   uint32_t p[kEntryCap], n[kEntryCap];  // query, leaf node
   uint8_t mask[kEntryCap];              // its boxes that meet the query
-  uint16_t pair[kExpand * kWide];       // entry | box << 8
+  uint16_t pair[kExpand * kWide + 32];  // entry | box << 8
 };
 static_assert(kEntryCap <= 256, "an expanded pair names its entry in eight bits");
 
 // The buffered leaf nodes' pairs, spread evenly over the lanes: the entries'
 // boxes are counted and listed kExpand entries at a time, then 32 listed
-// pairs at a time are decided.  Returns the pairs.
+// pairs at a time are decided; fewer than 32 left over go with the next
+// entries.  Returns the pairs.
 template <bool kRefine>
 __device__ __forceinline__ int drain(const TravArgs &a, HitBuf &h, int cnt, WarpEmit &we) {
   const int lane = threadIdx.x & 31;
-  int pairs = 0;
+  int pairs = 0, rest = 0;
   for (int base = 0; base < cnt; base += kExpand) {
     const int k0 = base + lane, k1 = k0 + 32;
     uint32_t m0 = k0 < cnt ? h.mask[k0] : 0u, m1 = k1 < cnt ? h.mask[k1] : 0u;
@@ -302,12 +321,14 @@ __device__ __forceinline__ int drain(const TravArgs &a, HitBuf &h, int cnt, Warp
       const int v = __shfl_up_sync(0xffffffffu, at, d);
       if (lane >= d) at += v;
     }
-    const int total = __shfl_sync(0xffffffffu, at, 31);
-    at -= mine;
+    const int total = rest + __shfl_sync(0xffffffffu, at, 31);
+    at += rest - mine;
     for (; m0; m0 &= m0 - 1u) h.pair[at++] = (uint16_t)(k0 | (__ffs(m0) - 1) << 8);
     for (; m1; m1 &= m1 - 1u) h.pair[at++] = (uint16_t)(k1 | (__ffs(m1) - 1) << 8);
     __syncwarp();
-    for (int r = 0; r < total; r += 32) {
+    // whole warps of pairs; the rest goes with the next entries
+    const int now = base + kExpand < cnt ? total & ~31 : total;
+    for (int r = 0; r < now; r += 32) {
       const bool valid = r + lane < total;
       uint32_t p = 0, b = 0;
       if (valid) {
@@ -321,8 +342,11 @@ __device__ __forceinline__ int drain(const TravArgs &a, HitBuf &h, int cnt, Warp
         screen_pair(a, valid, p, b, we);
       }
     }
-    pairs += total;
+    pairs += now;
+    rest = total - now;
+    const uint16_t left = lane < rest ? h.pair[now + lane] : (uint16_t)0;
     __syncwarp();
+    if (lane < rest) h.pair[lane] = left;
   }
   return pairs;
 }
@@ -332,10 +356,10 @@ __device__ __forceinline__ int drain(const TravArgs &a, HitBuf &h, int cnt, Warp
 // axis and four children one byte-wise difference each tests lo <= query hi
 // and query lo <= hi (the guard bit survives where it holds).
 __device__ __forceinline__ uint32_t meet_mask(const WideNode *nd, float4 qlo, float4 qhi) {
-  uint32_t f[8], lo[8], hi[8];
+  uint32_t f[8], c0[8], c1[8];
   ldg_words(nd->scale, f);
-  ldg_words(nd->lo, lo);
-  ldg_words(nd->hi, hi);
+  ldg_words(&nd->half[0], c0);
+  ldg_words(&nd->half[1], c1);
   const float ql[4] = {qlo.x, qlo.y, qlo.z, qlo.w}, qh[4] = {qhi.x, qhi.y, qhi.z, qhi.w};
   uint32_t r0 = 0x80808080u, r1 = 0x80808080u;
 #pragma unroll
@@ -343,8 +367,8 @@ __device__ __forceinline__ uint32_t meet_mask(const WideNode *nd, float4 qlo, fl
     const float sc = __uint_as_float(f[d]), of = __uint_as_float(f[4 + d]);
     const uint32_t l4 = __byte_perm(node_coord(ql[d], sc, of, false), 0u, 0x0000u);
     const uint32_t h4 = __byte_perm(node_coord(qh[d], sc, of, true), 0u, 0x0000u);
-    r0 &= (h4 - lo[2 * d]) & (hi[2 * d] - l4);
-    r1 &= (h4 - lo[2 * d + 1]) & (hi[2 * d + 1] - l4);
+    r0 &= (h4 - c0[d]) & (c0[4 + d] - l4);
+    r1 &= (h4 - c1[d]) & (c1[4 + d] - l4);
   }
   // the guard bits of children 0-3 and 4-7 gathered into the top byte: bit
   // 8 c and bit 8 c + 4 of x go to 24 + c and 28 + c (no two products of the
@@ -385,10 +409,13 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
   // the later ones by the counter (no atomics where a few warps do it all)
   uint32_t q_next = min((blockIdx.x * kTvWarps + w) * kQueryChunk, nq);
   uint32_t q_end = q_next + kQueryChunk;
-  WarpEmit we;
+  __shared__ WarpEmit emits[kTvWarps];
+  WarpEmit &we = emits[w];
+  if (lane == 0) we.s = we.e = ChunkCursor{0, 0, 0};
+  __syncwarp();
   for (;;) {
     unsigned idle = __ballot_sync(kFull, lv == 0u);
-    if (idle) {
+    if (idle && (dry || __popc(idle) >= kMinRefill)) {
       if (!dry) {
         // groups without queries take the next ones from the warp's pool
         const uint32_t cnt = (uint32_t)__popc(idle);  // whole groups are idle
@@ -619,8 +646,7 @@ int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   TravArgs a{};
   a.nodes = s->d_nodes.p;
   a.sbox = s->s_box.p;
-  a.sobj = s->s_obj.p;
-  a.nb = s->s_nb.p;
+  a.link = s->s_link.p;
   a.sid = s->d_id.p;
   // one query per sorted reference
   a.N = s->dkind != SCD_DECOMP_NONE ? s->n_refs : s->N;
