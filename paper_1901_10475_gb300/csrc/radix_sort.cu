@@ -15,8 +15,13 @@ namespace scd {
 
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsItems = 8;
-constexpr int kRsTile = kRsThreads * kRsItems;
+// Keys a thread: what the registers of three (keys alone) or four resident
+// blocks hold without spills.  Longer tiles make longer runs of a digit in the
+// scatter: keys alone, 12 instead of 8 take the 24 h catalog's canonical list
+// (164 M records, five passes) from 8.03 to 7.80 ms (16 spill: 8.9); with
+// values 12 are slower (17.4 M boxes, six passes: 0.93 -> 1.05).
+__host__ __device__ constexpr int rs_items(bool vals) { return vals ? 8 : 12; }
+__host__ __device__ constexpr int rs_tile(bool vals) { return kRsThreads * rs_items(vals); }
 
 template <class K>
 __device__ __forceinline__ uint32_t digit_of(K key, int shift) {
@@ -34,13 +39,14 @@ __device__ __forceinline__ int64_t sort_count(int64_t n, const unsigned long lon
 
 // kOpen: also count, per digit, the keys whose low tmask bits are all ones
 // (open run starts; holes too, which sort last) into ocounts
-template <class K, bool kOpen = false>
+template <class K, bool kVals, bool kOpen = false>
 __global__ void __launch_bounds__(kRsThreads) k_rs_upsweep(const K *__restrict__ keys, int64_t n,
                                                            const unsigned long long *__restrict__ d_n,
                                                            int shift, uint32_t *__restrict__ counts,
                                                            int64_t nblk,
                                                            uint32_t *__restrict__ ocounts = nullptr,
                                                            unsigned long long tmask = 0) {
+  constexpr int kRsItems = rs_items(kVals), kRsTile = rs_tile(kVals);
   n = sort_count(n, d_n);
   __shared__ uint32_t wh[kRsWarps][256];
   __shared__ uint32_t wo[kOpen ? kRsWarps : 1][256];
@@ -97,12 +103,12 @@ __global__ void __launch_bounds__(kThreads) k_rs_scan(uint32_t *__restrict__ cou
                                                   uint32_t *__restrict__ totals,
                                                   const unsigned long long *__restrict__ d_n =
                                                       nullptr,
-                                                  int64_t n = 0) {
+                                                  int64_t n = 0, int tile = 1) {
   constexpr int kWarps = kThreads / 32;
   __shared__ uint32_t ws[kWarps];
   uint32_t *c = counts + (int64_t)blockIdx.x * nblk;  // rows of nblk
   // with a device count, only the blocks that hold items counted
-  if (d_n) nblk = std::min<int64_t>(nblk, (sort_count(n, d_n) + kRsTile - 1) / kRsTile);
+  if (d_n) nblk = std::min<int64_t>(nblk, (sort_count(n, d_n) + tile - 1) / tile);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t carry = 0;
   for (int64_t b0 = 0; b0 < nblk; b0 += kThreads * kScanItems) {
@@ -219,12 +225,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 // its own rank among the open starts (from the open counts per digit and
 // tile, ocounts / ototals, and an in-tile prefix).
 template <class K, bool kVals, bool kPairs = false>
-__global__ void __launch_bounds__(kRsThreads, 4) k_rs_downsweep(
+__global__ void __launch_bounds__(kRsThreads, kVals ? 4 : 3) k_rs_downsweep(
     const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__restrict__ kout,
     uint32_t *__restrict__ vout, int64_t n, const unsigned long long *__restrict__ d_n, int shift,
     const uint32_t *__restrict__ counts, const uint32_t *__restrict__ totals, int64_t nblk,
     unsigned int *err, int even = 0, const uint32_t *__restrict__ ocounts = nullptr,
     const uint32_t *__restrict__ ototals = nullptr, PairEmit pe = PairEmit{}) {
+  constexpr int kRsItems = rs_items(kVals), kRsTile = rs_tile(kVals);
   n = sort_count(n, d_n);
   const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -721,9 +728,11 @@ static int rs_sms() {
 
 // the scan of 256 digits' rows of nblk counts
 static void rs_scan(uint32_t *counts, int64_t nblk, uint32_t *totals,
-                    const unsigned long long *d_n, int64_t n, cudaStream_t st) {
-  if (nblk <= 256 * kScanItems) k_rs_scan<256><<<256, 256, 0, st>>>(counts, nblk, totals, d_n, n);
-  else k_rs_scan<1024><<<256, 1024, 0, st>>>(counts, nblk, totals, d_n, n);
+                    const unsigned long long *d_n, int64_t n, int tile, cudaStream_t st) {
+  if (nblk <= 256 * kScanItems)
+    k_rs_scan<256><<<256, 256, 0, st>>>(counts, nblk, totals, d_n, n, tile);
+  else
+    k_rs_scan<1024><<<256, 1024, 0, st>>>(counts, nblk, totals, d_n, n, tile);
 }
 
 template <class K>
@@ -737,7 +746,8 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
   // tiles are copied whole into shared memory: 16-byte aligned arrays
   if ((reinterpret_cast<uintptr_t>(keys) | reinterpret_cast<uintptr_t>(vals)) & 15)
     return SCD_ERR_INTERNAL;
-  int64_t nblk = (n + kRsTile - 1) / kRsTile;
+  const int tile = rs_tile(vals != nullptr);
+  int64_t nblk = (n + tile - 1) / tile;
   if (!sc.keys_alt.ensure(sizeof(K) * (size_t)n, st)) return SCD_ERR_OOM;
   if (vals && !sc.vals_alt.ensure((size_t)n, st)) return SCD_ERR_OOM;
   if (!pe && n <= (d_n ? kClusterMax : kClusterHost)) {
@@ -753,7 +763,7 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
   uint32_t *va = vals, *vb = sc.vals_alt.p;
   // two tile buffers of keys (and values); persistent grid of the blocks
   // that fit at once
-  size_t smem = 2 * (sizeof(K) * kRsTile + (vals ? sizeof(uint32_t) * kRsTile : 0));
+  size_t smem = 2 * (sizeof(K) * tile + (vals ? sizeof(uint32_t) * tile : 0));
   static int grid_of[2][2] = {{0, 0}, {0, 0}};
   int ki = sizeof(K) == 8 ? 1 : 0, vi = vals ? 1 : 0;
   if (!grid_of[ki][vi]) {
@@ -794,18 +804,21 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
     if (pe && shift + 8 >= bits) {
       // the last pass: decoded pairs to their sorted positions
       const unsigned long long tmask = (1ull << pe->tb) - 1ull;
-      k_rs_upsweep<unsigned long long, true><<<ugrid, kRsThreads, 0, st>>>(
+      k_rs_upsweep<unsigned long long, false, true><<<ugrid, kRsThreads, 0, st>>>(
           (const unsigned long long *)ka, n, d_n, shift, counts, nblk, ocounts, tmask);
-      rs_scan(counts, nblk, totals, d_n, n, st);
-      rs_scan(ocounts, nblk, ototals, d_n, n, st);
+      rs_scan(counts, nblk, totals, d_n, n, tile, st);
+      rs_scan(ocounts, nblk, ototals, d_n, n, tile, st);
       k_rs_downsweep<unsigned long long, false, true><<<grid, kRsThreads, smem, st>>>(
           (const unsigned long long *)ka, nullptr, nullptr, nullptr, n, d_n, shift, counts,
           totals, nblk, sc.err, 0, ocounts, ototals, *pe);
       note_launch(4);
       return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
     }
-    k_rs_upsweep<K><<<ugrid, kRsThreads, 0, st>>>(ka, n, d_n, shift, counts, nblk);
-    rs_scan(counts, nblk, totals, d_n, n, st);
+    if (vals)
+      k_rs_upsweep<K, true><<<ugrid, kRsThreads, 0, st>>>(ka, n, d_n, shift, counts, nblk);
+    else
+      k_rs_upsweep<K, false><<<ugrid, kRsThreads, 0, st>>>(ka, n, d_n, shift, counts, nblk);
+    rs_scan(counts, nblk, totals, d_n, n, tile, st);
     if (vals)
       k_rs_downsweep<K, true><<<grid, kRsThreads, smem, st>>>(ka, va, kb, vb, n, d_n, shift,
                                                                counts, totals, nblk, sc.err);
@@ -841,10 +854,11 @@ int radix_partition_u64(const unsigned long long *kin, unsigned long long *kout,
   if (n >= (1ll << 32) - 512) return SCD_ERR_CAPACITY;
   if ((reinterpret_cast<uintptr_t>(kin) | reinterpret_cast<uintptr_t>(kout)) & 15)
     return SCD_ERR_INTERNAL;
-  const int64_t nblk = (n + kRsTile - 1) / kRsTile;
+  const int tile = rs_tile(false);
+  const int64_t nblk = (n + tile - 1) / tile;
   if (!sc.counts.ensure((size_t)(256 * nblk + 256), st)) return SCD_ERR_OOM;
   uint32_t *counts = sc.counts.p, *totals = sc.counts.p + 256 * nblk;
-  const size_t smem = 2 * sizeof(unsigned long long) * kRsTile;
+  const size_t smem = 2 * sizeof(unsigned long long) * tile;
   static int grid = 0;
   if (!grid) {
     int sms = 0, per_sm = 0, dev = 0;
@@ -856,9 +870,9 @@ int radix_partition_u64(const unsigned long long *kin, unsigned long long *kout,
                                                   kRsThreads, smem);
     grid = std::max(1, sms) * std::max(1, per_sm);
   }
-  k_rs_upsweep<unsigned long long><<<(unsigned)nblk, kRsThreads, 0, st>>>(kin, n, nullptr, shift,
-                                                                          counts, nblk);
-  rs_scan(counts, nblk, totals, nullptr, 0, st);
+  k_rs_upsweep<unsigned long long, false>
+      <<<(unsigned)nblk, kRsThreads, 0, st>>>(kin, n, nullptr, shift, counts, nblk);
+  rs_scan(counts, nblk, totals, nullptr, 0, tile, st);
   k_rs_downsweep<unsigned long long, false>
       <<<(unsigned)std::min<int64_t>(nblk, grid), kRsThreads, smem, st>>>(
           kin, nullptr, kout, nullptr, n, nullptr, shift, counts, totals, nblk, sc.err, 1);
@@ -891,7 +905,8 @@ void scan_u32_exclusive(uint32_t *a, int64_t n, uint32_t *total, cudaStream_t st
 }
 
 int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaStream_t st) {
-  int64_t nblk = (n + kRsTile - 1) / kRsTile;
+  const int tile = rs_tile(vals);
+  int64_t nblk = (n + tile - 1) / tile;
   if (!sc.keys_alt.ensure(key_bytes * (size_t)n, st)) return SCD_ERR_OOM;
   if (vals && !sc.vals_alt.ensure((size_t)n, st)) return SCD_ERR_OOM;
   if (!sc.counts.ensure((size_t)(256 * nblk + 256), st)) return SCD_ERR_OOM;
