@@ -178,11 +178,11 @@ __global__ void __launch_bounds__(256) k_build_boxes(BoxArgs a) {
   L.x = __double2float_rd(lo[0]);
   L.y = __double2float_rd(lo[1]);
   L.z = __double2float_rd(lo[2]);
-  L.w = (float)tlo;
+  L.w = (float)(int32_t)tlo;  // below 2^24: exact
   H.x = __double2float_ru(hi[0]);
   H.y = __double2float_ru(hi[1]);
   H.z = __double2float_ru(hi[2]);
-  H.w = (float)thi;
+  H.w = (float)(int32_t)thi;
   a.lo[b] = L;
   a.hi[b] = H;
   a.obj[b] = (uint32_t)i;
