@@ -199,40 +199,49 @@ __global__ void __launch_bounds__(kRfBoxThreads) k_rf_boxes(RfBoxArgs a) {
 // Where every chunk claims for itself that one counter bounds it: 24 h catalog,
 // 141 M intervals over ten rounds, 58.1 -> 57.0 ms for the refinement with four
 // chunks a claim (58.1 again with eight: too few warps at work late on).
+// A round that one chunk a warp covers takes them one by one (512 objects: 430
+// us, 434 in fours).
 constexpr int kRfClaim = 4;
 
-template <class Need, class Put>
-__device__ __forceinline__ void rf_next(unsigned long long *asked, int64_t cap, Need need,
-                                        Put put) {
-  const int64_t M = rf_count(asked, cap);
+template <int kChunks, class Need, class Put>
+__device__ __forceinline__ void rf_claim(int64_t M, unsigned long long *next, int64_t cap,
+                                         Need need, Put put) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < M;
-       base += kRfClaim * stride) {
-    uint32_t n[kRfClaim], at[kRfClaim], total = 0;
+       base += kChunks * stride) {
+    uint32_t n[kChunks], at[kChunks], total = 0;
 #pragma unroll
-    for (int u = 0; u < kRfClaim; ++u) {
+    for (int u = 0; u < kChunks; ++u) {
       const int64_t i = base + u * stride + lane;
       n[u] = i < M ? need(i) : 0u;
     }
 #pragma unroll
-    for (int u = 0; u < kRfClaim; ++u) {
+    for (int u = 0; u < kChunks; ++u) {
       const unsigned one = __ballot_sync(0xffffffffu, n[u] >= 1u);
       const unsigned two = __ballot_sync(0xffffffffu, n[u] == 2u);
       at[u] = total + __popc(one & lt) + __popc(two & lt);
       total += __popc(one) + __popc(two);
     }
     unsigned long long q0 = 0;
-    if (lane == 0 && total) q0 = atomicAdd(asked + 1, (unsigned long long)total);
+    if (lane == 0 && total) q0 = atomicAdd(next, (unsigned long long)total);
     q0 = __shfl_sync(0xffffffffu, q0, 0);
 #pragma unroll
-    for (int u = 0; u < kRfClaim; ++u) {
+    for (int u = 0; u < kChunks; ++u) {
       const unsigned long long q = q0 + at[u];
       if (n[u] && q < (unsigned long long)cap)
         put(base + u * stride + lane, q, n[u] == 2u && q + 1 < (unsigned long long)cap);
     }
   }
+}
+
+template <class Need, class Put>
+__device__ __forceinline__ void rf_next(unsigned long long *asked, int64_t cap, Need need,
+                                        Put put) {
+  const int64_t M = rf_count(asked, cap);
+  if (M <= (int64_t)gridDim.x * blockDim.x) rf_claim<1>(M, asked + 1, cap, need, put);
+  else rf_claim<kRfClaim>(M, asked + 1, cap, need, put);
 }
 
 // next round's intervals (order is free: appended by atomics)
