@@ -424,7 +424,7 @@ struct RfBuffers {
     const size_t c = (size_t)cap;
     for (int b = 0; b < 2; ++b)
       if (!obj[b].ensure(c, st) || !t0[b].ensure(c, st) || !t1[b].ensure(c, st)) return false;
-    if (cap > kMaxTreeBoxes) return false;
+    if (cap > kMaxRoundBoxes) return false;
     return idx.ensure(c, st) && flags.ensure(c, st) && sobj.ensure(c, st) && lo.ensure(c, st) &&
            hi.ensure(c, st) && key.ensure(c, st) && sbox.ensure(c, st) &&
            nbox.ensure((size_t)tree_scratch_boxes(cap), st) &&

@@ -96,9 +96,11 @@ struct __align__(32) WideNode {
 };
 static_assert(sizeof(WideNode) == 96, "three 32-byte sectors per node");
 constexpr int kWide = 8, kWideBits = 3;
-// 8^10 boxes: sorted positions are below 2^30
-constexpr int kMaxLevels = 10;
-constexpr int64_t kMaxTreeBoxes = 1ll << (kWideBits * kMaxLevels);
+// sorted positions are below 2^31; a traversal's pending node (its parent's
+// index and eight bits) fits 32 bits up to 8^10 boxes, ten levels
+constexpr int kMaxLevels = 11, kWordLevels = 10;
+constexpr int64_t kMaxTreeBoxes = 1ll << 31;
+constexpr int64_t kMaxRoundBoxes = 1ll << (kWideBits * kWordLevels);
 
 // the levels' places in one array of nodes, for up to `cap` boxes: level k
 // (1 .. levels) holds ceil(cap / 8^k) nodes from off[k]; the last has one

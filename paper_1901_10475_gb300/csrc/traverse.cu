@@ -187,7 +187,8 @@ __device__ __forceinline__ unsigned long long start_key(const TravArgs &a, unsig
 // the curve and visit nearly the same nodes, so the group visits the union of
 // them and one load serves its lanes.  A group's pending nodes are one 32-bit
 // word per level (the parent's index and a mask of its children still to
-// visit): at most ten words in shared memory, whatever the query, so no stack
+// visit; 64 bits above 2^30 boxes): one a level in shared memory, whatever the
+// query, so no stack
 // can overflow.
 //
 // Bound by the L1's wavefronts (its data pipe is busy 90% of the time, the
@@ -377,10 +378,12 @@ __device__ __forceinline__ uint32_t meet_mask(const WideNode *nd, float4 qlo, fl
   return (x * 0x01020408u) >> 24;
 }
 
-template <bool kRefine>
+template <bool kRefine, bool kHuge>
 __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
   __shared__ HitBuf hits[kTvWarps];
-  __shared__ uint32_t pend[kMaxLevels][kTvThreads / kGroup];  // [level - 1]: parent << 8 | mask
+  using Word = typename std::conditional<kHuge, unsigned long long, uint32_t>::type;
+  constexpr int kLevels = kHuge ? kMaxLevels : kWordLevels;
+  __shared__ Word pend[kLevels][kTvThreads / kGroup];  // [level - 1]: parent << 8 | mask
   __shared__ uint32_t off[kMaxLevels + 1];
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int kStride = kTvThreads / kGroup;
@@ -390,7 +393,7 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
   constexpr unsigned kLead = 0x55555555u;  // the groups' first lanes
   static_assert(kGroup == 2, "kLead and the group reduction are for pairs of lanes");
   HitBuf &buf = hits[w];
-  uint32_t *const mine = &pend[0][threadIdx.x / kGroup] - kStride;  // level l at mine[l * kStride]
+  Word *const mine = &pend[0][threadIdx.x / kGroup] - kStride;  // level l at mine[l * kStride]
   if (threadIdx.x <= kMaxLevels) off[threadIdx.x] = a.lv.off[threadIdx.x];
   __syncthreads();
   int nent = 0;  // warp-uniform
@@ -453,8 +456,9 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
         if (lv == 0u && gend > 0u) {
           // start at the smallest node that holds p0 and the last position
           const int h = (kWideBits + 31 - __clz((int)(p0 ^ (gend - 1u)))) / kWideBits;
-          const uint32_t top = p0 >> (kWideBits * h);
-          mine[h * kStride] = (top >> kWideBits) << 8 | 1u << (top & 7u);
+          const uint32_t top = kHuge ? (uint32_t)((unsigned long long)p0 >> (kWideBits * h))
+                                     : p0 >> (kWideBits * h);
+          mine[h * kStride] = (Word)(top >> kWideBits) << 8 | 1u << (top & 7u);
           lv = 1u << h;
         }
         if (have < cnt) {
@@ -471,11 +475,11 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
         // spread over the warp instead of holding it.
         if (idle == kFull) break;
         const int hl = lv ? 31 - __clz((int)lv) : 0;
-        const uint32_t word = lv ? mine[hl * kStride] : 0u;
+        const Word word = lv ? mine[hl * kStride] : 0u;
         const bool more = (lv & (lv - 1u)) != 0u;  // a lower level has some too
         idle &= kLead;
         const unsigned donors =
-            __ballot_sync(kFull, more || __popc(word & 0xffu) > 1) & kLead;
+            __ballot_sync(kFull, more || __popc((uint32_t)word & 0xffu) > 1) & kLead;
         const int moves = min(__popc(idle), __popc(donors));
         if (moves > 0) {
           const int lead = lane - sub;  // the group's first lane
@@ -483,8 +487,8 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
           const int ri = __popc(idle & lb), rd = __popc(donors & lb);
           const bool take = ((idle >> lead) & 1u) && ri < moves;
           const bool give = ((donors >> lead) & 1u) && rd < moves;
-          const uint32_t top = 0x80u >> (__clz((int)(word & 0xffu)) - 24);  // last child's bit
-          const uint32_t part = more ? word : (word & ~0xffu) | top;
+          const uint32_t top = 0x80u >> (__clz((int)((uint32_t)word & 0xffu)) - 24);  // last child's bit
+          const Word part = more ? word : (word & ~(Word)0xffu) | top;
           // the receiver of rank k takes from the donor of rank k
           int src = lane;
           if (take) {
@@ -492,7 +496,7 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
             for (int k = 0; k < ri; ++k) m &= m - 1u;
             src = __ffs(m) - 1 + sub;
           }
-          const uint32_t gword = __shfl_sync(kFull, part, src);
+          const Word gword = __shfl_sync(kFull, part, src);
           const int glevel = __shfl_sync(kFull, hl, src);
           p = __shfl_sync(kFull, p, src);
           cend = __shfl_sync(kFull, cend, src);
@@ -519,12 +523,12 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
     // the next pending node of the lowest level
     const bool on = lv != 0u;
     const int l = on ? __ffs(lv) - 1 : 1;
-    const uint32_t word = mine[l * kStride];
+    const Word word = mine[l * kStride];
     __syncwarp();  // read by the whole group before any lane rewrites it
     uint32_t mask = 0, node = 0;
     if (on) {
-      const uint32_t rest = word & (word - 1u);
-      node = (word >> 8) * kWide + (__ffs(word) - 1);
+      const Word rest = word & (word - 1u);
+      node = (uint32_t)(word >> 8) * kWide + (__ffs((int)(uint32_t)word) - 1);
       mine[l * kStride] = rest;
       if (!(rest & 0xffu)) lv &= lv - 1u;
       mask = meet_mask(a.nodes + off[l] + node, qlo, qhi);
@@ -539,7 +543,7 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
     // the children that a query of the group meets
     const uint32_t any = mask | __shfl_xor_sync(kFull, mask, 1);
     if (on && l > 1 && any) {
-      mine[(l - 1) * kStride] = node << 8 | any;
+      mine[(l - 1) * kStride] = (Word)node << 8 | any;
       lv |= 1u << (l - 1);
     }
     __syncwarp();
@@ -595,14 +599,15 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
 }
 
 // persistent: as many blocks as fit on the GPU at once
-template <bool kRefine>
+template <bool kRefine, bool kHuge = false>
 static int launch_traverse(TravArgs &a, cudaStream_t st) {
   static int wave = 0;
   if (!wave) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<kRefine>, kTvThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<kRefine, kHuge>, kTvThreads,
+                                                  0);
     wave = std::max(sms, 1) * std::max(per_sm, 1);
   }
   // sorted boxes and nodes are read with 32-byte loads
@@ -610,7 +615,7 @@ static int launch_traverse(TravArgs &a, cudaStream_t st) {
     return SCD_ERR_INTERNAL;
   a.chunk = kMinChunk;
   while (a.chunk < kMaxChunk && 2 * (int64_t)a.chunk * wave * kTvWarps < a.N) a.chunk *= 2;
-  k_traverse<kRefine><<<(unsigned)wave, kTvThreads, 0, st>>>(a);
+  k_traverse<kRefine, kHuge><<<(unsigned)wave, kTvThreads, 0, st>>>(a);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
@@ -670,7 +675,8 @@ int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   a.rr = s->d_rr.p;
   a.edges = s->d_edges.p;
   a.objT = s->n_scenes > 0 ? s->d_objT.p : nullptr;
-  return launch_traverse<false>(a, s->stream);
+  return a.lv.levels > kWordLevels ? launch_traverse<false, true>(a, s->stream)
+                                   : launch_traverse<false>(a, s->stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -773,9 +779,10 @@ __device__ __forceinline__ unsigned long long end_at(const UnpackArgs &a, unsign
 // before and after it, so that every group is whole; the open runs' ends are
 // looked up afterwards, by the whole block.  Bound by instruction issue (70%),
 // at twice its bytes' time (8 read and 16 written a pair): 24 h catalog, 164 M
-// pairs, 1.35 ms (2.07 with the ends looked up in line and the groups found by
-// comparing neighbours; a separate pass over the keys that sorted the groups in
-// place and a plain unpack took 2.05).
+// pairs, 1.69 ms (4.1 GB of DRAM traffic); 55 M pairs 0.45 (0.69 with the ends
+// looked up in line and the groups found by comparing neighbours).  A separate
+// pass over the keys that sorted the groups in place and a plain unpack took
+// 2.05 ms for the 164 M.
 constexpr int kUpHalo = 256;  // 2^w at most
 
 __global__ void __launch_bounds__(kUpThreads) k_emit(UnpackArgs a) {
