@@ -3,8 +3,8 @@
 Default workload: one 24 h screen of a 16,848-object catalog-shaped
 population at steps P/100.  A step is one pass of the whole hot path from
 device-resident elements to the device-resident canonical pair list:
-per-object steps, FP64 propagation, FP32 boxes and Morton keys, radix sort,
-hierarchy, refit, traversal with merged emission, canonical sort.  The JSON
+per-object steps, FP64 propagation, FP32 boxes and curve keys, radix sort,
+implicit tree, traversal with merged emission, canonical sort.  The JSON
 line's ``value`` is milliseconds per screen (whole job: all ranks' screens
 over the max-rank time); ``e2e`` is the same through the C ABI with host
 buffers (elements copied in, pairs copied out inside the timed region).
@@ -84,15 +84,15 @@ WORKLOADS = {
         "metric": "ms per adaptive-refinement solve at n=512, 6000 s (every collision witness)",
         "desc": ("n=512 uniform LEO (a 6678-8378 km, e < 0.01, i 0-100 deg), r = 2.5 km, 6000 s "
                  "at 1 s ticks: Alg 5-6 as data-parallel rounds from period-bounded first "
-                 "intervals (per round the boxes of all active intervals, their Morton sort, a "
-                 "radix tree and the persistent traversal; all rounds queued without host "
+                 "intervals (per round the boxes of all active intervals, their curve sort, the "
+                 "implicit tree and the persistent traversal; all rounds queued without host "
                  "reads), tick candidates decided by the narrow phase; against the fixed "
                  "10-tick screen plus the narrow phase on the same population")},
     "refine24h": {
         "metric": "ms per 24h adaptive-refinement solve at n=16848 (every collision witness)",
         "desc": ("the n=16848 mixture, 24 h at 1 s ticks: Alg 5-6 as data-parallel rounds from "
                  "period-bounded first intervals (per round the boxes of all active "
-                 "intervals, their Morton sort, a radix tree and the persistent traversal; all "
+                 "intervals, their curve sort, the implicit tree and the persistent traversal; all "
                  "rounds queued without host reads), tick candidates decided by the narrow "
                  "phase; against the fixed P/100 screen plus the narrow phase on the same "
                  "population")},
@@ -211,7 +211,9 @@ class ClockSampler:
 
 def algorithmic_bytes(m: dict, n: int) -> dict:
     """Algorithmic HBM bytes of one screen by phase: every array read or
-    written once per pass that needs it (one box per leaf)."""
+    written once per pass that needs it (one box per leaf).  The hierarchy's
+    terms are a binary tree's (40 bytes a box in the traversal; the implicit
+    tree holds 14), kept so that the fractions compare over time."""
     N = m["boxes"]
     R = m.get("refs") or N  # sorted entries (references when decomposed)
     M = R
@@ -555,13 +557,12 @@ def run_refine(args, world, wl="refine512"):
         # the continuous-time variant at eps = 1 s on the same population
         ctimes, (spans, crb) = timed(lambda: scd.scd_refine_continuous(sc.handle, 1.0),
                                      args.steps, args.warmup)
-    # algorithmic bytes of the rounds, per interval: its box, Morton key and
-    # index written (44 B); six radix passes over key and index (36 B each:
+    # algorithmic bytes of the rounds, per interval: its box, curve key and
+    # index written (44 B); five radix passes over key and index (36 B each:
     # read twice, written once); the gather of the sorted box and object
-    # (76 B); the radix tree's links and parents (40 B) and refit (90 B);
-    # the traversal's sorted box, node and id reads (72 B); flags and the
-    # split's reads and writes (40 B)
-    per_box = 44 + 6 * 36 + 76 + 40 + 90 + 72 + 40
+    # (76 B); the tree's nodes written (14 B); the traversal's sorted box, node,
+    # object and id reads (54 B); flags and the split's reads and writes (40 B)
+    per_box = 44 + 5 * 36 + 76 + 14 + 54 + 40
     byt = int(rb.sum()) * per_box
     ms = statistics.mean(times)
     pk, src = _peaks()

@@ -222,7 +222,7 @@ SCD_API int scd_scene_get_tuning(const scd_scene *s, scd_tuning *t);
  * from one read of the box count.  Errors: KEPLER_NOCONV, OOM, CUDA. */
 SCD_API int scd_build_boxes(scd_scene *s);
 
-/* Steps A5-A10: sort, hierarchy, refit, traversal and canonical list
+/* Steps A5-A10: sort, hierarchy, traversal and canonical list
  * (Sec. 3.2 query semantics; Sec. 5 decomposition when d != NULL and
  * d->kind != NONE).  host_out: host array of cap pairs.  On success *n_out
  * is the number of pairs written.  If cap is too small: BUFFER_TOO_SMALL,

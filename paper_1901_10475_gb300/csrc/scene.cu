@@ -381,7 +381,7 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
       TRY(radix_sort_u32(s->d_key32.p, s->d_id.p, N, kb, s->sort_sc, st));
     }
     if (s->events_ready) cudaEventRecord(s->ev[3], st);
-    // A6-A7: hierarchy and refit
+    // A6-A7: the tree
     TRY(build_hierarchy(s));
   } else {
     // A10: references per cell, their sort, the hierarchy and cell roots
