@@ -313,6 +313,21 @@ __host__ __device__ inline bool box_overlap(const float4 &la, const float4 &ha,
          la.z <= hb.z && lb.z <= ha.z && la.w <= hb.w && lb.w <= ha.w;
 }
 
+// Record slots are numbered in 32 bits, as the record sorts index them: a list
+// whose slots total kSlotLimit or more is refused.
+constexpr unsigned long long kSlotLimit = (1ull << 32) - 1;
+// the slots that a buffer of cap records offers
+inline uint32_t slot_cap(int64_t cap) {
+  return (unsigned long long)cap < kSlotLimit ? (uint32_t)cap : (uint32_t)kSlotLimit;
+}
+// The first slot of a chunk claimed at b.  Totals are whole chunks, so every
+// chunk of a list that is accepted lies below 2^32; one that does not belongs
+// to a list that is refused and goes to the last place where its end does not
+// wrap.
+__host__ __device__ inline uint32_t chunk_first(unsigned long long b, uint32_t chunk) {
+  return b + chunk <= kSlotLimit ? (uint32_t)b : (uint32_t)kSlotLimit - chunk;
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------

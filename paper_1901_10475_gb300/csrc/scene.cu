@@ -409,8 +409,7 @@ static int find_eager(scd_scene *s, const scd_decomp *d, int dkind, int raw_mode
     TRY(read_counters(s));
     unsigned long long need = raw_mode ? s->h_ctr.n_raw
                                        : std::max(s->h_ctr.n_starts, s->h_ctr.n_ends);
-    // the record sort indexes with 32-bit counts
-    if (need >= (1ull << 32) - 1) return SCD_ERR_CAPACITY;
+    if (need >= kSlotLimit) return SCD_ERR_CAPACITY;
     if (need <= (unsigned long long)s->pair_cap) done = true;
     else s->pair_cap = (int64_t)(need + need / 8 + 1024);
     if (N > 0) note_slots_per_box(rkind, N, (double)need / (double)N);

@@ -39,7 +39,7 @@ struct TravArgs {
   uint32_t open_tag;          // last tick of an open run start
   unsigned long long *starts, *ends;
   uint32_t *rawval;           // raw cells' (or unpacked run starts') last tick
-  uint32_t cap;               // record slots (at most 2^32 - 1025)
+  uint32_t cap;               // record slots (slot_cap)
   uint32_t chunk;             // slots reserved at a time
   DevCounters *ctr;
   // static decomposition (kind SCD_DECOMP_NONE: one tree over all boxes)
@@ -93,8 +93,6 @@ constexpr unsigned long long kHole = ~0ull;
 // records).  Every lane of the warp calls put() together; the chunk state is
 // warp-uniform.
 constexpr unsigned kMinChunk = 32, kMaxChunk = 512;
-// (slot numbers in 32 bits: the record sorts take no more, and a list that
-// would need more is refused)
 struct ChunkCursor {
   uint32_t next, end, count;
 };
@@ -116,12 +114,9 @@ __device__ __forceinline__ void chunk_put(ChunkCursor &c, unsigned long long *bu
   uint32_t next = c.next;
   if (next + cnt > c.end) {
     chunk_fill_holes(c, buf, cap);
-    unsigned long long b = 0;
-    if (lane == 0) {
-      b = atomicAdd(slots, (unsigned long long)chunk);
-      if (b > 0xffffffffull - 2 * kMaxChunk) b = 0xffffffffull - 2 * kMaxChunk;  // past any cap
-    }
-    next = __shfl_sync(0xffffffffu, (uint32_t)b, 0);
+    uint32_t b = 0;
+    if (lane == 0) b = chunk_first(atomicAdd(slots, (unsigned long long)chunk), chunk);
+    next = __shfl_sync(0xffffffffu, b, 0);
     if (lane == 0) c.end = next + chunk;
   }
   if (pred) {
@@ -665,7 +660,7 @@ int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   a.starts = s->d_starts.p;
   a.ends = s->d_ends.p;
   a.rawval = s->d_rawval.p;
-  a.cap = (uint32_t)std::min<int64_t>(s->pair_cap, 0xffffffffll - 2 * kMaxChunk);
+  a.cap = slot_cap(s->pair_cap);
   a.ctr = s->d_ctr.p;
   a.dkind = s->dkind;
   a.n_slabs = s->n_slabs;
