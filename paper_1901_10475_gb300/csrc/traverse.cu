@@ -689,6 +689,8 @@ struct UnpackArgs {
   const unsigned long long *d_n;     // the count, when known on the device only
   unsigned long long n_ends;         // ends (a capacity when d_ne is set)
   const unsigned long long *d_ne;
+  // the slots handed out for starts and ends, when known on the device only
+  const unsigned long long *d_sslots, *d_eslots;
   int ob, tb;
   int packed, raw;
   int w;                             // lowest tick bits the sorts left out
@@ -704,6 +706,13 @@ __device__ __forceinline__ int64_t unpack_count(const UnpackArgs &a) {
   return a.d_n && *a.d_n < (unsigned long long)a.n ? (int64_t)*a.d_n : a.n;
 }
 
+// Counts from the device (a replayed find) may have outgrown the capacities they
+// were captured for: records are missing then, and holes stand among the first n.
+// Nothing is emitted; the host sees the same counts and runs the find again.
+__device__ __forceinline__ bool outgrown(const UnpackArgs &a) {
+  return a.d_n && (*a.d_sslots > (unsigned long long)a.n || *a.d_eslots > a.n_ends);
+}
+
 __device__ __forceinline__ uint32_t last_of(const UnpackArgs &a, unsigned long long key,
                                             int64_t r) {
   return a.packed ? (uint32_t)(key & ((1ull << a.tb) - 1ull)) : __ldg(a.lastv + r);
@@ -714,6 +723,7 @@ __device__ __forceinline__ uint32_t last_of(const UnpackArgs &a, unsigned long l
 
 // open starts per tile
 __global__ void __launch_bounds__(kUpThreads) k_open_count(UnpackArgs a) {
+  if (outgrown(a)) return;  // (the prefix over the tiles is not read either)
   const int64_t n = unpack_count(a);
   __shared__ uint32_t ws[kUpThreads / 32];
   // (past a device count: zeros, which the prefix over all tiles reads)
@@ -746,23 +756,26 @@ static_assert(kUpItems * (kUpThreads / 32) == 64, "the tile prefix takes two cou
 
 // The r-th end in sorted order: the ends stand in the order of (i, j, tick >>
 // w), so it is the (r - g0)-th smallest of its group of equal prefixes, which
-// starts at g0 (nearly always the end alone).
+// starts at g0 (nearly always the end alone).  Ends are distinct, so a group has
+// at most 2^w; holes or a longer group are no end (kHole, which no start zips
+// with), found within 2^w loads.
 __device__ __forceinline__ unsigned long long end_at(const UnpackArgs &a, unsigned long long r,
                                                      unsigned long long n_ends) {
   const unsigned long long e = __ldg(a.ends + r);
-  if (a.w == 0) return e;
-  const unsigned long long pre = e >> a.w;
+  if (a.w == 0 || e == kHole) return e;
+  const unsigned long long pre = e >> a.w, most = 1ull << a.w;
   unsigned long long g0 = r, g1 = r + 1;
-  while (g0 > 0 && (__ldg(a.ends + g0 - 1) >> a.w) == pre) --g0;
-  while (g1 < n_ends && (__ldg(a.ends + g1) >> a.w) == pre) ++g1;
+  while (g0 > 0 && g1 - g0 <= most && (__ldg(a.ends + g0 - 1) >> a.w) == pre) --g0;
+  while (g1 < n_ends && g1 - g0 <= most && (__ldg(a.ends + g1) >> a.w) == pre) ++g1;
   if (g1 - g0 == 1) return e;
+  if (g1 - g0 > most) return kHole;
   for (unsigned long long x = g0; x < g1; ++x) {
     const unsigned long long v = __ldg(a.ends + x);
     unsigned long long less = 0;
     for (unsigned long long y = g0; y < g1; ++y) less += __ldg(a.ends + y) < v;
     if (less == r - g0) return v;
   }
-  return e;  // not reached: the ends are distinct
+  return kHole;  // ends that are not distinct
 }
 
 // The starts, sorted by all but the lowest w bits of their tick, as pairs in
@@ -790,6 +803,7 @@ __global__ void __launch_bounds__(kUpThreads) k_emit(UnpackArgs a) {
   __shared__ uint32_t same[kUpItems * kWarps + 2];
   __shared__ uint2 opens[kUpTile];  // open starts: slot | place + halo << 16, rank among the opens
   __shared__ int nopen;
+  if (outgrown(a)) return;
   const int64_t n = unpack_count(a);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned long long tmask = (1ull << a.tb) - 1ull, omask = (1ull << a.ob) - 1ull;
@@ -862,8 +876,10 @@ __global__ void __launch_bounds__(kUpThreads) k_emit(UnpackArgs a) {
         int g1 = x + above + 1;
         if (below > 31 || above > 31 || g0 <= 0 || g1 >= kUpTile) {
           // longer, or at the tile's edge: along the keys
-          for (g0 = x; g0 > first && (ks[halo + g0 - 1] ^ key) < group_size;) --g0;
-          for (g1 = x + 1; g1 < last && (ks[halo + g1] ^ key) < group_size;) ++g1;
+          // (2^w either way at most: more would not be records)
+          const int from = max(first, x - halo), to = min(last, x + 1 + halo);
+          for (g0 = x; g0 > from && (ks[halo + g0 - 1] ^ key) < group_size;) --g0;
+          for (g1 = x + 1; g1 < to && (ks[halo + g1] ^ key) < group_size;) ++g1;
         }
         if (g1 - g0 > 1)
           for (int y = g0; y < g1; ++y) {
@@ -1133,6 +1149,8 @@ int canonicalize_dev(scd_scene *s, int obj_bits, int t_bits) {
   a.d_n = &c->v_starts;
   a.n_ends = (unsigned long long)cap;
   a.d_ne = &c->v_ends;
+  a.d_sslots = &c->n_starts;
+  a.d_eslots = &c->n_ends;
   if (int rc2 = unpack(s, a, st)) return rc2;
   return cudaGetLastError() == cudaSuccess ? SCD_OK : SCD_ERR_CUDA;
 }
