@@ -334,13 +334,20 @@ __host__ __device__ inline uint32_t chunk_first(unsigned long long b, uint32_t c
 
 void *dev_alloc(size_t bytes, cudaStream_t st);
 void dev_free(void *p, cudaStream_t st);
+// one more than any stamp handed out before in this process
+unsigned long long next_stamp();
 
 template <class T>
 struct DevBuf {
   T *p = nullptr;
   size_t n = 0;
+  // of the memory held: a later one whenever p changes.  A captured graph holds
+  // the buffers' addresses; it is good while the sum of their stamps is the same
+  // (the addresses themselves would not do: freed memory may come back smaller).
+  unsigned long long stamp = 0;
   bool ensure(size_t count, cudaStream_t st) {
     if (count <= n && p) return true;
+    stamp = next_stamp();
     if (p) dev_free(p, st);
     p = nullptr;
     n = 0;
@@ -360,13 +367,17 @@ struct DevBuf {
       dev_free(q, st);
       return false;
     }
+    stamp = next_stamp();
     if (p) dev_free(p, st);
     p = q;
     n = count < 1 ? 1 : count;
     return true;
   }
   void release(cudaStream_t st) {
-    if (p) dev_free(p, st);
+    if (p) {
+      stamp = next_stamp();
+      dev_free(p, st);
+    }
     p = nullptr;
     n = 0;
   }
@@ -379,11 +390,15 @@ struct SortScratch {
   DevBuf<uint32_t> counts;
   DevBuf<uint32_t> ocounts;  // open run starts per digit and tile (last pass into pairs)
   unsigned int *err = nullptr;  // device word that receives ERR_SORT (may be null)
+  template <class F>
+  void each(F f) {
+    f(keys_alt);
+    f(vals_alt);
+    f(counts);
+    f(ocounts);
+  }
   void release(cudaStream_t st) {
-    keys_alt.release(st);
-    vals_alt.release(st);
-    counts.release(st);
-    ocounts.release(st);
+    each([st](auto &b) { b.release(st); });
   }
 };
 

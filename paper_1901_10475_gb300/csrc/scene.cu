@@ -25,6 +25,9 @@ namespace scd {
 void note_launch(int k) { g_launches.fetch_add((unsigned long long)k); }
 unsigned long long launch_count() { return g_launches.load(); }
 
+static std::atomic<unsigned long long> g_stamps{0};
+unsigned long long next_stamp() { return g_stamps.fetch_add(1) + 1; }
+
 void *dev_alloc(size_t bytes, cudaStream_t st) {
   if (g_alloc) return g_alloc(bytes, (void *)st, g_alloc_ctx);
   void *p = nullptr;
@@ -470,12 +473,30 @@ static int enqueue_find(scd_scene *s, const scd_decomp *d, int dkind, int ob, in
   return SCD_OK;
 }
 
-static void graph_key_of(const scd_scene *s, int64_t key[8]) {
+// every buffer that a find reads or writes on the device
+template <class F>
+static void find_buffers(scd_scene *s, F f) {
+  f(s->d_el); f(s->d_par); f(s->d_k); f(s->d_segcnt); f(s->d_segoff); f(s->d_scan_tmp);
+  f(s->d_band); f(s->d_ctr);
+  f(s->d_lo); f(s->d_hi); f(s->d_obj); f(s->d_key64); f(s->d_key32); f(s->d_id);
+  f(s->s_box); f(s->d_posof); f(s->s_link); f(s->s_cell); f(s->d_nodes); f(s->d_nbox);
+  f(s->d_refcnt); f(s->d_refoff); f(s->d_refkey); f(s->d_refid); f(s->d_rr); f(s->d_edges);
+  f(s->d_abits); f(s->d_cellend);
+  f(s->d_objT); f(s->d_objscene); f(s->d_sceneoff); f(s->d_pairoff);
+  f(s->d_starts); f(s->d_ends); f(s->d_rawval); f(s->d_tilecnt); f(s->d_out);
+  s->sort_sc.each(f);
+  s->ends_sc.each(f);
+}
+
+// sizes and tuning that the captured launches hold, and the buffers
+static void graph_key_of(scd_scene *s, int64_t key[8]) {
+  unsigned long long stamps = 0;
+  find_buffers(s, [&stamps](const auto &b) { stamps += b.stamp; });
   key[0] = s->dkind;
   key[1] = s->n_slabs * 100000 + s->p_bands;
   key[2] = s->N;
   key[3] = s->pair_cap;
-  key[4] = 0;
+  key[4] = (int64_t)stamps;
   key[5] = s->tune.morton_bits * 10 + s->tune.space_warp;
   key[6] = (int64_t)(s->tune.time_scale * 1e6f) * 1000000 + (int64_t)(split_of(s->tune) * 10.0f);
   key[7] = s->dkind ? s->n_refs : 0;
@@ -516,8 +537,8 @@ static int find_graph(scd_scene *s, const scd_decomp *d, int dkind, int ob, int 
       finish_metrics(s, 0);
       return SCD_OK;
     }
-    s->graph_ok = false;
   }
+  s->graph_ok = false;  // whatever the eager run and the capture come to
   // eager run (sizes every buffer; its result is the answer), then capture
   TRY(find_eager(s, d, dkind, 0, ob, tb));
   s->last_graph = 0;
@@ -746,28 +767,10 @@ extern "C" SCD_API void scd_scene_destroy(scd_scene *s) {
   if (!s) return;
   cudaStream_t st = s->stream;
   cudaStreamSynchronize(st);
-  s->d_el.release(st); s->d_par.release(st); s->d_k.release(st);
-  s->d_segcnt.release(st); s->d_segoff.release(st); s->d_scan_tmp.release(st);
-  s->d_band.release(st); s->d_ctr.release(st);
-  s->d_lo.release(st); s->d_hi.release(st); s->d_obj.release(st);
-  s->d_key64.release(st); s->d_key32.release(st); s->d_id.release(st);
-  s->s_box.release(st);
-  s->d_posof.release(st); s->s_link.release(st);
-  s->d_nodes.release(st); s->d_nbox.release(st);
-  s->d_starts.release(st); s->d_ends.release(st); s->d_rawval.release(st);
-  s->d_tilecnt.release(st);
-  s->d_out.release(st);
+  find_buffers(s, [st](auto &b) { b.release(st); });
   s->d_narrow.release(st);
   s->d_npobj.release(st);
-  s->sort_sc.release(st);
-  s->ends_sc.release(st);
-  s->s_cell.release(st);
-  s->d_refcnt.release(st); s->d_refoff.release(st); s->d_refkey.release(st);
-  s->d_refid.release(st); s->d_rr.release(st); s->d_edges.release(st);
-  s->d_abits.release(st); s->d_cellend.release(st);
   s->d_feat.release(st); s->d_ny.release(st); s->d_learned.release(st);
-  s->d_objT.release(st); s->d_objscene.release(st); s->d_sceneoff.release(st);
-  s->d_pairoff.release(st);
   s->d_part.release(st); s->d_parte.release(st);
   rf_release(s);
   if (s->events_ready)
