@@ -403,20 +403,24 @@ struct RfBuffers {
   // and the scratch of the sorts after the rounds
   SortScratch sc, sc_post;
   explicit RfBuffers(cudaStream_t s) : st(s) {}
-  ~RfBuffers() {
+  // the buffers of the rounds' queue (which a captured graph holds) ...
+  template <class F>
+  void each_round(F f) {
     for (int b = 0; b < 2; ++b) {
-      obj[b].release(st);
-      t0[b].release(st);
-      t1[b].release(st);
+      f(obj[b]);
+      f(t0[b]);
+      f(t1[b]);
     }
-    idx.release(st); flags.release(st); sobj.release(st); first.release(st);
-    lo.release(st); hi.release(st); key.release(st); cand.release(st); state.release(st);
-    wkey.release(st); sbox.release(st); nbox.release(st); nodes.release(st);
-    ctr.release(st); sort_err.release(st); pairs.release(st);
-    wit.release(st); span.release(st); tlo.release(st); thi.release(st); tobj.release(st);
-    scnt.release(st); soff.release(st); stmp.release(st);
-    sc.release(st);
-    sc_post.release(st);
+    f(idx); f(flags); f(sobj); f(lo); f(hi); f(key); f(cand); f(state); f(sbox); f(nbox);
+    f(nodes); f(ctr); f(sort_err); f(tlo); f(thi); f(tobj); f(soff);
+    sc.each(f);
+  }
+  ~RfBuffers() {
+    auto rel = [this](auto &b) { b.release(st); };
+    each_round(rel);
+    // ... and the ones around it
+    rel(first); rel(wkey); rel(pairs); rel(wit); rel(span); rel(scnt); rel(stmp);
+    sc_post.each(rel);
   }
   // every per-interval buffer for `cap` intervals a round, and `ccap`
   // candidates
@@ -596,7 +600,7 @@ struct RfCache {
   cudaStream_t gst = nullptr;
   cudaEvent_t in = nullptr, out = nullptr;
   cudaGraphExec_t exec = nullptr;
-  int64_t key[11] = {};
+  int64_t key[10] = {};
   unsigned long long nlaunch = 0;  // kernels in the graph
   explicit RfCache(cudaStream_t st) : B(st) {}
   ~RfCache() {
@@ -610,21 +614,23 @@ struct RfCache {
   }
 };
 
-static void rf_key(const scd_scene *s, const RfBuffers &B, int64_t cap, int64_t ccap, int rounds,
-                   int levels, int64_t k[11]) {
+static void rf_key(const scd_scene *s, RfBuffers &B, int64_t cap, int64_t ccap, int rounds,
+                   int levels, int64_t k[10]) {
+  // (a call that ran out of memory may have moved buffers and kept the sizes)
+  unsigned long long stamps = s->d_par.stamp;
+  B.each_round([&stamps](const auto &b) { stamps += b.stamp; });
   k[0] = cap;
   k[1] = ccap;
-  k[2] = 0;
+  k[2] = (int64_t)stamps;
   k[3] = rounds;
   k[4] = levels;
   k[5] = s->n;
   k[6] = s->T;
   k[7] = s->box_mode * 1000000 + (int64_t)(split_of(s->tune) * 10.0f);
-  k[8] = (int64_t)reinterpret_cast<uintptr_t>(B.obj[0].p) ^ (int64_t)reinterpret_cast<uintptr_t>(s->d_par.p);
   int64_t tb;
   memcpy(&tb, &s->tick_s, sizeof(tb));
-  k[9] = tb;
-  k[10] = (int64_t)(rf_start_unit(s) * 1e6);  // baked into the first round's launch
+  k[8] = tb;
+  k[9] = (int64_t)(rf_start_unit(s) * 1e6);  // baked into the first round's launch
 }
 
 // queue the rounds: by the cached graph when its shape matches, else
@@ -633,7 +639,7 @@ static int rf_rounds(scd_scene *s, RfBuffers &B, RfCache *gc, int64_t cap, int64
                      int rounds, int levels, unsigned long long h[RF_WORDS],
                      unsigned long long *round_counts, unsigned long long &most,
                      unsigned long long &left) {
-  int64_t k[11];
+  int64_t k[10];
   rf_key(s, B, cap, ccap, rounds, levels, k);
   if (gc && gc->exec && memcmp(k, gc->key, sizeof(k)) == 0) {
     if (cudaEventRecord(gc->in, B.st) != cudaSuccess ||
@@ -732,7 +738,7 @@ static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int leve
       s->rf_cap = cap;
       s->rf_ccap = ccap;
       if (gc) {
-        int64_t k[11];
+        int64_t k[10];
         rf_key(s, B, cap, ccap, rounds, levels, k);
         if (!gc->exec || memcmp(k, gc->key, sizeof(k)) != 0)
           rf_capture(s, *gc, cap, ccap, rounds, levels);
