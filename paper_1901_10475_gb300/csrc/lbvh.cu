@@ -235,14 +235,9 @@ int64_t tree_scratch_boxes(int64_t cap) {
 
 // the launches of one tree: level 0 with the gather, then three levels each
 static int launch_tree(TreeArgs a, SBox *nbox, cudaStream_t st) {
-  static int wave = 0;
-  if (!wave) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree<true>, kTreeThreads, 0);
-    wave = std::max(1, sms) * std::max(1, per_sm);
-  }
+  static PerDevice waves;
+  const int wave =
+      waves.get(current_device(), [] { return resident_blocks(k_tree<true>, kTreeThreads); });
   if (a.n > kMaxTreeBoxes) return SCD_ERR_CAPACITY;
   a.lv = tree_levels(a.n);
   int64_t tiles = (a.n + kTreeThreads - 1) / kTreeThreads;

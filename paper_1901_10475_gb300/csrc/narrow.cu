@@ -467,10 +467,9 @@ extern "C" SCD_API int scd_narrow_phase(scd_scene *s, const scd_pair *d_pairs, i
     k_np_objects<<<(unsigned)((s->n + 31) / 32), 32, 0, s->stream>>>(s->d_par.p, s->n, s->tick_s,
                                                                       obj, s->d_narrow.p);
     note_launch();
-    static int per_sm = 0, sms = 0;
-    if (!per_sm) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_narrow, kNpThreads, 0);
-    if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-    int64_t blocks = (int64_t)std::max(sms, 1) * std::max(per_sm, 1);
+    static PerDevice waves;
+    int64_t blocks =
+        waves.get(current_device(), [] { return resident_blocks(k_narrow, kNpThreads); });
     constexpr int kPerBlock = kNpMinClaim * (kNpThreads / 32);
     const int64_t need = (n_pairs + kPerBlock - 1) / kPerBlock;
     if (need < blocks) blocks = need;

@@ -696,8 +696,8 @@ static int rs_cluster(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  static int fits = -1;
-  if (fits < 0) {
+  static PerDevice of;
+  const int fits = of.get(current_device(), [&] {
     int clusters = 0;
     const bool ok =
         cudaFuncSetAttribute(k_rs_cluster<K, kVals>,
@@ -706,24 +706,14 @@ static int rs_cluster(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
                              (int)cfg.dynamicSmemBytes) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, k_rs_cluster<K, kVals>, &cfg) == cudaSuccess;
     if (!ok) cudaGetLastError();
-    fits = ok && clusters > 0;
-  }
+    return (int)(ok && clusters > 0);
+  });
   if (!fits) return SCD_ERR_STATE;
   if (cudaLaunchKernelEx(&cfg, k_rs_cluster<K, kVals>, keys, vals, keys_alt, vals_alt, n, d_n, lo,
                          bits) != cudaSuccess)
     return SCD_ERR_CUDA;
   note_launch();
   return SCD_OK;
-}
-
-static int rs_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return std::max(1, sms);
 }
 
 // the scan of 256 digits' rows of nblk counts
@@ -764,40 +754,24 @@ static int rs_impl(K *keys, uint32_t *vals, int64_t n, const unsigned long long 
   // two tile buffers of keys (and values); persistent grid of the blocks
   // that fit at once
   size_t smem = 2 * (sizeof(K) * tile + (vals ? sizeof(uint32_t) * tile : 0));
-  static int grid_of[2][2] = {{0, 0}, {0, 0}};
-  int ki = sizeof(K) == 8 ? 1 : 0, vi = vals ? 1 : 0;
-  if (!grid_of[ki][vi]) {
-    int sms = 0, per_sm = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (vals) {
-      cudaFuncSetAttribute(k_rs_downsweep<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rs_downsweep<K, true>, kRsThreads,
-                                                    smem);
-    } else {
-      cudaFuncSetAttribute(k_rs_downsweep<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rs_downsweep<K, false>,
-                                                    kRsThreads, smem);
-    }
-    grid_of[ki][vi] = std::max(1, sms) * std::max(1, per_sm);
-  }
-  const unsigned grid = (unsigned)std::min<int64_t>(nblk, grid_of[ki][vi]);
+  static PerDevice waves[2];  // (of each key type: keys alone, with values)
+  const int wave = waves[vals != nullptr].get(current_device(), [&] {
+    return vals ? resident_blocks(k_rs_downsweep<K, true>, kRsThreads, smem)
+                : resident_blocks(k_rs_downsweep<K, false>, kRsThreads, smem);
+  });
+  const unsigned grid = (unsigned)std::min<int64_t>(nblk, wave);
   // the counting pass: a block a tile, or with a device count as many as the
   // SMs hold (eight of 256 threads)
-  const unsigned ugrid = (unsigned)(d_n ? std::min<int64_t>(nblk, 8 * rs_sms()) : nblk);
+  const unsigned ugrid = (unsigned)(d_n ? std::min<int64_t>(nblk, 8 * device_sms()) : nblk);
   uint32_t *ocounts = nullptr, *ototals = nullptr;
   if (pe) {
     if (!sc.ocounts.ensure((size_t)(256 * nblk + 256), st)) return SCD_ERR_OOM;
     ocounts = sc.ocounts.p;
     ototals = sc.ocounts.p + 256 * nblk;
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_rs_downsweep<unsigned long long, false, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attr = true;
-    }
+    static PerDevice pairs;  // (the opt-in; the grid is the keys')
+    pairs.get(current_device(), [&] {
+      return resident_blocks(k_rs_downsweep<unsigned long long, false, true>, kRsThreads, smem);
+    });
   }
   int passes = 0;
   for (int shift = lo; shift < bits; shift += 8, ++passes) {
@@ -859,17 +833,10 @@ int radix_partition_u64(const unsigned long long *kin, unsigned long long *kout,
   if (!sc.counts.ensure((size_t)(256 * nblk + 256), st)) return SCD_ERR_OOM;
   uint32_t *counts = sc.counts.p, *totals = sc.counts.p + 256 * nblk;
   const size_t smem = 2 * sizeof(unsigned long long) * tile;
-  static int grid = 0;
-  if (!grid) {
-    int sms = 0, per_sm = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_rs_downsweep<unsigned long long, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rs_downsweep<unsigned long long, false>,
-                                                  kRsThreads, smem);
-    grid = std::max(1, sms) * std::max(1, per_sm);
-  }
+  static PerDevice waves;
+  const int grid = waves.get(current_device(), [&] {
+    return resident_blocks(k_rs_downsweep<unsigned long long, false>, kRsThreads, smem);
+  });
   k_rs_upsweep<unsigned long long, false>
       <<<(unsigned)nblk, kRsThreads, 0, st>>>(kin, n, nullptr, shift, counts, nblk);
   rs_scan(counts, nblk, totals, nullptr, 0, tile, st);

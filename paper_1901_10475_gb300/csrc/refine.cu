@@ -443,13 +443,7 @@ static unsigned grid_of(int64_t n) { return (unsigned)((n + kRfThreads - 1) / kR
 // resident at once, or fewer (its threads loop over the round's count, read
 // on the device, so an almost empty round costs one short wave)
 static unsigned wave_of(int64_t n) {
-  static int wave = 0;
-  if (!wave) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    wave = std::max(1, sms) * (2048 / kRfThreads);
-  }
+  const int wave = device_sms() * (2048 / kRfThreads);
   return std::min<unsigned>(grid_of(std::max<int64_t>(n, 1)), (unsigned)wave);
 }
 

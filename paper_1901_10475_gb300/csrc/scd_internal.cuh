@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "../../include/scd.h"
@@ -331,6 +333,47 @@ __host__ __device__ inline uint32_t chunk_first(unsigned long long b, uint32_t c
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
+
+// Launch set-up that belongs to a device (resident blocks, a kernel's opt-in to
+// large shared memory or clusters): made on a device's first use, by whichever
+// thread gets there first, and once per device, as attributes are.
+class PerDevice {
+  static constexpr int kMax = 64;
+  std::once_flag once_[kMax];
+  int value_[kMax] = {};
+
+ public:
+  template <class F>
+  int get(int dev, F make) {
+    if (dev < 0 || dev >= kMax) return make();
+    std::call_once(once_[dev], [&] { value_[dev] = make(); });
+    return value_[dev];
+  }
+};
+inline int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+inline int device_sms() {
+  static PerDevice of;
+  const int dev = current_device();
+  return of.get(dev, [dev] {
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, sms);
+  });
+}
+// blocks of a kernel that the current device holds at once (smem: dynamic
+// shared memory, opted in to)
+template <class Kernel>
+inline int resident_blocks(Kernel kernel, int threads, size_t smem = 0) {
+  int per_sm = 0;
+  if (smem > 0)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+  return device_sms() * std::max(1, per_sm);
+}
 
 void *dev_alloc(size_t bytes, cudaStream_t st);
 void dev_free(void *p, cudaStream_t st);

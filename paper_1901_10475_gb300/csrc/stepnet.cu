@@ -527,16 +527,9 @@ extern "C" SCD_API int scd_stepnet_forward(const scd_stepnet *n, const float *d_
 static int train_pass(scd_stepnet *n, const float *d_x, const float *d_t, int64_t count, float *g,
                       const AdamArgs *adam) {
   cudaStream_t st = n->stream;
-  static int wave = 0;
-  if (!wave) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_fwd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(TrainSmem));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_bwd, kTT, sizeof(TrainSmem));
-    wave = std::max(sms, 1) * std::max(per_sm, 1);
-  }
+  static PerDevice waves;
+  const int wave = waves.get(
+      current_device(), [] { return resident_blocks(k_fwd_bwd, kTT, sizeof(TrainSmem)); });
   const int blocks = (int)std::min<int64_t>((count + kTS - 1) / kTS, wave);
   if (!n->part.ensure((size_t)blocks * kPart, st)) return SCD_ERR_OOM;
   k_fwd_bwd<<<blocks, kTT, sizeof(TrainSmem), st>>>(view(n), d_x, d_t, count,

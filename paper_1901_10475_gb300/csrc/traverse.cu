@@ -596,15 +596,9 @@ __global__ void __launch_bounds__(kTvThreads, 8) k_traverse(TravArgs a) {
 // persistent: as many blocks as fit on the GPU at once
 template <bool kRefine, bool kHuge = false>
 static int launch_traverse(TravArgs &a, cudaStream_t st) {
-  static int wave = 0;
-  if (!wave) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traverse<kRefine, kHuge>, kTvThreads,
-                                                  0);
-    wave = std::max(sms, 1) * std::max(per_sm, 1);
-  }
+  static PerDevice waves;
+  const int wave = waves.get(
+      current_device(), [] { return resident_blocks(k_traverse<kRefine, kHuge>, kTvThreads); });
   // sorted boxes and nodes are read with 32-byte loads
   if ((reinterpret_cast<uintptr_t>(a.sbox) | reinterpret_cast<uintptr_t>(a.nodes)) & 31)
     return SCD_ERR_INTERNAL;
@@ -973,11 +967,9 @@ static PairEmit pair_emit(scd_scene *s, int obj_bits, int t_bits, const unsigned
 static int unpack(scd_scene *s, UnpackArgs a, cudaStream_t st) {
   a.tiles = (a.n + kUpTile - 1) / kUpTile;
   if (a.tiles == 0) return SCD_OK;
-  static int sms = 0;
-  if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
   // a block a tile, or with a device count as many as the SMs hold
   const unsigned grid =
-      (unsigned)(a.d_n ? std::min<int64_t>(a.tiles, 8 * std::max(1, sms)) : a.tiles);
+      (unsigned)(a.d_n ? std::min<int64_t>(a.tiles, 8 * device_sms()) : a.tiles);
   if (!a.raw) {
     if (!s->d_tilecnt.ensure((size_t)a.tiles + 1, st)) return SCD_ERR_OOM;
     a.bcnt = s->d_tilecnt.p;

@@ -33,3 +33,13 @@ def test_chunks_past_the_limit_do_not_wrap(rules, chunk):
     for b in (2**32 - chunk, 2**32, 2**33 + chunk, 2**63):
         assert rules.rule_chunk_first(b, chunk) + chunk < 2**32
     assert rules.rule_slot_cap(2**33) < 2**32
+
+
+def test_launch_setup_is_made_once_per_device(rules):
+    made = (C.c_int * 16)()
+    assert rules.rule_per_device(16, 8, made) == 1
+    assert list(made) == [1] * 16
+    # (past the table: made on every use)
+    made = (C.c_int * 65)()
+    assert rules.rule_per_device(65, 1, made) == 1
+    assert list(made) == [1] * 65
