@@ -426,9 +426,9 @@ struct RfBuffers {
   // candidates
   bool size(int64_t cap, int64_t ccap) {
     const size_t c = (size_t)cap;
+    if (cap > kMaxRoundBoxes) return false;
     for (int b = 0; b < 2; ++b)
       if (!obj[b].ensure(c, st) || !t0[b].ensure(c, st) || !t1[b].ensure(c, st)) return false;
-    if (cap > kMaxRoundBoxes) return false;
     return idx.ensure(c, st) && flags.ensure(c, st) && sobj.ensure(c, st) && lo.ensure(c, st) &&
            hi.ensure(c, st) && key.ensure(c, st) && sbox.ensure(c, st) &&
            nbox.ensure((size_t)tree_scratch_boxes(cap), st) &&
@@ -721,7 +721,7 @@ static int rf_run(scd_scene *s, RfBuffers &B, RfCache *gc, int &rounds, int leve
     if (rc != SCD_OK) return rc;
     bool again = false;
     if (most > (unsigned long long)cap) {
-      cap = (int64_t)std::max<unsigned long long>(2ull * (unsigned long long)cap, 2ull * most);
+      cap = rf_grown(cap, most);
       again = true;
     }
     if (h[RF_NCAND] > (unsigned long long)ccap) {

@@ -284,6 +284,12 @@ inline int sort_key_bits(const scd_tuning &t) {
 // variant, i (20) | j (20) | the later start (22) | whether the starts agree
 // (1), which sorts by (i, j, t0, t1) of the intersection.
 constexpr uint32_t kRfHit = 1u, kRfHitLong = 2u;
+// the capacity to try next when a round asked for `most` intervals of `cap`:
+// twice either, within what a round's tree takes while that suffices
+inline int64_t rf_grown(int64_t cap, unsigned long long most) {
+  const unsigned long long twice = std::max(2ull * (unsigned long long)cap, 2ull * most);
+  return (int64_t)std::min(twice, std::max(most, (unsigned long long)kMaxRoundBoxes));
+}
 __host__ __device__ inline unsigned long long rf_tick_key(uint32_t t, uint32_t i, uint32_t j) {
   return ((unsigned long long)t << 40) | ((unsigned long long)i << 20) | (unsigned long long)j;
 }

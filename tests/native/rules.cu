@@ -14,6 +14,10 @@ uint32_t rule_chunk_first(unsigned long long b, uint32_t chunk) {
   return scd::chunk_first(b, chunk);
 }
 
+// refinement: the next capacity to try, and the most intervals a round takes
+int64_t rule_rf_grown(int64_t cap, unsigned long long most) { return scd::rf_grown(cap, most); }
+int64_t rule_round_limit() { return scd::kMaxRoundBoxes; }
+
 // Launch set-up of `devices` devices asked for by `threads` threads at once: how
 // often each device's was made (made[dev]); 1 if every answer was its device's.
 int rule_per_device(int devices, int threads, int *made) {

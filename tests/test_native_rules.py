@@ -14,6 +14,8 @@ def rules(tmp_path_factory):
     m.rule_slot_cap.argtypes = [C.c_int64]
     m.rule_chunk_first.restype = C.c_uint32
     m.rule_chunk_first.argtypes = [C.c_ulonglong, C.c_uint32]
+    m.rule_rf_grown.restype = m.rule_round_limit.restype = C.c_int64
+    m.rule_rf_grown.argtypes = [C.c_int64, C.c_ulonglong]
     return m
 
 
@@ -43,3 +45,14 @@ def test_launch_setup_is_made_once_per_device(rules):
     made = (C.c_int * 65)()
     assert rules.rule_per_device(65, 1, made) == 1
     assert list(made) == [1] * 65
+
+
+def test_a_round_that_fits_is_not_refused_for_its_retry(rules):
+    limit = rules.rule_round_limit()
+    assert limit == 2**30
+    for cap in (1 << 16, 10**6, 2**29 + 1, limit - 1):
+        for most in (cap + 1, 2 * cap, 2**29, limit - 1, limit):
+            if cap < most <= limit:
+                assert most <= rules.rule_rf_grown(cap, most) <= limit
+        assert rules.rule_rf_grown(cap, limit + 1) > limit  # refused
+    assert rules.rule_rf_grown(1 << 16, 100_000) == 200_000
