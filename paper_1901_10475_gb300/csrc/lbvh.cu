@@ -238,7 +238,6 @@ static int launch_tree(TreeArgs a, SBox *nbox, cudaStream_t st) {
   static PerDevice waves;
   const int wave =
       waves.get(current_device(), [] { return resident_blocks(k_tree<true>, kTreeThreads); });
-  if (a.n > kMaxTreeBoxes) return SCD_ERR_CAPACITY;
   a.lv = tree_levels(a.n);
   int64_t tiles = (a.n + kTreeThreads - 1) / kTreeThreads;
   uint32_t *const finish = a.finish;
@@ -266,7 +265,6 @@ int build_tree(scd_scene *s, const unsigned long long *keys_sorted, const uint32
                int64_t Nq, int cell_shift) {
   cudaStream_t st = s->stream;
   const bool cells = cell_shift >= 0;
-  if (Nq > kMaxTreeBoxes) return SCD_ERR_CAPACITY;
   if (!s->s_box.ensure(Nq, st) || !s->d_posof.ensure(s->N, st) || !s->s_link.ensure(Nq, st) ||
       !s->d_nodes.ensure(tree_levels(Nq).total, st) ||
       !s->d_nbox.ensure(tree_scratch_boxes(Nq), st) || (cells && !s->s_cell.ensure(Nq, st)))

@@ -266,9 +266,8 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 4 : 3) k_rs_downsweep(
   gdig[d] = digit_scan_excl(even ? (totals[d] + 1u) & ~1u : totals[d], scanbuf);
   if constexpr (kPairs) odig[d] = digit_scan_excl(ototals[d], scanbuf);
   const unsigned long long tmask = kPairs ? (1ull << pe.tb) - 1ull : 0ull;
-  const int64_t nvalid = kPairs ? sort_count(pe.n, pe.d_n) : 0;
-  const unsigned long long n_ends =
-      kPairs ? (pe.d_ne && *pe.d_ne < pe.n_ends ? *pe.d_ne : pe.n_ends) : 0ull;
+  const int64_t nvalid = kPairs ? pe.n : 0;
+  const unsigned long long n_ends = kPairs ? pe.n_ends : 0ull;
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -880,9 +879,9 @@ int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaSt
   return SCD_OK;
 }
 
-int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, const unsigned long long *d_n,
-                         int lo, int bits, SortScratch &sc, const PairEmit &pe, cudaStream_t st) {
-  return rs_impl<unsigned long long>(keys, nullptr, n, d_n, lo, bits, sc, st, &pe);
+int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, int lo, int bits, SortScratch &sc,
+                         const PairEmit &pe, cudaStream_t st) {
+  return rs_impl<unsigned long long>(keys, nullptr, n, nullptr, lo, bits, sc, st, &pe);
 }
 
 int radix_sort_u64_dev(unsigned long long *keys, uint32_t *vals, int64_t n_cap,

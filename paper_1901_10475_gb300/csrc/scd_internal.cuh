@@ -458,46 +458,45 @@ struct SortScratch {
 struct PairEmit {
   int ob, tb;
   const unsigned long long *ends;     // the sorted ends of the open runs
-  unsigned long long n_ends;          // their count (a capacity when d_ne is set)
-  const unsigned long long *d_ne;
+  unsigned long long n_ends;          // their count
   scd_pair *out;
   int64_t n;                          // starts that are records (the rest are holes)
-  const unsigned long long *d_n;
   unsigned int *flags;                // receives ERR_ZIP
 };
 
-// Sort (key, value) pairs by the low `bits` bits of the key, LSD, 8-bit
-// digits, stable.  keys/vals are sorted in place (via the scratch ping-pong).
-// vals may be null (keys only).  Returns cudaSuccess or the launch error.
-int radix_sort_u32(uint32_t *keys, uint32_t *vals, int64_t n, int bits, SortScratch &sc,
-                   cudaStream_t st);
-int radix_sort_u64(unsigned long long *keys, uint32_t *vals, int64_t n, int bits,
-                   SortScratch &sc, cudaStream_t st);
-// the same by key bits [lo, bits) only (the bits below lo are payload)
-// so: the sorted arrays are left where the last pass put them (keys and vals, or
-// the scratch, by the number of passes) and named there, which saves the copy
-// back of an odd number of passes.
+// Where a sort left its result: the arrays given, or the scratch, by the number
+// of passes; asking for it saves the copy back of an odd number.
 struct SortOut {
   const void *keys;
   const uint32_t *vals;
 };
+
+// Sort (key, value) pairs by key bits [lo, bits), LSD, whole 8-bit digits from lo
+// on (a last, partial digit takes the bits above it along: keys have none set
+// there), stable; the bits below lo are payload.  vals may be null (keys only).
+// The result lies in keys and vals, or with `so` where that says.  Returns a
+// status.
+int radix_sort_u32(uint32_t *keys, uint32_t *vals, int64_t n, int bits, SortScratch &sc,
+                   cudaStream_t st);
+int radix_sort_u64(unsigned long long *keys, uint32_t *vals, int64_t n, int bits,
+                   SortScratch &sc, cudaStream_t st);
 int radix_sort_u64(unsigned long long *keys, uint32_t *vals, int64_t n, int lo, int bits,
                    SortScratch &sc, cudaStream_t st, SortOut *so = nullptr);
-// size the scratch for sorts of up to n elements (nothing allocated later)
-int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaStream_t st);
-// the same with the element count read on the device (min(*d_n, n_cap)), for
-// sorts inside a captured graph; grids are sized for n_cap
-// Sort the packed run starts keys[0, n) (a capacity with d_n) by bits
-// [lo, bits) and write the sorted records as pairs into pe.out: the passes
-// before the last as radix_sort_u64, the last one scattering decoded pairs
-// (each open start zipped with its end) instead of keys.  The keys are left
-// in an unspecified order.
-int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, const unsigned long long *d_n,
-                         int lo, int bits, SortScratch &sc, const PairEmit &pe, cudaStream_t st);
-// (without so the copy back takes the whole capacity)
+// The same with the element count read on the device (min(*d_n, n_cap)), for
+// queues without host reads; grids are sized for n_cap, and without `so` the copy
+// back takes all of it.
 int radix_sort_u64_dev(unsigned long long *keys, uint32_t *vals, int64_t n_cap,
                        const unsigned long long *d_n, int lo, int bits, SortScratch &sc,
                        cudaStream_t st, SortOut *so = nullptr);
+// Size the scratch for sorts of up to n elements, with values or without as
+// said: they then allocate nothing.
+int sort_reserve(SortScratch &sc, int64_t n, size_t key_bytes, bool vals, cudaStream_t st);
+// Sort the packed run starts keys[0, n) by bits [lo, bits) and write the sorted
+// records as pairs into pe.out: the passes before the last as radix_sort_u64,
+// the last one scattering decoded pairs (each open start zipped with its end)
+// instead of keys.  The keys are left in an unspecified order.
+int radix_sort_u64_pairs(unsigned long long *keys, int64_t n, int lo, int bits, SortScratch &sc,
+                         const PairEmit &pe, cudaStream_t st);
 
 // Run starts carry their last tick below the (i, j, first tick) key when
 // both fit in 64 bits and the all-ones tick field is free to tag open runs

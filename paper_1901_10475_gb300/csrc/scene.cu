@@ -271,7 +271,7 @@ extern "C" SCD_API int scd_build_boxes(scd_scene *s) {
     return SCD_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return SCD_ERR_CUDA;
   int64_t N = (int64_t)s->h_ctr_pinned->n_boxes;
-  if (N <= 0 || N >= (1ll << 31)) return SCD_ERR_INVALID_ARG;
+  if (N <= 0 || N >= kMaxTreeBoxes) return SCD_ERR_INVALID_ARG;
   s->N = N;
   bool ok = s->d_lo.ensure(N, st) && s->d_hi.ensure(N, st) && s->d_obj.ensure(N, st) &&
             s->d_id.ensure(N, st) && s->d_key32.ensure(N, st) &&

@@ -641,7 +641,6 @@ int traverse(scd_scene *s, int raw_mode, int obj_bits, int t_bits) {
   a.nodes = s->d_nodes.p;
   a.sbox = s->s_box.p;
   a.link = s->s_link.p;
-  a.sid = s->d_id.p;
   // one query per sorted reference
   a.N = s->dkind != SCD_DECOMP_NONE ? s->n_refs : s->N;
   a.lv = tree_levels(a.N);
@@ -948,17 +947,14 @@ static UnpackArgs unpack_args(scd_scene *s, int raw_mode, int obj_bits, int t_bi
 }
 
 static PairEmit pair_emit(scd_scene *s, int obj_bits, int t_bits, const unsigned long long *ends,
-                          unsigned long long n_ends, const unsigned long long *d_ne,
-                          scd_pair *out, int64_t n, const unsigned long long *d_n) {
+                          unsigned long long n_ends, scd_pair *out, int64_t n) {
   PairEmit pe;
   pe.ob = obj_bits;
   pe.tb = t_bits;
   pe.ends = ends;
   pe.n_ends = n_ends;
-  pe.d_ne = d_ne;
   pe.out = out;
   pe.n = n;
-  pe.d_n = d_n;
   pe.flags = &s->d_ctr.p->trav_flags;
   return pe;
 }
@@ -1097,9 +1093,9 @@ int canonicalize_streamed(scd_scene *s, int obj_bits, int t_bits, scd_pair *host
     unsigned long long *ks = s->d_part.p + ps[d0], *ke = s->d_parte.p + pe[d0];
     if (m > 0) {
       if (me > 0) TRY_(radix_sort_u64(ke, nullptr, eslots, bits, s->sort_sc, st));
-      TRY_(radix_sort_u64_pairs(ks, slots, nullptr, lo, bits + lo, s->sort_sc,
+      TRY_(radix_sort_u64_pairs(ks, slots, lo, bits + lo, s->sort_sc,
                                 pair_emit(s, obj_bits, t_bits, ke, (unsigned long long)me,
-                                          nullptr, s->d_out.p + out_at, m, nullptr),
+                                          s->d_out.p + out_at, m),
                                 st));
     } else if (me > 0) {
       return SCD_ERR_INTERNAL;  // ends without starts
