@@ -47,8 +47,8 @@ constexpr float kNpSlackKm = 1e-4f, kNpSlackRel = 1e-6f;
 // more than the rounding of the few FP32 operations it takes
 constexpr float kNpSkipShrink = 1.0f - 1e-4f;
 // rounding allowance added to the Kepler residual [rad]: FP32 rounding of
-// M, of e and of the residual's own terms (sinf within 2 ulp), together
-// below 2e-6 rad for |E|, |M| < 2 pi
+// M, of e and of the residual's own terms, and the error of sin E (7e-7),
+// together below 1.3e-6 rad for |E|, |M| < 2 pi (measured: see pv32)
 constexpr float kNpResidualSlack = 3.5e-6f;
 
 // narrow-phase state words (device): earliest witness as t << 32 | candidate,
@@ -173,8 +173,13 @@ __device__ __forceinline__ float mean_anomaly32(const float4 m, float tf) {
 // and cosine of the corrected E come from those before it to second order (the
 // third is below 5e-12), together within 7e-7 of the true ones.  The error
 // bounds take the residual of Kepler's equation at the result; their
-// allowances, kNpResidualSlack rad and 4e-6 a of the position, are four times
-// what the sine's error and the rounding of the terms amount to.
+// allowances, kNpResidualSlack rad and 4e-6 a of the position, are 2.7 times
+// what the sine's error and the rounding of the terms can amount to, and the
+// residual's part of the bound is taken four times over besides.  Measured against
+// FP64, 67 M draws in each of e < 0.02, 0.75, 0.95 and 0.999 over 24 h: sine and
+// cosine within 6.2e-7, the residual within 8.0e-7 rad, the position at the FP32
+// E within 6.5e-7 a; in all the position within 2.0% of its bound and the velocity
+// within 1.6% (with the accurate sine, cosine and division 1.1% and 1.0%).
 constexpr float kNpNewton = 3e-4f;
 
 __device__ __forceinline__ void pv32(const NpTick &o, float tf, float x[3], float v[3],

@@ -440,18 +440,24 @@ __global__ void __launch_bounds__(kRsThreads, kVals ? 4 : 3) k_rs_downsweep(
 // distributed shared memory and write their runs to global memory (L2 at
 // these sizes); the cluster's hardware barrier separates the steps.  Up to
 // kSoloMax keys one block does it alone, the keys in shared memory throughout.
-// A pass of three kernels takes about 18 us of launches and latency however
-// few the keys.  Five passes of (key, value) pairs: 1,204 keys 16 us (86 in
-// three kernels a pass), 3,913 26 (97), 15,050 42 (96), 45,150 51 (98), 90,300 68
-// (97), 154,112 92 (97), 210,700 108 (101): the SMs' ranking takes over.
+// A pass of three kernels launched one by one takes about 18 us however few the
+// keys, in a captured graph about 11.  Five passes of (key, value) pairs, launched: 1,204
+// keys 16 us (86 in three kernels a pass), 3,913 26 (97), 15,050 42 (96), 45,150
+// 51 (98), 90,300 68 (97), 154,112 92 (97), 210,700 108 (101): the SMs' ranking
+// takes over.  In a graph: 1,638 keys 19 us (50), 16,384 42 (55), 81,920 70 (55),
+// 163,840 106 (52).
 // ---------------------------------------------------------------------------
 constexpr int kClBlocks = 16, kClThreads = 1024, kClWarps = kClThreads / 32;
 constexpr int kClItems = 16;  // keys per thread at most
 constexpr int kSoloItems = 4;
 constexpr int64_t kSoloMax = (int64_t)kSoloItems * kClThreads;
-// up to 163,840 keys; where the count is on the device and the host knows only
-// a capacity, up to the most that fits (the refinement's first round is its
-// largest by far: 512 objects 192,512, then 2,594 and fewer)
+// Up to 163,840 keys, where sorts that the host launches one by one break even.
+// (The box sorts of a captured find break even near 45,000 keys: its 86,000 boxes
+// cost it 13 us of 360.)  Where the count is on the device and the host knows only
+// a capacity, up to the most that fits: a refinement's rounds shrink fast after the
+// first, which alone fills the capacity.  Whole refinements with first rounds of
+// 192,512, 225,600 and 259,440 intervals (then 2,450, 3,322 and 3,700): 392, 493 and
+// 440 us; with 163,840 as the limit 459, 555 and 484.
 constexpr int64_t kClusterHost = (int64_t)10 * kClBlocks * kClThreads;
 constexpr int64_t kClusterMax = (int64_t)kClItems * kClBlocks * kClThreads;
 
