@@ -209,11 +209,66 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def _bits_for(v: int) -> int:
+    return max(1, int(v).bit_length())
+
+
+def phase_bytes(m: dict, n: int) -> dict:
+    """HBM bytes of one screen by phase: every array that the present code
+    reads or writes, once per pass that runs.  Of a replayed or eager find on
+    the device; the reference sort of a decomposed screen is in `build`."""
+    N = m["boxes"]
+    R = m.get("refs") or N  # sorted entries (references when decomposed)
+    cells = m.get("cells", 1)
+    runs = m["records"]
+    opens = m.get("open_runs", runs)  # runs of more than one cell: one end record each
+    small = 163840                    # sorts up to here read their keys once a pass
+    key_b = 4 if m["morton_bits"] <= 8 else 8
+    curve = 4 * m["morton_bits"]
+    split = 1 if m.get("split_km", 0.0) != 0.0 else 0
+
+    def sort_bytes(count, passes, kb, values):
+        return passes * count * (kb * (2 if count <= small else 3) + 8 * values)
+
+    if cells > 1:
+        cbits = max(1, (cells - 1).bit_length())
+        bits = min(64, curve + split + cbits)
+        refs = N * 32 + R * (8 + 4) + sort_bytes(R, -(-bits // 8), 8, 1)
+        sort = 0
+    else:
+        bits = curve + (split if m["morton_bits"] < 12 else 0)
+        if N <= 1 << 20 and bits > 40:
+            bits = 40  # the top ones order as well
+        refs = 0
+        sort = sort_bytes(N, -(-bits // 8), key_b, 1)
+    ob, tb = _bits_for(n - 1), _bits_for(m["T"])
+    rbits = 2 * ob + tb
+    rpasses = -(-rbits // 8)
+    packed = 2 * (ob + tb) <= 64 and m["T"] < (1 << tb) - 1
+    # packed records: the last, partial digit's bits are left to the emission
+    if packed and rpasses >= 2 and rbits - 8 * (rpasses - 1) <= tb:
+        rpasses -= 1
+    return {
+        # elements in; boxes (32 B), object id, box id and key out
+        "boxes": 56 * n + N * (32 + 4 + 4 + key_b),
+        "sort": sort,
+        # boxes gathered by id and written in order, positions by id, nodes (96 bytes
+        # for eight children and 1/7 more above them); id, object and both neighbours'
+        # positions in, links out
+        "build": refs + R * (4 + 32 + 32 + 4 + 14 + 4 + 4 + 8 + 16),
+        # every sorted box, link and node read once; records written
+        "traverse": R * (32 + 16 + 14) + (runs + opens) * 8,
+        # the sorts of the run starts and of the open runs' ends, the open count, the
+        # emission (starts and ends in, pairs out)
+        "canon": (sort_bytes(runs, rpasses, 8, 0 if packed else 1)
+                  + sort_bytes(opens, rpasses, 8, 0) + runs * 8 + runs * (8 + 16) + opens * 8),
+    }
+
+
 def algorithmic_bytes(m: dict, n: int) -> dict:
-    """Algorithmic HBM bytes of one screen by phase: every array read or
-    written once per pass that needs it (one box per leaf).  The hierarchy's
-    terms are a binary tree's (40 bytes a box in the traversal; the implicit
-    tree holds 14), kept so that the fractions compare over time."""
+    """The bytes of a binary tree's screen (40 bytes a box in its traversal, a
+    refit in its build, every digit of every key sorted), which earlier lines
+    were rated by; the line names them `algorithmic_bytes_binary_tree`."""
     N = m["boxes"]
     R = m.get("refs") or N  # sorted entries (references when decomposed)
     M = R
@@ -926,14 +981,12 @@ def main():
         m = r["metrics"]
         line["config"].update({"boxes": m["boxes"], "pairs": r["n_pairs"],
                                "records": m["records"], "open_runs": m["open_runs"],
-                               "leaf_size": m["leaf_size"],
-                               "morton_bits": m["morton_bits"], "stack_depth": m["stack_depth"],
-                               "block_threads": m["block_threads"]})
+                               "morton_bits": m["morton_bits"], "split_km": m["split_km"]})
         line["box_pair_tests_per_s"] = r["tests"] / (sum(r["times"]) * 1e-3)
         line["node_tests"] = m["node_tests"]
         line["leaf_tests"] = m["leaf_tests"]
         ph = r["phase_ms"]
-        byt = algorithmic_bytes(m, r["n"])
+        byt = phase_bytes(m, r["n"])
         # the dominant phase of the screen (the narrow phase of narrow24h is
         # reported on its own, under "narrow")
         dom = max((k for k in ph if k != "ms_narrow"), key=ph.get)
@@ -951,7 +1004,9 @@ def main():
                                                "(profiles/k_traverse2_catalog16848_24h.md)"
                                                if traffic is not None else None),
                             "peak_source": src, "phase_ms": ph,
-                            "algorithmic_bytes": byt[name]}
+                            "algorithmic_bytes": byt[name],
+                            "algorithmic_bytes_binary_tree":
+                                algorithmic_bytes(m, r["n"])[name]}
         if "phase_ms_source" in r:
             line["roofline"]["phase_ms_source"] = r["phase_ms_source"]
         line["gpu_launches"] = r["launches"]

@@ -214,7 +214,7 @@ SCD_API int scd_scene_set_elements_device(scd_scene *s, const scd_element *d_ele
 /* Tuning for later calls; NULL fields are not allowed, use scd_default_tuning. */
 SCD_API int scd_scene_set_tuning(scd_scene *s, const scd_tuning *t);
 SCD_API int scd_default_tuning(scd_tuning *t);
-/* The scene's tuning in force .  Copied into *t. */
+/* The scene's tuning in force.  Copied into *t. */
 SCD_API int scd_scene_get_tuning(const scd_scene *s, scd_tuning *t);
 
 /* Steps A1-A4: per-object steps, FP64 propagation, outward-rounded FP32
